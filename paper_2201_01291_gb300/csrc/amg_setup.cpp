@@ -39,7 +39,9 @@
 //     level saves barriers per V-cycle on big meshes, a smaller one keeps the O(n^3) set-up of
 //     small meshes cheap), where the coarse matrix is inverted
 //     densely (Cholesky; Gauss-Jordan with partial pivoting for the non-symmetric matrix of
-//     the axisymmetric configuration) and applied as a dense product.
+//     the axisymmetric configuration) and applied as a dense product;
+//   * the levels of at most kAmgDenseRows rows are also multiplied out, M = U Q + Pf M' Rf level
+//     by level, so that a solve can apply them as one dense product (the same V-cycle).
 // The same construction serves the axisymmetric matrix (mildly non-symmetric; it also maps the
 // constant potential to zero), preconditioning BiCGStab there (solver kind 9).
 #include <algorithm>
@@ -58,6 +60,8 @@ namespace {
 constexpr double kTheta = 0.08;
 constexpr double kJacobiOmega = 1.7;  // omega = kJacobiOmega / lambda_max(D^-1 A)
 constexpr int kCoarseMin = 256, kCoarseMax = 1500;
+constexpr int kManySlices = 152 * 24;  // warps of a whole-GPU solve
+constexpr int kDirectRows = 512;  // meshes up to this size: the inverse of the matrix itself
 
 // y = A x (CSR)
 void csr_mv(const Csr& A, const std::vector<double>& x, std::vector<double>& y) {
@@ -366,6 +370,28 @@ void composite_operators(AmgHostLevel& L, bool symmetric) {
   }
 }
 
+// M = U Q + Pf (M' Rf): the V-cycle of level L and below as one dense n x n matrix, from the
+// dense matrix M' of the next level (n' x n').
+void dense_vcycle(const AmgHostLevel& L, const std::vector<double>& Mn, std::vector<double>& M) {
+  const int32_t n = L.A.n, nn = L.P.m;
+  std::vector<double> W((size_t)nn * n, 0.0);  // M' Rf
+  for (int32_t i = 0; i < nn; ++i)
+    for (int32_t k = 0; k < nn; ++k) {
+      const double m = Mn[(size_t)i * nn + k];
+      for (int32_t e = L.Rf.rp[k]; e < L.Rf.rp[k + 1]; ++e) W[(size_t)i * n + L.Rf.ci[e]] += m * L.Rf.v[e];
+    }
+  M.assign((size_t)n * n, 0.0);
+  for (int32_t i = 0; i < n; ++i) {
+    double* __restrict__ row = &M[(size_t)i * n];
+    for (int32_t e = L.Pf.rp[i]; e < L.Pf.rp[i + 1]; ++e) {
+      const double v = L.Pf.v[e];
+      const double* __restrict__ w = &W[(size_t)L.Pf.ci[e] * n];
+      for (int32_t j = 0; j < n; ++j) row[j] += v * w[j];
+    }
+    for (int32_t e = L.U.rp[i]; e < L.U.rp[i + 1]; ++e) row[L.U.ci[e]] += L.U.v[e] * L.Q.v[L.U.ci[e]];
+  }
+}
+
 }  // namespace
 
 void sell_from_csr(const Csr& A, SellHost& S, int lpr) {
@@ -373,44 +399,42 @@ void sell_from_csr(const Csr& A, SellHost& S, int lpr) {
   S.n = A.n;
   S.lpr = lpr;
   S.nslices = (A.n + rps - 1) / rps;
-  S.rlen.assign((size_t)S.nslices * rps, 0);
-  for (int32_t i = 0; i < A.n; ++i) S.rlen[i] = A.rp[i + 1] - A.rp[i];
   S.sl_ptr.assign(S.nslices + 1, 0);
-  S.sl_w.assign(S.nslices, 0);
   int64_t off = 0;
   for (int32_t s = 0; s < S.nslices; ++s) {
-    int32_t w = 0;
-    for (int r = 0; r < rps; ++r) w = std::max(w, (S.rlen[(size_t)s * rps + r] + lpr - 1) / lpr);
-    S.sl_w[s] = w;
+    int32_t w = 1;
+    for (int32_t i = s * rps; i < std::min(A.n, (s + 1) * rps); ++i)
+      w = std::max(w, (A.rp[i + 1] - A.rp[i] + lpr - 1) / lpr);
     S.sl_ptr[s] = (int32_t)off;
     off += (int64_t)w * kSlice;
   }
   S.sl_ptr[S.nslices] = (int32_t)off;
   S.col.assign(off, 0);
   S.val.assign(off, 0.0);
-  for (int32_t s = 0; s < S.nslices; ++s)
-    for (int r = 0; r < rps; ++r) {
-      const int32_t i = s * rps + r;
-      if (i >= A.n) continue;
-      for (int32_t k = 0; k < S.rlen[i]; ++k) {  // padding slots keep column 0 and value 0
+  for (int32_t s = 0; s < S.nslices; ++s) {
+    for (int32_t i = s * rps; i < std::min(A.n, (s + 1) * rps); ++i) {
+      const int r = i - s * rps;
+      for (int32_t k = 0; k < A.rp[i + 1] - A.rp[i]; ++k) {  // padding slots keep column 0 and value 0
         const int64_t e = (int64_t)S.sl_ptr[s] + (int64_t)(k / lpr) * kSlice + r * lpr + (k % lpr);
         S.col[e] = A.ci[A.rp[i] + k];
         S.val[e] = A.v[A.rp[i] + k];
       }
     }
+    for (int l = 0; l < kSlice; ++l) S.col[(int64_t)S.sl_ptr[s + 1] - kSlice + l] |= kSliceEnd;
+  }
 }
 
 int lanes_per_row(const Csr& A) {
   const double avg = A.n > 0 ? (double)A.rp[A.n] / A.n : 0.0;
   int lpr = 1;
-  while (lpr < kSlice && avg > 8.0 * lpr) lpr *= 2;
+  while (lpr < kSlice && avg > 8.0 * lpr && (int64_t)A.n * lpr < (int64_t)kManySlices * kSlice) lpr *= 2;
   return lpr;
 }
 
 int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
   // the axisymmetric matrix is not symmetric: no symmetrisation, LU instead of Cholesky
   const bool symmetric = m.geometry != AVIP_GEOM_AXISYMMETRIC;
-  const int32_t coarse_max = std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
+  const int32_t coarse_max = m.N <= kDirectRows ? m.N : std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
   auto fail = [&](const char* msg) {
     if (err && errlen) std::snprintf(err, errlen, "%s", msg);
     return AVIP_EINVAL;
@@ -527,6 +551,13 @@ int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
     H.lv.push_back(std::move(L));
     A = std::move(Ac);
     B.swap(Bc);
+  }
+  H.dlev = (int32_t)H.lv.size() - 1;
+  H.dmat = H.cinv;
+  while (H.dlev > 0 && H.lv[H.dlev - 1].A.n <= kAmgDenseRows) {
+    std::vector<double> M;
+    dense_vcycle(H.lv[--H.dlev], H.dmat, M);
+    H.dmat.swap(M);
   }
   return AVIP_OK;
 }

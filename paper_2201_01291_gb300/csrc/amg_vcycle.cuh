@@ -9,16 +9,24 @@
 // completed by an earlier one.  The values are FP32 by default (the preconditioner only shapes
 // the search directions; the iterate, the residuals and the stopping test stay FP64) or FP64.
 //
+// The levels below the finest one of at most kAmgDenseRows rows are applied as one dense product
+// (AmgDenseT): phase p of the cycle is the down phase of level p for p < dl (the dense level), the
+// dense product for p = dl, the up phase of level 2 dl - p above, and phase 2 dl + 1 is the
+// product with the matrix.  Every operator streams through the warps' rings (stream.cuh).
+//
 // `Ops` supplies the synchronisation of the participating threads: barrier() completes every
 // vector written before it, sum(v) returns the sum of v over all participants (and is a
-// barrier too); both return false if a wait was abandoned.  gwarp / nwarps number the
-// participating warps.
+// barrier too); both return false if a wait was abandoned.  ops.ring is the calling warp's ring,
+// gwarp / nwarps number the participating warps.
 #pragma once
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "avip_internal.h"
 #include "grid_sync.cuh"
 #include "sell.cuh"
+#include "stream.cuh"
 
 namespace avip {
 
@@ -44,47 +52,115 @@ struct DotAcc<float> {
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
+// A solve's hierarchy and phase table in shared memory (one per block), and its dense level.
+struct SolveShared {
+  PhaseDesc tab[kMaxPhases];
+  unsigned long long H[sizeof(AmgDevT<double>) / 8];
+  unsigned long long bar[128];      // the rings' mbarriers, kDepth per warp
+  double gain;
+  int bad;                          // a warp's copy did not arrive (Ring::wait)
+};
+// Dynamic shared memory of a solve: the rings, then the dense product's right-hand side.
+constexpr size_t kRhsBytes = sizeof(double) * kAmgDenseRows;
+template <typename T>
+struct AmgCtx {
+  const AmgDevT<T>* H;  // shared memory
+  AmgDenseT<T> D;
+  double gain;          // of the Dirichlet lift (dirichlet_gain; a division, so one thread per block)
+  T* rhs;               // shared memory: the dense product's right-hand side, zero-padded
+  __device__ __forceinline__ int mat_phase() const { return 2 * D.level + 1; }
+};
+
+// The larger dense level as long as a CTA's share of it stays within 256 KB per product (2.5 us of
+// L2 bandwidth); the coarsest inverse on fewer CTAs.
+constexpr size_t kDenseBytesPerCta = 256 * 1024;
+template <typename T>
+__device__ __forceinline__ int dense_choice(const AmgDevT<T>& H, int nctas) {
+  const size_t bytes = (size_t)H.L[H.dense[0].level].n * H.dense[0].steps * kSlice * sizeof(T);
+  return bytes <= kDenseBytesPerCta * (size_t)nctas ? 0 : 1;
+}
+
+// Start of a solve: the hierarchy's descriptors copied to shared memory, the phase table written
+// and the calling warp's ring started at the matrix phase (the solve begins with a true residual)
+// or at the finest down phase.  TA: type of the streamed matrix values.  Every thread of the
+// participating blocks calls it.
+template <typename T, typename TA, class R>
+__device__ AmgCtx<T> solve_begin(SolveShared& sh, R& ring, char* dyn, const PcgArgs& a,
+                                 const AmgDevT<T>* __restrict__ Hg, const TA* aval, int nctas, int gwarp, int nwarps,
+                                 int lane, bool matrix_first) {
+  static_assert(sizeof(AmgDevT<T>) == sizeof(AmgDevT<double>), "one shared copy for both types");
+  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(Hg);
+  for (int k = threadIdx.x; k < (int)(sizeof(AmgDevT<T>) / 8); k += blockDim.x) sh.H[k] = src[k];
+  if (threadIdx.x == 0) {
+    sh.gain = dirichlet_gain(a);
+    sh.bad = 0;
+  }
+  __syncthreads();
+  AmgCtx<T> C;
+  C.gain = sh.gain;
+  C.rhs = reinterpret_cast<T*>(dyn + (blockDim.x >> 5) * R::kWarpBytes);
+  C.H = reinterpret_cast<const AmgDevT<T>*>(sh.H);
+  C.D = C.H->dense[dense_choice(*C.H, nctas)];
+  const int dl = C.D.level, p = (int)threadIdx.x;
+  if (p <= 2 * dl + 1) {
+    PhaseDesc d;
+    if (p == 2 * dl + 1) {
+      d = PhaseDesc{a.colS, aval, a.A.sl_ptr, a.A.nslices, a.A.N, 1, sizeof(TA) == 8};
+    } else if (p == dl) {
+      const int n = C.H->L[dl].n;
+      d = PhaseDesc{nullptr, C.D.m, nullptr, n, n, C.D.steps, sizeof(T) == 8};
+    } else {
+      const SellMatT<T>& M = p < dl ? C.H->L[p].Rf : C.H->L[2 * dl - p].UP;
+      d = PhaseDesc{M.col, M.val, M.sl_ptr, M.nslices, M.n, M.lpr, sizeof(T) == 8};
+    }
+    sh.tab[p] = d;
+  }
+  __syncthreads();
+  ring.init(sh.tab, 2 * dl + 2, dyn + (threadIdx.x >> 5) * R::kWarpBytes,
+            sh.bar + (threadIdx.x >> 5) * R::kDepth, &sh.bad, gwarp, nwarps, lane, matrix_first ? 2 * dl + 1 : 0);
+  return C;
+}
+
 // Down phase of level l: xp = Q b on the rows of level l (Q = omega D^-1 is diagonal: an
 // elementwise pass) and b' = Rf b on the rows of level l + 1 (a streamed product), b given by
 // `src` (complete on entry).  `hook` takes part in every row i of level l: hook.begin(i) loads
 // the row's own operands, hook.end(i, pre) runs with them (the CG update folded into the
-// finest level's phase).  The elementwise pass takes one row per thread at a time (issuing the
-// loads of several rows before their use kept more registers live than the 64 - 80 a thread has
-// at 768 - 1024 threads per block: the spills cost more than the extra loads in flight saved);
-// then every warp streams a contiguous share of Rf.
-template <typename T, int U, class Src, class Hook>
-__device__ __forceinline__ void amg_down(const AmgDevT<T>* __restrict__ H, int l, Src src, Hook hook, int gwarp,
+// finest level's phase).
+template <typename T, class Ops, class Src, class Hook>
+__device__ __forceinline__ void amg_down(const AmgCtx<T>& C, Ops& ops, int l, Src src, Hook hook, int gwarp,
                                          int nwarps, int lane) {
-  const AmgLevelT<T>& L = H->L[l];
-  T* __restrict__ bn = H->L[l + 1].b;
+  const AmgLevelT<T>& L = C.H->L[l];
+  T* __restrict__ bn = C.H->L[l + 1].b;
   T* __restrict__ xp = L.xp;
   const T* __restrict__ qd = L.qd;
   const int n = L.n;
-  for (int i = gwarp * kSlice + lane; i < n; i += nwarps * kSlice) {
-    const auto pre = hook.begin(i);
-    const T bi = src(i);
-    const T qi = __ldg(qd + i);
-    hook.end(i, pre);
+  // two rows per thread at a time, their loads issued together
+  const int stride = nwarps * kSlice;
+  for (int i = gwarp * kSlice + lane; i < n; i += 2 * stride) {
+    const int j = i + stride;
+    const bool two = j < n;
+    const auto pi = hook.begin(i);
+    const T bi = src(i), qi = __ldg(qd + i);
+    const auto pj = hook.begin(two ? j : i);
+    const T bj = src(two ? j : i), qj = __ldg(qd + (two ? j : i));
+    hook.end(i, pi);
     xp[i] = qi * bi;
+    if (two) {
+      hook.end(j, pj);
+      xp[j] = qj * bj;
+    }
   }
-  int sa, sb;
-  warp_slices(L.Rf.nslices, gwarp, nwarps, sa, sb);
-  spmv_stream<T, U>(L.Rf, sa, sb, lane, src, NoBegin(), [&](int j, T v, NoPre) { bn[j] = v; });
+  stream_rows<T, T>(ops.ring, l, lane, src, NoBegin(), [&](int j, T v, NoPre) { bn[j] = v; });
 }
 
 // Up phase of level l: x = U xp + Pf x' = [U | Pf] [xp; x'] on the rows of level l (x' = the
 // next level's solution, complete on entry), each row handed to out.end(i, value, pre) with the
 // operands out.begin(i) fetched ahead.
-template <typename T, int U, class Out>
-__device__ __forceinline__ void amg_up(const AmgDevT<T>* __restrict__ H, int l, Out out, int gwarp, int nwarps,
-                                       int lane) {
-  const AmgLevelT<T>& L = H->L[l];
-  const T* __restrict__ xp = L.xp;
-  const T* __restrict__ xn = H->L[l + 1].x;
-  const int n = L.n;
-  int sa, sb;
-  warp_slices(L.UP.nslices, gwarp, nwarps, sa, sb);
-  spmv_stream<T, U>(L.UP, sa, sb, lane, [xp, xn, n](int c) { return __ldca(c < n ? xp + c : xn + (c - n)); },
+template <typename T, class Ops, class Out>
+__device__ __forceinline__ void amg_up(const AmgCtx<T>& C, Ops& ops, int l, Out out, int lane) {
+  const AmgLevelT<T>& L = C.H->L[l];
+  const T* __restrict__ xp = L.xp;  // followed by x'
+  stream_rows<T, T>(ops.ring, 2 * C.D.level - l, lane, [xp](int c) { return __ldca(xp + c); },
                     [&](int i) { return out.begin(i); },
                     [&](int i, T v, const decltype(out.begin(0))& pre) { out.end(i, v, pre); });
 }
@@ -101,91 +177,79 @@ struct StoreOut {  // x_i = value
   __device__ void end(int i, T v, NoPre) const { x[i] = v; }
 };
 
-// Coarsest level: x = A_c^-1 b as a dense product, one warp per row; b given by `src`
-// (complete on entry), each row handed to out(row, value) by lane 0.
-template <typename T, class Src, class Out>
-__device__ __forceinline__ void amg_coarse(const AmgDevT<T>* __restrict__ H, Src src, Out out, int gwarp,
-                                           int nwarps, int lane) {
-  constexpr int K = 8;  // independent loads per lane in flight
-  const int n = H->nc;
-  const T* __restrict__ cinv = H->cinv;
-  for (int row = gwarp; row < n; row += nwarps) {
-    const T* __restrict__ crow = cinv + (size_t)row * n;
-    T s = T(0);
-    for (int k0 = lane; k0 < n; k0 += 32 * K) {
-      T c[K], b[K];
-#pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int k = k0 + 32 * u;
-        c[u] = k < n ? __ldg(crow + k) : T(0);
-        b[u] = k < n ? src(k) : T(0);
-      }
-#pragma unroll
-      for (int u = 0; u < K; ++u) s = fma_t(c[u], b[u], s);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out(row, s);
-  }
+// The dense product x = M b of the phase dl, b given by src: every block first copies all of b to
+// shared memory (one load per thread), so that the product's inner loop has no memory latency.
+template <typename T, class Ops, class Src, class Out>
+__device__ __forceinline__ void amg_dense(const AmgCtx<T>& C, Ops& ops, Src src, Out out, int lane) {
+  const int n = C.H->L[C.D.level].n, np = C.D.steps * kSlice;
+  for (int k = threadIdx.x; k < np; k += blockDim.x) C.rhs[k] = k < n ? src(k) : T(0);
+  __syncthreads();
+  stream_dense<T>(ops.ring, C.D.level, lane, C.rhs, out);
 }
 
-// The V-cycle below the finest level: down phases of levels 1 .. nlev-2, the coarsest solve,
-// up phases of levels nlev-2 .. 1, one barrier after each.  Entered once the finest down phase
-// is complete (nlev >= 2); on return the level-1 solution is complete.
+// The V-cycle below the finest level: down phases of levels 1 .. dl-1, the dense product, up
+// phases of levels dl-1 .. 1, one barrier after each.  Entered once the finest down phase is
+// complete (dl >= 1); on return the level-1 solution is complete.
 template <typename T, class Ops>
-__device__ bool amg_inner(const AmgDevT<T>* __restrict__ H, Ops& ops, int gwarp, int nwarps, int lane) {
-  const int nl = H->nlev;
-  for (int l = 1; l + 1 < nl; ++l) {
-    const T* __restrict__ b = H->L[l].b;
-    amg_down<T, Ops::kStream>(H, l, [b](int c) { return __ldca(b + c); }, NoHook(), gwarp, nwarps, lane);
+__device__ bool amg_inner(const AmgCtx<T>& C, Ops& ops, int gwarp, int nwarps, int lane) {
+  const int dl = C.D.level;
+  for (int l = 1; l < dl; ++l) {
+    const T* __restrict__ b = C.H->L[l].b;
+    amg_down(C, ops, l, [b](int c) { return __ldca(b + c); }, NoHook(), gwarp, nwarps, lane);
     if (!ops.barrier()) return false;
   }
   {
-    const T* __restrict__ cb = H->L[nl - 1].b;
-    T* __restrict__ cx = H->L[nl - 1].x;
-    amg_coarse(H, [cb](int k) { return __ldca(cb + k); }, [cx](int row, T v) { cx[row] = v; }, gwarp, nwarps, lane);
+    const T* __restrict__ cb = C.H->L[dl].b;
+    T* __restrict__ cx = C.H->L[dl].x;
+    amg_dense(C, ops, [cb](int k) { return __ldca(cb + k); }, [cx](int row, T v) { cx[row] = v; }, lane);
     if (!ops.barrier()) return false;
   }
-  for (int l = nl - 2; l >= 1; --l) {
-    amg_up<T, Ops::kStream>(H, l, StoreOut<T>{H->L[l].x}, gwarp, nwarps, lane);
+  for (int l = dl - 1; l >= 1; --l) {
+    amg_up(C, ops, l, StoreOut<T>{C.H->L[l].x}, lane);
     if (!ops.barrier()) return false;
   }
   return true;
 }
 
 // One V-cycle z = M b0, b0 complete on entry (TB: its type; TZ: the type z is stored in).  With
-// want_dot the last barrier is a grid sum that returns dot = b0.z; otherwise a plain barrier.
-// Returns false if a wait was abandoned.
-template <typename T, typename TB, typename TZ, class Ops>
-__device__ bool vcycle(const AmgDevT<T>* __restrict__ H, const TB* __restrict__ b0, TZ* __restrict__ z, Ops& ops,
-                       int gwarp, int nwarps, int lane, bool want_dot, double& dot) {
+// an epilogue (NE > 0) the last barrier is a sum of b0.z handed to it (sum_epi); otherwise a plain
+// barrier.  Returns false if a wait was abandoned.
+template <typename T, typename TB, typename TZ, class Ops, int NE, class Epi>
+__device__ bool vcycle(const AmgCtx<T>& C, const TB* __restrict__ b0, TZ* __restrict__ z, Ops& ops, int gwarp,
+                       int nwarps, int lane, double (&res)[NE], bool& flag, Epi epi) {
+  constexpr bool kDot = !std::is_same<Epi, NoEpilogue>::value;
   auto src = [b0](int c) { return (T)__ldca(b0 + c); };
   DotAcc<double> acc;
   struct Out {  // z_i = value, b0_i z_i into the dot product
     const TB* b0;
     TZ* z;
     DotAcc<double>* acc;
-    __device__ double begin(int i) const { return (double)__ldca(b0 + i); }
-    __device__ void end(int i, T v, double bi) const {
+    __device__ TB begin(int i) const { return kDot ? __ldca(b0 + i) : TB(0); }
+    __device__ void end(int i, T v, TB bi) const {
       z[i] = (TZ)v;
-      acc->add(bi, (double)v);
+      if (kDot) acc->add((double)bi, (double)v);
     }
   } out{b0, z, &acc};
-  if (H->nlev == 1) {
-    amg_coarse(H, src, [&](int row, T v) { out.end(row, v, out.begin(row)); }, gwarp, nwarps, lane);
+  if (C.D.level == 0) {
+    amg_dense(C, ops, src, [&](int row, T v) { out.end(row, v, out.begin(row)); }, lane);
   } else {
-    amg_down<T, Ops::kStream>(H, 0, src, NoHook(), gwarp, nwarps, lane);
+    amg_down(C, ops, 0, src, NoHook(), gwarp, nwarps, lane);
     if (!ops.barrier()) return false;
-    if (!amg_inner(H, ops, gwarp, nwarps, lane)) return false;
-    amg_up<T, Ops::kStream>(H, 0, out, gwarp, nwarps, lane);
+    if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
+    amg_up(C, ops, 0, out, lane);
   }
-  if (want_dot) {
-    double v[1] = {acc.value()};
-    if (!ops.sum(v)) return false;
-    dot = v[0];
-    return true;
+  if constexpr (kDot) {
+    return ops.template sum_epi<NE>(acc.value(), res, flag, epi);
+  } else {
+    return ops.barrier();
   }
-  return ops.barrier();
+}
+template <typename T, typename TB, typename TZ, class Ops>
+__device__ bool vcycle(const AmgCtx<T>& C, const TB* __restrict__ b0, TZ* __restrict__ z, Ops& ops, int gwarp,
+                       int nwarps, int lane) {
+  double none[1];
+  bool flag;
+  return vcycle(C, b0, z, ops, gwarp, nwarps, lane, none, flag, NoEpilogue());
 }
 
 // CG preconditioned by the V-cycle on the scaled system (kinds 8, 11 and the batched FP64 form):
@@ -193,18 +257,18 @@ __device__ bool vcycle(const AmgDevT<T>* __restrict__ H, const TB* __restrict__ 
 // type T) writes the preconditioned residual z in FP64 (only w = A z gathers it).  The residual update r - alpha q and
 // x += alpha p of iteration k are folded into the finest down phase of iteration k + 1, whose
 // products gather r - alpha q directly (the new residual goes to the other buffer, r2), so an
-// iteration takes 2 nlev grid-wide phases: the finest down phase (sum of r.r: stop test), the
+// iteration takes 2 dl + 2 grid-wide phases: the finest down phase (sum of r.r: stop test), the
 // levels below, the finest up phase (sum of r.z), and w = A z (sum of p.q).  `leader` is the
 // one thread that writes the solve statistics.  Returns false if a wait was abandoned.
 template <typename T, class Ops>
-__device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H, double* __restrict__ z, Ops& ops,
-                             int gwarp, int nwarps, int lane, bool leader) {
+__device__ bool amg_cg_solve(const PcgArgs& a, const AmgCtx<T>& C, double* __restrict__ z, Ops& ops, int gwarp,
+                             int nwarps, int lane, bool leader) {
   constexpr int kMaxRestarts = 8;
-  const int N = a.A.N, nsl = a.A.nslices, nl = H->nlev;
+  const int N = a.A.N, nsl = a.A.nslices, dl = C.D.level, mat = C.mat_phase();
   const double* nb = a.nbuf + (size_t)a.sc->parity * AVIP_MAX_SPECIES * a.Npad;
 
   // ---- x = D^1/2 phi (warm start) and b'
-  const double gain = dirichlet_gain(a);
+  const double gain = C.gain;
   const int hist = history_length(a);
   double bb[1] = {0.0};
   for (int s = gwarp; s < nsl; s += nwarps) {
@@ -229,10 +293,6 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
   if (!ops.sum(bb)) return false;
   {
     const double thresh = a.rtol * a.rtol * bb[0];
-    // the Poisson matrix as a streamed operator, and this warp's contiguous share of its slices
-    const SellMatT<double> A0{a.A.sl_ptr, a.A.sl_w, a.A.rlen, a.A.col, a.A.aval, N, nsl, 1};
-    int ma, mb;
-    warp_slices(nsl, gwarp, nwarps, ma, mb);
     double* rc = a.r;   // current residual
     double* rn = a.r2;  // the other buffer
     // the vectors the finest down phase gathers, in the hierarchy's type: with T = float, FP32
@@ -259,8 +319,8 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
             const double* __restrict__ bv = a.b;
             double* __restrict__ rw = rc;
             T* __restrict__ tw = tc;
-            spmv_stream<double, Ops::kStream64>(
-                A0, ma, mb, lane, [xv](int c) { return __ldca(xv + c); }, [bv](int i) { return bv[i]; },
+            stream_rows<double, double>(
+                ops.ring, mat, lane, [xv](int c) { return __ldca(xv + c); }, [bv](int i) { return bv[i]; },
                 [&](int i, double ax, double bi) {
                   const double r = bi - ax;
                   rw[i] = r;
@@ -268,9 +328,15 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
                   r2[0] = fma(r, r, r2[0]);
                 });
           }
-          if (!ops.sum(r2)) return false;
-          rr_true = r2[0];
-          if (rr_true <= thresh) break;
+          double tot[1];
+          bool small;
+          if (!ops.template sum_epi<1>(r2[0], tot, small, [thresh](double t, double* o) {
+                o[0] = t;
+                return t <= thresh;
+              }))
+            return false;
+          rr_true = tot[0];
+          if (small) break;
           if (!isfinite(rr_true)) {  // non-finite data: stop at once
             status = AVIP_ENAN;
             break;
@@ -320,17 +386,21 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
               *rr = fma(v, v, *rr);
             }
           } hook{rv, qv, a.p, a.x, rn, &rr, tn, al, upd};
-          if (nl == 1) {
+          if (dl == 0) {
             for (int s = gwarp; s < nsl; s += nwarps) {
               const int i = s * kSlice + lane;
               if (i < N) hook.end(i, hook.begin(i));
             }
           } else {
-            amg_down<T, Ops::kStream>(H, 0, [res](int c) { return (T)res(c); }, hook, gwarp, nwarps, lane);
+            amg_down(C, ops, 0, [res](int c) { return (T)res(c); }, hook, gwarp, nwarps, lane);
           }
           if (upd) {
-            double v[1] = {rr};
-            if (!ops.sum(v)) return false;
+            double tot[1];
+            if (!ops.template sum_epi<1>(rr, tot, check, [thresh](double t, double* o) {
+                  o[0] = t;
+                  return t <= thresh || !isfinite(t);
+                }))
+              return false;
             ++it;
             double* t = rc;
             rc = rn;
@@ -338,14 +408,14 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
             T* tt = tc;
             tc = tn;
             tn = tt;
-            check = v[0] <= thresh || !isfinite(v[0]);
             if (check) continue;  // confirm on the true residual
           } else if (!ops.barrier()) {
             return false;
           }
         }
         // ---- the levels below, then the finest up phase: z = U0 xp0 + Pf0 x1, r.z
-        double rzv[1];
+        double rzb[2];  // r.z, beta
+        bool positive;
         {
           DotAcc<double> acc;
           const double* __restrict__ rv = rc;
@@ -360,18 +430,23 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
               acc->add(ri, zi);
             }
           } out{rv, z, &acc};
-          if (nl == 1) {
-            amg_coarse(H, [rv](int k) { return (T)__ldca(rv + k); },
-                       [&](int row, T v) { out.end(row, v, out.begin(row)); }, gwarp, nwarps, lane);
+          if (dl == 0) {
+            amg_dense(C, ops, [rv](int k) { return (T)__ldca(rv + k); },
+                      [&](int row, T v) { out.end(row, v, out.begin(row)); }, lane);
           } else {
-            if (!amg_inner(H, ops, gwarp, nwarps, lane)) return false;
-            amg_up<T, Ops::kStream>(H, 0, out, gwarp, nwarps, lane);
+            if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
+            amg_up(C, ops, 0, out, lane);
           }
-          rzv[0] = acc.value();
-          if (!ops.sum(rzv)) return false;
+          const double rz_old = rz;
+          const bool first = fresh;
+          if (!ops.template sum_epi<2>(acc.value(), rzb, positive, [rz_old, first](double t, double* o) {
+                o[0] = t;
+                o[1] = first ? 0.0 : t / rz_old;
+                return t > 0.0 && isfinite(t);
+              }))
+            return false;
         }
-        const double rz_new = rzv[0];
-        if (!(rz_new > 0.0) || !isfinite(rz_new)) {  // the preconditioned residual lost positivity
+        if (!positive) {  // the preconditioned residual lost positivity
           if (it == 0 || restarts >= kMaxRestarts) {
             status = AVIP_ENOTCONV;
             break;
@@ -379,8 +454,9 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
           check = true;
           continue;
         }
-        const double beta = fresh ? 0.0 : rz_new / rz;
-        rz = rz_new;
+        const double beta = rzb[1];
+        const bool first = fresh;
+        rz = rzb[0];
         fresh = false;
         // ---- w = A z, q = w + beta q, p = z + beta p, p.q -> alpha
         double pq[1] = {0.0};
@@ -392,20 +468,27 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
           struct PreA {
             double z, q, p;
           };
-          spmv_stream<double, Ops::kStream64>(
-              A0, ma, mb, lane, [zc](int c) { return __ldca(zc + c); },
+          stream_rows<double, double>(
+              ops.ring, mat, lane, [zc](int c) { return __ldca(zc + c); },
               [=](int i) { return PreA{__ldca(zc + i), qv[i], pv[i]}; },
               [&](int i, double w, const PreA& o) {
-                const double qn = beta == 0.0 ? w : fma(beta, o.q, w);
-                const double pn = beta == 0.0 ? o.z : fma(beta, o.p, o.z);
+                const double qn = first ? w : fma(beta, o.q, w);  // (restart: old p, q unused)
+                const double pn = first ? o.z : fma(beta, o.p, o.z);
                 qv[i] = qn;
                 if (kCopies) tqw[i] = (T)qn;
                 pv[i] = pn;
                 pq[0] = fma(pn, qn, pq[0]);
               });
         }
-        if (!ops.sum(pq)) return false;
-        alpha = rz / pq[0];
+        double al[1];
+        bool unused;
+        const double rz_now = rz;
+        if (!ops.template sum_epi<1>(pq[0], al, unused, [rz_now](double t, double* o) {
+              o[0] = rz_now / t;
+              return false;
+            }))
+          return false;
+        alpha = al[0];
       }
     }
     // ---- phi = D^-1/2 x
@@ -429,20 +512,17 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H,
 // Mixed-precision solve with the FP32 hierarchy (kind 10 and the batched mixed form): FP64
 // outer residual and correction, FP32 inner CG preconditioned by the FP32 V-cycle.
 template <class Ops>
-__device__ bool amg_mixed_solve(const PcgArgs& a, Ops& ops, int gwarp, int nwarps, int lane, bool leader) {
+__device__ bool amg_mixed_solve(const PcgArgs& a, const AmgCtx<float>& C, Ops& ops, int gwarp, int nwarps, int lane,
+                                bool leader) {
   const int N = a.A.N, nsl = a.A.nslices;
   const double* nb = a.nbuf + (size_t)a.sc->parity * AVIP_MAX_SPECIES * a.Npad;
-  const AmgDevT<float>* __restrict__ H = a.amg32;
-  const SellMatT<float> A32{a.A.sl_ptr, a.A.sl_w, a.A.rlen, a.A.col, a.aval32, N, nsl, 1};
-  int ma, mb;
-  warp_slices(nsl, gwarp, nwarps, ma, mb);
   float* __restrict__ r32 = a.r32;
   float* __restrict__ e32 = a.e32;
   float* __restrict__ p32 = a.p32;
   float* __restrict__ q32 = a.q32;
   float* __restrict__ z32 = a.z32;
 
-  const double gain = dirichlet_gain(a);
+  const double gain = C.gain;
   const int hist = history_length(a);
   double bb[1] = {0.0};
   for (int s = gwarp; s < nsl; s += nwarps) {
@@ -479,20 +559,28 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, Ops& ops, int gwarp, int nwarp
         a.r[i] = r;
         r2[0] = fma(r, r, r2[0]);
       }
-      if (!ops.sum(r2)) return false;
-      rr64 = r2[0];
+      double rs[3];  // r.r, its root and 1 / root
+      bool small;
+      if (!ops.template sum_epi<3>(r2[0], rs, small, [thresh](double t, double* o) {
+            o[0] = t;
+            o[1] = sqrt(t);
+            o[2] = 1.0 / o[1];
+            return t <= thresh;
+          }))
+        return false;
+      rr64 = rs[0];
       if (!isfinite(rr64)) {
         status = AVIP_ENAN;
         break;
       }
-      if (rr64 <= thresh || bb[0] == 0.0) break;
+      if (small || bb[0] == 0.0) break;
       if (it >= a.max_iter) {
         status = AVIP_ENOTCONV;
         break;
       }
       ++outer;
       const int it_outer = it;
-      const double rnorm = sqrt(rr64), rscale = 1.0 / rnorm;
+      const double rnorm = rs[1], rscale = rs[2];
       // ---- FP32 right-hand side r / ||r||, e = 0
       double g0[1];
       {
@@ -509,32 +597,47 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, Ops& ops, int gwarp, int nwarp
       }
       if (!ops.sum(g0)) return false;
       const double inner_thresh = a.inner_rtol * a.inner_rtol * g0[0];
-      double rr = g0[0], rz = 0.0;
-      bool fresh = true;
-      while (rr > inner_thresh && it < a.max_iter) {
-        double rz_new = 0.0;
-        if (!vcycle(H, (const float*)r32, z32, ops, gwarp, nwarps, lane, true, rz_new)) return false;
-        if (!(rz_new > 0.0) || !isfinite(rz_new)) break;  // refine with what the inner solve has
-        const float beta = fresh ? 0.f : (float)(rz_new / rz);
-        rz = rz_new;
+      double rz = 0.0;
+      bool fresh = true, go_on = g0[0] > inner_thresh;
+      while (go_on && it < a.max_iter) {
+        double rzb[2];  // r.z, beta
+        bool positive;
+        const double rz_old = rz;
+        const bool first = fresh;
+        if (!vcycle(C, (const float*)r32, z32, ops, gwarp, nwarps, lane, rzb, positive,
+                    [rz_old, first](double t, double* o) {
+                      o[0] = t;
+                      o[1] = first ? 0.0 : t / rz_old;
+                      return t > 0.0 && isfinite(t);
+                    }))
+          return false;
+        if (!positive) break;  // refine with what the inner solve has
+        const float beta = (float)rzb[1];
+        rz = rzb[0];
         fresh = false;
         DotAcc<float> kpq;
         struct PreA {
           float z, q, p;
         };
-        spmv_stream<float, Ops::kStream>(
-            A32, ma, mb, lane, [z32](int c) { return __ldca(z32 + c); },
+        stream_rows<float, float>(
+            ops.ring, C.mat_phase(), lane, [z32](int c) { return __ldca(z32 + c); },
             [=](int i) { return PreA{__ldca(z32 + i), q32[i], p32[i]}; },
             [&](int i, float w, const PreA& o) {
-              const float qn = beta == 0.f ? w : fmaf(beta, o.q, w);  // (restart: old p, q unused)
-              const float pn = beta == 0.f ? o.z : fmaf(beta, o.p, o.z);
+              const float qn = first ? w : fmaf(beta, o.q, w);  // (restart: old p, q unused)
+              const float pn = first ? o.z : fmaf(beta, o.p, o.z);
               q32[i] = qn;
               p32[i] = pn;
               kpq.add(pn, qn);
             });
-        double pq[1] = {kpq.value()};
-        if (!ops.sum(pq)) return false;
-        const float alpha = (float)(rz / pq[0]);
+        double al[1];
+        bool more;
+        const double rz_now = rz;
+        if (!ops.template sum_epi<1>(kpq.value(), al, more, [rz_now](double t, double* o) {
+              o[0] = rz_now / t;
+              return false;
+            }))
+          return false;
+        const float alpha = (float)al[0];
         DotAcc<float> krr;
         for (int s = gwarp; s < nsl; s += nwarps) {
           const int i = s * kSlice + lane;
@@ -544,9 +647,12 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, Ops& ops, int gwarp, int nwarp
           r32[i] = r;
           krr.add(r, r);
         }
-        double rn[1] = {krr.value()};
-        if (!ops.sum(rn)) return false;
-        rr = rn[0];
+        if (!ops.template sum_epi<1>(krr.value(), al, more, [inner_thresh](double t, double* o) {
+              o[0] = t;
+              return t > inner_thresh;
+            }))
+          return false;
+        go_on = more;
         ++it;
       }
       if (it == it_outer) {  // the inner solve could not start: no progress is possible
@@ -580,82 +686,91 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, Ops& ops, int gwarp, int nwarp
 }
 
 
-// Grid-wide synchronisation of a cooperative launch (counter barrier of grid_sync.cuh).
-// kStream / kStream64: steps per batch of the streamed products with FP32 / FP64 values (8 and 8
-// for the whole-GPU kernels, measured fastest with their 24 warps per SM, and for the cluster
-// solves).
+// Grid-wide synchronisation of a cooperative launch (counter barrier of grid_sync.cuh); MAXV: most
+// values of one sum.  sum_epi evaluates `epi(total, out)` on one thread per block: a division or
+// comparison that every thread repeats costs a 1024-thread block 600 cycles per FP64 instruction
+// (a division 5,000), one thread 64.  It returns a flag, and up to three derived scalars in out.
+template <class R, int MAXV>
 struct GridOps {
-  // steps of 32 elements loaded ahead by the streamed products: FP32 operators, FP64 matrix.
-  // Measured on the pin-plane solve (500k rows, 1024 threads): 6 / 4 gave 99.9 us per CG
-  // iteration, 8 / 4 101.2, 4 / 4 104.9, 12 / 4 139 (register spills), 8 / 8 (with row batches
-  // of 4 in the down phase) 127
-  static constexpr int kStream = 6, kStream64 = 4;
   FlagSync& fs;
-  double* smem;
-  __device__ bool barrier() { return grid_barrier(fs); }
-  template <int NV>
-  __device__ bool sum(double (&v)[NV]) {
-    return grid_allsum<NV>(v, fs, smem);
+  R ring;
+  __device__ bool barrier() { return grid_barrier<MAXV>(fs); }
+  template <int NE, class Epi>
+  __device__ bool sum_epi(double v, double (&out)[NE], bool& flag, Epi epi) {
+    double s[1] = {v}, e[NE + 1];
+    if (!grid_allsum<1, NE + 1, MAXV>(s, e, fs, nullptr,
+                                      [&epi](const double* t, double* o) { o[NE] = epi(t[0], o) ? 1.0 : 0.0; }))
+      return false;
+#pragma unroll
+    for (int k = 0; k < NE; ++k) out[k] = e[k];
+    flag = __double2hiint(e[NE]) != 0;
+    return true;
+  }
+  __device__ bool sum(double (&v)[1]) {
+    double e[1];
+    return grid_allsum<1, 0, MAXV>(v, e, fs, nullptr, NoEpilogue());
   }
 };
 
 // Synchronisation of one thread-block cluster: hardware cluster barrier (release / acquire at
 // cluster scope, so global-memory writes of the cluster are visible after it) and sums through
-// distributed shared memory (at most 32 CTAs; deterministic: fixed shuffle tree over the ranks).
-// `part` (2 x 4 doubles), `wsum` (32 x 4 doubles) and `res` (4 doubles) are the calling CTA's
-// shared scratch.
-// S, S64: steps loaded ahead by the streamed FP32 / FP64 products (8 / 8 at 512 threads per CTA,
-// 6 / 4 at 768, where fewer registers are left per thread).
-template <int S, int S64>
-struct ClusterOpsT {
-  static constexpr int kStream = S, kStream64 = S64;
+// distributed shared memory (at most 16 CTAs; deterministic: fixed order of threads and ranks).
+// A CTA's partial is pushed into every CTA's table before the barrier, so that only local
+// shared memory is read after it.
+struct ClusterSums {
+  double thr[1024];     // per-thread values
+  double grp[4];
+  double part[2][16];   // [parity][rank]
+  double res[4];
+  int flag;
+};
+template <class R>
+struct ClusterOps {
   cooperative_groups::cluster_group cl;
-  double* part;  // [2][4]: this CTA's partials, double-buffered
-  double* wsum;  // [32][4]: warp partials
-  double* res;   // [4]: cluster totals for this CTA's threads
+  ClusterSums& sh;
+  R ring;
   unsigned seq;
   __device__ bool barrier() {
-    cl.sync();
+    cluster_sync();
     return true;
   }
-  template <int NV>
-  __device__ bool sum(double (&v)[NV]) {
-    static_assert(NV <= 4, "cluster sum: at most 4 values");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = v[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) wsum[warp * 4 + k] = t;
-    }
+  // Cluster barrier with one releasing fence per CTA (after bar.sync, so it covers the writes of
+  // all its threads) instead of one per thread: 2,250 -> 1,880 cycles at 16 x 512 threads with
+  // stores in flight.
+  __device__ void cluster_sync() {
     __syncthreads();
-    const int buf = seq & 1;
-    ++seq;
-    if (threadIdx.x < NV) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += wsum[w * 4 + threadIdx.x];
-      part[buf * 4 + threadIdx.x] = t;
-    }
-    cl.sync();
-    // warp 0 gathers the C partials (lane r reads rank r) and reduces them with a fixed
-    // shuffle tree; the totals reach the other warps through shared memory
+    if (threadIdx.x == 0) asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  template <int NE, class Epi>
+  __device__ bool sum_epi(double v, double (&out)[NE], bool& flag, Epi epi) {
+    static_assert(NE <= 4, "ClusterSums::res");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = (int)cl.num_blocks();
+    double* part = sh.part[seq++ & 1];
+    double s[1] = {v}, bt[1];
+    block_group_sum<1>(s, bt, sh.thr, sh.grp);
+    if (warp == 0 && lane < C) *cl.map_shared_rank(part + cl.block_rank(), lane) = bt[0];
+    cluster_sync();
     if (warp == 0) {
-      const int C = (int)cl.num_blocks();
+      double t = lane < C ? part[lane] : 0.0;
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        double t = lane < C ? *cl.map_shared_rank(part + buf * 4 + k, lane) : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) res[k] = t;
-      }
+      for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) sh.flag = epi(t, sh.res) ? 1 : 0;
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = res[k];
+    for (int k = 0; k < NE; ++k) out[k] = sh.res[k];
+    flag = sh.flag != 0;
     return true;
+  }
+  __device__ bool sum(double (&v)[1]) {
+    bool f;
+    return sum_epi<1>(v[0], v, f, [](double t, double* o) {
+      o[0] = t;
+      return false;
+    });
   }
 };
-using ClusterOps = ClusterOpsT<8, 8>;
 
 }  // namespace avip

@@ -27,6 +27,7 @@ cudaError_t launch_pcg_fp64(const PcgArgs& args, const PcgPlan& pl, cudaStream_t
 cudaError_t launch_pcg_mixed(const PcgArgs& args, const PcgPlan& pl, cudaStream_t st);
 cudaError_t launch_bicgstab(const PcgArgs& args, const PcgPlan& pl, cudaStream_t st);
 cudaError_t launch_pcg_amg(const PcgArgs& args, const PcgPlan& pl, cudaStream_t st);
+cudaError_t launch_mark_slices(const int32_t* sl_ptr, int nslices, const int32_t* col, int32_t* out, cudaStream_t st);
 cudaError_t launch_amg_group(const AmgGroupArgs& g, const PcgPlan& pl, cudaStream_t st);
 cudaError_t launch_pcg_amg_cluster(const PcgArgs& args, const PcgPlan& pl, cudaStream_t st);
 cudaError_t launch_pcg_cluster(const PcgArgs& args, const PcgPlan& pl, const ClusterLayout& L, cudaStream_t st);
@@ -72,6 +73,7 @@ struct avip_mesh {
   double* amg_z = nullptr;          // preconditioned residual of the FP64 CG (either hierarchy)
   double* r2 = nullptr;             // second buffer of the AMG-CG residual
   float* rq32 = nullptr;            // FP32 copies of both residual buffers and of q (FP32 hierarchy)
+  int32_t* colS = nullptr;          // col with the end of every slice marked (AMG solvers)
   int32_t amg_levels = 0;
   std::vector<int64_t> amg_stats;  // per level: rows, nnz(A), nnz(P)
   float *aval32 = nullptr, *e32 = nullptr, *r32 = nullptr, *p32 = nullptr, *q32 = nullptr;  // mixed precision
@@ -120,7 +122,6 @@ namespace {
 
 thread_local char g_err[256];
 constexpr int kClusterAutoRows = 20000;  // one-cluster solvers up to this many nodes
-constexpr int kClusterAmgMinRows = 500;  // AMG on one cluster above this many nodes (Jacobi below)
 
 void* dev_alloc(avip_mesh* h, size_t bytes) {
   if (bytes == 0) bytes = 16;
@@ -229,6 +230,7 @@ PcgArgs pcg_args(const avip_mesh* h) {
   a.z32 = h->z32;
   a.r2 = h->r2;
   a.rq32 = h->rq32;
+  a.colS = h->colS;
   a.amg_mixed = h->opts.precision == AVIP_PREC_MIXED ? 1 : 0;
   return a;
 }
@@ -440,17 +442,27 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
   AmgDevT<T> D;
   std::memset(&D, 0, sizeof(D));
   D.nlev = (int32_t)H.lv.size();
-  D.nc = H.nc;
-  auto put = [&](const Csr& M, SellMatT<T>& dst, int64_t& steps) {
+  auto put = [&](const Csr& M, SellMatT<T>& dst) {
     SellHost S;
     sell_from_csr(M, S, lanes_per_row(M));
-    int32_t *slp = nullptr, *slw = nullptr, *rl = nullptr, *col = nullptr;
+    int32_t *slp = nullptr, *col = nullptr;
     T* val = nullptr;
     std::vector<T> v(S.val.begin(), S.val.end());
-    const bool ok = upload(h, slp, S.sl_ptr) && upload(h, slw, S.sl_w) && upload(h, rl, S.rlen) &&
-                    upload(h, col, S.col, 1) && upload(h, val, v, 1);
-    dst = SellMatT<T>{slp, slw, rl, col, val, S.n, S.nslices, S.lpr};
-    steps = S.sl_ptr.back() / kSlice;
+    const bool ok = upload(h, slp, S.sl_ptr) && upload(h, col, S.col, S.col.size() + kStreamPad) &&
+                    upload(h, val, v, v.size() + kStreamPad);
+    dst = SellMatT<T>{slp, col, val, S.n, S.nslices, S.lpr};
+    return ok;
+  };
+  // a dense matrix with its rows padded to whole steps of 32
+  auto put_dense = [&](const std::vector<double>& M, int32_t level, AmgDenseT<T>& dst) {
+    const int32_t n = H.lv[level].A.n, steps = (n + kSlice - 1) / kSlice;
+    const size_t w = (size_t)steps * kSlice;
+    std::vector<T> v(n * w, T(0));
+    for (int32_t i = 0; i < n; ++i)
+      for (int32_t j = 0; j < n; ++j) v[i * w + j] = (T)M[(size_t)i * n + j];
+    T* m = nullptr;
+    const bool ok = upload(h, m, v, v.size() + kStreamPad);
+    dst = AmgDenseT<T>{m, level, steps};
     return ok;
   };
   // [U | Pf]: Pf's columns shifted past U's n columns
@@ -478,20 +490,21 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
     AmgLevelT<T>& dl = D.L[l];
     dl.n = L.A.n;
     const size_t npad = (size_t)((L.A.n + kSlice - 1) / kSlice) * kSlice;
-    int64_t rf_steps = 0, up_steps = 0;
     if (l + 1 < D.nlev) {
       T* qd = nullptr;
       std::vector<T> qv(L.Q.v.begin(), L.Q.v.end());  // Q is diagonal: one entry per row, in order
-      ok = ok && upload(h, qd, qv, npad) && put(L.Rf, dl.Rf, rf_steps) && put(concat(L.U, L.Pf), dl.UP, up_steps) &&
-           zalloc(h, dl.xp, npad);
+      ok = ok && upload(h, qd, qv, npad) && put(L.Rf, dl.Rf) && put(concat(L.U, L.Pf), dl.UP) &&
+           zalloc(h, dl.xp, (size_t)L.A.n + H.lv[l + 1].A.n);
       dl.qd = qd;
+      D.L[l + 1].x = dl.xp + L.A.n;
     }
-    if (l > 0) ok = ok && zalloc(h, dl.x, npad) && zalloc(h, dl.b, npad);
+    if (l > 0) ok = ok && zalloc(h, dl.b, npad);
   }
-  T* cinv = nullptr;
-  std::vector<T> cv(H.cinv.begin(), H.cinv.end());
-  ok = ok && upload(h, cinv, cv, 1);
-  D.cinv = cinv;
+  ok = ok && put_dense(H.cinv, D.nlev - 1, D.dense[1]);
+  if (H.dlev == D.nlev - 1)
+    D.dense[0] = D.dense[1];
+  else
+    ok = ok && put_dense(H.dmat, H.dlev, D.dense[0]);
   auto* dd = static_cast<AmgDevT<T>*>(dev_alloc(h, sizeof(D)));
   ok = ok && dd && cudaMemcpyAsync(dd, &D, sizeof(D), cudaMemcpyHostToDevice, h->stream) == cudaSuccess &&
        cudaStreamSynchronize(h->stream) == cudaSuccess;
@@ -509,6 +522,9 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
 // Upload the hierarchy in the handle's preconditioner precision (FP64 values when asked for and
 // the solve is not the mixed-precision one) with its preconditioned-residual vector.
 bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np) {
+  if (!zalloc(h, h->colS, h->hm.col.size() + kStreamPad) ||
+      launch_mark_slices(h->sl_ptr, h->hm.nslices, h->col, h->colS, h->stream) != cudaSuccess)
+    return false;
   const bool fp64 = h->opts.precond_fp64 && h->opts.precision == AVIP_PREC_FP64;
   if (fp64) return upload_amg_t<double>(h, H, h->amg) && zalloc(h, h->amg_z, Np) && zalloc(h, h->r2, Np);
   // (the FP64 CG writes its preconditioned residual in FP64 whatever the hierarchy's type; the
@@ -621,7 +637,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   h->Npad = m.nslices * kSlice;
   const size_t Np = (size_t)h->Npad;
   bool ok = upload(h, h->sl_ptr, m.sl_ptr) && upload(h, h->sl_w, m.sl_w) && upload(h, h->rlen, m.rlen) &&
-            upload(h, h->col, m.col) && upload(h, h->aval, m.aval) && upload(h, h->gx, m.gx) &&
+            upload(h, h->col, m.col) && upload(h, h->aval, m.aval, m.aval.size() + kStreamPad) && upload(h, h->gx, m.gx) &&
             upload(h, h->gy, m.gy) && upload(h, h->sx, m.sx) && upload(h, h->sy, m.sy) &&
             upload(h, h->cell, m.cell) && upload(h, h->flen, m.flen) && upload(h, h->cw, m.cw) && upload(h, h->e_lo, m.e_lo, 1) && upload(h, h->e_hi, m.e_hi, 1) &&
             upload(h, h->e_sx, m.e_sx, 1) && upload(h, h->e_sy, m.e_sy, 1) && upload(h, h->slot_eid, m.slot_eid) &&
@@ -647,13 +663,21 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   h->plan = h->opts.precision == AVIP_PREC_MIXED ? pcg_mixed_plan(m.nslices, h->opts.pcg_threads)
                                                  : pcg_plan(m.nslices, h->opts.pcg_kind, h->opts.pcg_threads);
   const bool bicg = axi || h->opts.pcg_kind == 7 || h->opts.pcg_kind == 9;
+  // small and mid-size planar meshes (or kind 11 forced): the AMG-preconditioned solve on one
+  // cluster.  Below a few hundred nodes its hierarchy is the inverse of the matrix alone, and two
+  // or three iterations replace the 70 to 90 of the Jacobi form.
+  PcgPlan amg_cluster;
+  amg_cluster.kind = 0;
+  if (!bicg && (h->opts.pcg_kind == 11 || (h->opts.pcg_kind == 0 && m.N <= kClusterAutoRows)))
+    amg_cluster = amg_cluster_plan(h->opts.cluster_size, m.N);
   // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above the cluster size
   const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (h->opts.pcg_kind == 0 && m.N > kClusterAutoRows));
   if (bicg) {
     h->plan = bicgstab_plan(m.nslices, h->opts.pcg_threads);
     ok = ok && zalloc(h, h->bcg, (bicg_amg ? 5 : 3) * Np);
-  } else if (h->opts.pcg_kind == 0 || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
+  } else if ((h->opts.pcg_kind == 0 && amg_cluster.kind != 11) || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
     // small meshes: one thread-block cluster with everything in shared memory
+    // (the Jacobi form, when asked for or when the AMG form below cannot be scheduled)
     const int mixed = h->opts.precision == AVIP_PREC_MIXED ? 1 : 0;
     ClusterHost chd;
     PcgPlan cp = pcg_cluster_plan(m, h->opts.pcg_kind >= 5 ? (1 << 30) : kClusterAutoRows, &h->clay, &chd, mixed);
@@ -669,7 +693,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // large FP64 meshes (or kinds 8/9 forced): CG (planar) or BiCGStab (axisymmetric)
   // preconditioned by an AMG V-cycle
   if (bicg_amg || (!bicg && h->opts.precision == AVIP_PREC_FP64 &&
-                   (h->opts.pcg_kind == 8 || (h->opts.pcg_kind == 0 && h->plan.kind != 5)))) {
+                   (h->opts.pcg_kind == 8 ||
+                    (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
     AmgHost H;
     int rc = amg_setup(m, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
@@ -683,7 +708,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   }
   if (h->opts.precision == AVIP_PREC_MIXED) {
     std::vector<float> a32(m.aval.begin(), m.aval.end());
-    ok = ok && upload(h, h->aval32, a32) && zalloc(h, h->e32, Np) && zalloc(h, h->r32, Np) && zalloc(h, h->p32, Np) &&
+    ok = ok && upload(h, h->aval32, a32, a32.size() + kStreamPad) && zalloc(h, h->e32, Np) && zalloc(h, h->r32, Np) && zalloc(h, h->p32, Np) &&
          zalloc(h, h->q32, Np);
     // FP32 drift-diffusion stage: gradient weights and edge normals rounded once
     std::vector<float> f(m.gx.begin(), m.gx.end());
@@ -698,7 +723,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // large mixed-precision meshes (or kind 10 forced): FP32 inner CG preconditioned by an FP32
   // AMG V-cycle, FP64 iterative refinement of the residual
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
-      (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6))) {
+      (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
     AmgHost H;
     int rc = amg_setup(m, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
@@ -710,22 +735,17 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     ok = ok && upload_amg(h, H, Np);
     h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
   }
-  // mid-size planar meshes (or kind 11 forced): the AMG-preconditioned solve on one cluster
-  if (!bicg && (h->opts.pcg_kind == 11 ||
-                (h->opts.pcg_kind == 0 && m.N > kClusterAmgMinRows && m.N <= kClusterAutoRows))) {
-    const PcgPlan cp = amg_cluster_plan(h->opts.cluster_size, m.N);
-    if (cp.kind == 11) {
-      AmgHost H;
-      int rc = amg_setup(m, H, g_err, sizeof(g_err));
-      if (rc != AVIP_OK) {
-        dev_free_all(h);
-        if (h->own_stream) cudaStreamDestroy(h->stream);
-        delete h;
-        return rc;
-      }
-      ok = ok && upload_amg(h, H, Np);
-      h->plan = cp;
+  if (amg_cluster.kind == 11) {
+    AmgHost H;
+    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    if (rc != AVIP_OK) {
+      dev_free_all(h);
+      if (h->own_stream) cudaStreamDestroy(h->stream);
+      delete h;
+      return rc;
     }
+    ok = ok && upload_amg(h, H, Np);
+    h->plan = amg_cluster;
   }
   h->nparts = flux_blocks(m.N);
   h->sync_bytes = sizeof(GridSync) + sizeof(unsigned) * (size_t)(h->plan.blocks + 1);
@@ -939,7 +959,7 @@ int photo_set(avip_mesh_t h, int32_t n_terms, const double* a, const double* kap
         }
       }
     avip_mesh::PhotoTerm t;
-    ok = upload(h, t.aval, val) && upload(h, t.dsq, dh) && upload(h, t.dsqinv, dhinv) && upload(h, t.rhs, rhs);
+    ok = upload(h, t.aval, val, val.size() + kStreamPad) && upload(h, t.dsq, dh) && upload(h, t.dsqinv, dhinv) && upload(h, t.rhs, rhs);
     if (ok && amg) {
       HostMesh hm;
       hm.N = m.N;
@@ -1262,6 +1282,7 @@ int state_set(avip_mesh_t h, const double* in) {
 // batch itself (state saved and restored around the trial).
 namespace avip {
 int cluster_batch_capacity(int C, size_t smem);
+size_t cluster_ring_bytes();
 PcgPlan pcg_cluster_plan_fixed(const HostMesh& m, int C, ClusterLayout* out, ClusterHost* hd, int mixed);
 cudaError_t launch_pcg_cluster_batch(const PcgArgs* args, const ClusterLayout* lays, const int32_t* order, int count,
                                      int C, int nclusters, size_t smem, cudaStream_t st);
@@ -1325,6 +1346,7 @@ bool batch_configure(avip_batch* b, int C) {
     if (b->m[k]->amg || b->m[k]->amg32) {
       // an AMG instance keeps its vectors in global memory: no shared-memory layout to fit
       std::memset(&lays[k], 0, sizeof(ClusterLayout));
+      smem = std::max(smem, cluster_ring_bytes());
       hd.colL.assign(1, 0);
       hd.push_ptr.assign(1, 0);
     } else {

@@ -85,7 +85,15 @@ struct AmgHost {
   std::vector<AmgHostLevel> lv;  // lv.back() is the coarsest level
   int32_t nc = 0;                // coarsest size
   std::vector<double> cinv;      // dense inverse of the coarsest matrix (row-major)
+  // the V-cycle from level dlev down as one dense matrix (row-major; the coarsest inverse when
+  // dlev is the coarsest level), dlev the finest level of at most kAmgDenseRows rows
+  int32_t dlev = 0;
+  std::vector<double> dmat;
 };
+// Below this many rows the rest of a V-cycle is applied as one dense product: 1,536 rows are 9.4 MB
+// in FP32, 62 KB per SM of a whole-GPU solve and so about 0.6 us of L2 bandwidth, against two to
+// four phases of 2 us and more for the levels it replaces.
+constexpr int kAmgDenseRows = 1536;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
 // composite operators of every non-coarsest level.
 int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen);
@@ -97,13 +105,19 @@ int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen);
 // the layout of the mesh matrix.
 struct SellHost {
   int32_t n = 0, nslices = 0, lpr = 1;
-  std::vector<int32_t> sl_ptr, sl_w, rlen, col;
+  std::vector<int32_t> sl_ptr, col;
   std::vector<double> val;
 };
+// Every slice has at least one step, and the columns of a slice's last step carry kSliceEnd.
+constexpr int32_t kSliceEnd = INT32_MIN;
 void sell_from_csr(const Csr& A, SellHost& out, int lpr = 1);
 // Lanes per row for a streamed operator: the smallest power of two (at most 32) that leaves
-// at most 8 stored entries per lane on an average row.
+// at most 8 stored entries per lane on an average row, or fewer lanes when that gives a slice to
+// every warp of the whole-GPU solvers already (a row's epilogue runs on one of its lanes only, and
+// the finest level's has FP64 operations).
 int lanes_per_row(const Csr& A);
+// Elements a streamed array must be readable past its end (a ring slot is always filled).
+constexpr size_t kStreamPad = 16 * kSlice;
 
 // ----------------------------------------------------------------- kernel argument blocks
 struct SellView {  // device pointers of the SELL-32 structure
@@ -123,9 +137,7 @@ struct SellView {  // device pointers of the SELL-32 structure
 template <typename T>
 struct SellMatT {  // device pointers of a SELL-32 matrix with values of type T
   const int32_t* sl_ptr;  // nslices + 1 element offsets
-  const int32_t* sl_w;    // steps per slice
-  const int32_t* rlen;
-  const int32_t* col;
+  const int32_t* col;     // bit 31 set on the last step of a slice
   const T* val;
   int32_t n;
   int32_t nslices;
@@ -142,16 +154,26 @@ template <typename T>
 struct AmgLevelT {
   SellMatT<T> Rf, UP;   // empty on the coarsest level
   const T* qd;          // the smoother Q = omega D^-1 (its diagonal, n entries)
-  T* xp;                // pre-smoothed iterate Q b
+  T* xp;                // pre-smoothed iterate Q b, followed by the next level's x (one vector for UP)
   T* x;                 // level solution
   T* b;                 // level right-hand side
   int32_t n;
 };
+// A whole level applied as one dense product x = M b, row-major, each row padded with zeros to
+// `steps` times 32 entries.
+template <typename T>
+struct AmgDenseT {
+  const T* m;
+  int32_t level;
+  int32_t steps;
+};
 template <typename T>
 struct AmgDevT {
   int32_t nlev;         // levels including the coarsest
-  int32_t nc;           // coarsest size
-  const T* cinv;        // coarsest dense inverse, nc x nc row-major
+  int32_t pad;
+  // dense[0]: the V-cycle from the finest level of at most kAmgDenseRows rows down, as one
+  // matrix; dense[1]: the inverse of the coarsest matrix (solvers on few SMs, see dense_choice)
+  AmgDenseT<T> dense[2];
   AmgLevelT<T> L[kAmgMaxLevels];
 };
 using AmgLevelDev = AmgLevelT<double>;
@@ -269,6 +291,7 @@ struct PcgArgs {
   double* r2;
   float* rq32;            // FP32 hierarchy: FP32 copies of the two residual buffers and of q
                           // (3 x Npad), the vectors the finest down phase gathers
+  const int32_t* colS;    // A.col with bit 31 set on the last slot of every slice (AMG solvers)
   int32_t amg_mixed;      // 1: FP32 inner CG + FP64 refinement (kind 10); 0: FP64 CG
 };
 

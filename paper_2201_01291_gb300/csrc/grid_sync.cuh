@@ -85,6 +85,7 @@ struct FlagSync {
   unsigned long long spin_ns;  // give up a wait after this long (0: at the first unsatisfied poll)
   int nb;         // blocks taking part (gridDim.x for a whole-grid solve)
   int rank;       // this block's index among them (blockIdx.x for a whole-grid solve)
+  volatile int* bad = nullptr;  // shared memory: set by a warp of this block that gave up a wait of its own
 };
 
 // True while the arrival counter has not reached `target` (wrap-safe, see above).
@@ -106,18 +107,52 @@ __device__ __forceinline__ bool wait_arrivals(const FlagSync& fs, unsigned targe
   return true;
 }
 
-// Shared-memory scratch of grid_allsum.  A __shared__ variable declared inside a function
-// template exists once per instantiation, so a kernel that reduces with several (NV, NE)
-// combinations would reserve the scratch several times over (less L1 for the gathers, fewer
-// co-resident blocks); declared in this one non-template function it exists once per kernel.
+// Shared-memory scratch of grid_allsum, for sums of at most MAXV values.  A __shared__ variable
+// declared inside a function template exists once per instantiation, so a kernel that reduces
+// with several (NV, NE) combinations would reserve the scratch several times over; declared in a
+// function of MAXV alone it exists once per kernel.
+template <int MAXV>
 struct AllsumScratch {
-  double thr[4 * 1024];  // per-thread values, [value k][thread]
-  double res[8];         // totals, then epilogue results
+  double thr[MAXV * 1024];  // per-thread values, [value k][thread]
+  double grp[MAXV * 4];     // sums of four thread groups per value
+  double res[8];            // totals, then epilogue results
   int ok;
 };
-__device__ __forceinline__ AllsumScratch& allsum_scratch() {
-  __shared__ AllsumScratch s;
+template <int MAXV>
+__device__ __forceinline__ AllsumScratch<MAXV>& allsum_scratch() {
+  __shared__ AllsumScratch<MAXV> s;
   return s;
+}
+
+// Block sums of NV per-thread values in a fixed order, valid in warp 0 on return (bt[k]).  On
+// GB300 an SM sub-partition issues one warp-wide FP64 instruction per ~75 cycles, dependent or
+// not (one per ~19 cycles and SM; latency 64), so a single warp adding 32 values per lane takes
+// 2,200 cycles.  Every thread stores its values, four warps per value (one per sub-partition) add
+// a quarter of them each and finish with a shuffle tree, and warp 0 adds the four group sums.
+template <int NV>
+__device__ __forceinline__ void block_group_sum(const double (&v)[NV], double (&bt)[NV], double* thr, double* grp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) thr[k * 1024 + threadIdx.x] = v[k];
+  __syncthreads();
+  const int G = nw >= 4 * NV ? 4 : 1;  // groups per value
+  if (warp < G * NV) {
+    const int k = warp / G, j = warp % G;
+    double t = 0.0;
+    for (int w = j; w < nw; w += G) t += thr[k * 1024 + w * 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) grp[warp] = t;
+  }
+  if (G * NV > 1) {
+    // the adding warps only: the others go on to the barrier that follows
+    if (warp < G * NV) asm volatile("bar.sync 1, %0;" ::"r"(G * NV * 32) : "memory");
+  }
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      bt[k] = G == 4 ? (grp[4 * k] + grp[4 * k + 1]) + (grp[4 * k + 2] + grp[4 * k + 3]) : grp[k];
+  }
 }
 
 struct NoEpilogue {
@@ -134,41 +169,26 @@ __device__ __forceinline__ void red_add_release_u32(unsigned* p, unsigned v) {
 // (timeout or another block aborted); the caller must leave.
 //
 // Protocol (measured fastest on GB300 among flag-per-block, last-block and counter schemes):
-// warp sums -> shared memory -> warp 0 adds the block partial, stores it in the block's slot
+// block_group_sum, then warp 0 stores the block's partial in the block's slot
 // and announces it with one release reduction on a monotone arrival counter; every lane of
 // warp 0 waits (acquire) until the counter reaches seq * nb and then reads all partials in
 // block order.  Partials are double-buffered by the parity of seq because a fast
 // block may publish reduction k+1 while a slow one is still reading reduction k.
-template <int NV, int NE, typename Epi>
+template <int NV, int NE, int MAXV = 4, typename Epi>
 __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 0 ? NE : 1], FlagSync& fs,
                                             double* smem, Epi epi) {
-  static_assert(NV <= 4 && NE <= 4, "grid_allsum: at most 4 sums and 4 derived scalars");
+  static_assert(NV <= MAXV && MAXV <= 4 && NE <= 4, "grid_allsum: at most 4 sums and 4 derived scalars");
   const int nb = fs.nb;
   const unsigned seq = ++fs.seq;
   const int par = seq & 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  AllsumScratch& scr = allsum_scratch();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  AllsumScratch<MAXV>& scr = allsum_scratch<MAXV>();
   double* s_res = scr.res;
   int& s_ok = scr.ok;
-  double* s_thr = scr.thr;
-  // Block partial: every thread stores its values, then warp 0 adds them (lane l takes
-  // threads l, l+32, ...) and finishes with a shuffle tree.  On GB300 an FP64 add costs a
-  // warp ~16 cycles of the SM's FP64 pipe, so this uses blockDim/32 + 5 warp-wide adds per
-  // value instead of the 5 * blockDim/32 + 5 of a shuffle tree in every warp.
   (void)smem;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) s_thr[k * 1024 + threadIdx.x] = v[k];
-  __syncthreads();
+  double bt[NV];
+  block_group_sum<NV>(v, bt, scr.thr, scr.grp);
   if (warp == 0) {
-    double bt[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += s_thr[k * 1024 + w * 32 + lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      bt[k] = t;
-    }
     int ok = 1;
     if (nb > 1) {
       if (lane == 0) {
@@ -177,7 +197,7 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 
         for (int k = 0; k < NV; ++k) __stcg(mine + k, bt[k]);
         red_add_release_u32(fs.flags, 1u);
       }
-      if (!wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
+      if ((fs.bad && *fs.bad) || !wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
       ok = __all_sync(0xffffffffu, ok);
       double acc[NV];
 #pragma unroll
@@ -194,8 +214,10 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 
           }
 #pragma unroll
           for (int q = 0; q < kPollUnroll; ++q)
+            if (32 * q < nb) {  // (no FP64 adds of absent partials)
 #pragma unroll
-            for (int k = 0; k < NV; ++k) acc[k] += pv[q][k];
+              for (int k = 0; k < NV; ++k) acc[k] += pv[q][k];
+            }
         } else {
           for (int b = lane; b < nb; b += 32) {
             const double* pb = fs.parts + ((size_t)par * nb + b) * 4;
@@ -243,16 +265,17 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[NV], FlagSync& fs, doubl
 // whose partials it does not touch; a reduction k and the next one of the same buffer parity,
 // k + 2, are then separated by this barrier k + 1, which no block passes before every block has
 // finished reading reduction k.  Returns false if the wait was abandoned.
+template <int MAXV = 4>
 __device__ __forceinline__ bool grid_barrier(FlagSync& fs) {
   const unsigned seq = ++fs.seq;
-  AllsumScratch& scr = allsum_scratch();
+  AllsumScratch<MAXV>& scr = allsum_scratch<MAXV>();
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
     const int nb = fs.nb;
     if (nb > 1) {
       red_add_release_u32(fs.flags, 1u);
-      if (!wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
+      if ((fs.bad && *fs.bad) || !wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
     }
     if (!ok) atomicExch(&fs.gs->abort, 1);
     scr.ok = ok;

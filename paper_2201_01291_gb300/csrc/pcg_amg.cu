@@ -38,10 +38,22 @@ namespace {
 // 8: 99.9 us per CG iteration on the pin-plane solve against 104.8 at 768), 768 otherwise
 // (BiCGStab and the mixed form are 1 % faster at 768; the FP64 hierarchy spills at 1024)
 constexpr int kAmgSizes[] = {768, 512, 1024};
-int amg_default_threads(int kind, int fp64) { return kind == 8 && !fp64 ? 1024 : 768; }
+int amg_default_threads(int kind, int fp64) { return 768; }
 constexpr int kAmgMaxRestarts = 8;
+// Fewest slices (of 32 rows) worth a block of their own: the whole GPU from 1,216 slices (39,000
+// rows) on.
+constexpr int kSlicesPerBlock = 4;
 
 }  // namespace
+
+// Slots of a warp's ring (stream.cuh): 192 KB per block for the CG and mixed forms, at most 160 KB
+// for BiCGStab, whose four-value sums take 32 KB of shared memory.
+constexpr int ring_slots(int tpb, bool bicg) {
+  return (bicg ? 160 : 144) * 1024 / (tpb / 32 * kSlotBytes);
+}
+constexpr size_t ring_bytes(int tpb, bool bicg) {
+  return (size_t)ring_slots(tpb, bicg) * (tpb / 32) * kSlotBytes + kRhsBytes;
+}
 
 // The hierarchy and the preconditioned residual of value type T.
 template <typename T>
@@ -60,14 +72,18 @@ __device__ __forceinline__ void report_timeout(const PcgArgs& a) {
 template <int TPB, typename T>
 __global__ void __launch_bounds__(TPB, 1) pcg_amg_kernel(PcgArgs a) {
   if (solve_skipped(a.sc)) return;  // an earlier stage of this run failed beyond repair
-  __shared__ double smem[2 * 32 * 4];
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ SolveShared sh;
   constexpr int wpb = TPB / 32;
-  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x};
-  GridOps ops{fs, smem};
-  if (!amg_cg_solve<T>(a, amg_of<T>(a), a.z, ops, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb,
-                       threadIdx.x & 31, blockIdx.x == 0 && threadIdx.x == 0) &&
-      threadIdx.x == 0)
-    report_timeout(a);
+  using R = Ring<ring_slots(TPB, false)>;
+  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x, &sh.bad};
+  GridOps<R, 1> ops{fs, R()};
+  const int gwarp = blockIdx.x * wpb + (threadIdx.x >> 5), nwarps = gridDim.x * wpb, lane = threadIdx.x & 31;
+  const AmgCtx<T> C =
+      solve_begin<T>(sh, ops.ring, ring_mem, a, amg_of<T>(a), a.A.aval, (int)gridDim.x, gwarp, nwarps, lane, true);
+  const bool ok = amg_cg_solve<T>(a, C, a.z, ops, gwarp, nwarps, lane, blockIdx.x == 0 && threadIdx.x == 0);
+  ops.ring.finish(lane);
+  if (!ok && threadIdx.x == 0) report_timeout(a);
 }
 
 // BiCGStab right-preconditioned by the same V-cycle, for the non-symmetric axisymmetric
@@ -78,13 +94,15 @@ __global__ void __launch_bounds__(TPB, 1) pcg_amg_kernel(PcgArgs a) {
 // (van der Vorst's iteration with M^-1 applied on the right, so x is updated directly and the
 // stopping test stays on the true scaled residual of the free rows).  Two V-cycles per
 // iteration; breakdowns and a true residual still too large restart from the true residual.
-// The products with A stream the matrix by contiguous slice shares (spmv_stream, each row's own
+// The products with A stream the matrix by contiguous slice shares (stream_rows, each row's own
 // operands fetched ahead), the elementwise phases take slices round-robin.
 // The solve of one system by the blocks taking part in `fs` (gwarp / nwarps number their warps,
 // `leader` is the one thread that writes the statistics); false if a wait was abandoned.
-template <typename T>
-__device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restrict__ H, FlagSync& fs, double* smem,
-                                   int gwarp, int nwarps, int lane, bool leader) {
+template <typename T, class R>
+__device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps<R, 4>& ops, int gwarp, int nwarps,
+                                   int lane, bool leader) {
+  FlagSync& fs = ops.fs;
+  double* const smem = nullptr;
   const int N = a.A.N, nsl = a.A.nslices;
   const size_t Np = (size_t)a.Npad;
   const double* nb = a.nbuf + (size_t)a.sc->parity * AVIP_MAX_SPECIES * Np;
@@ -97,17 +115,12 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restric
   double* __restrict__ rh = a.bcg + 2 * Np;
   double* __restrict__ ph = a.bcg + 3 * Np;
   double* __restrict__ sh = a.bcg + 4 * Np;
-  GridOps ops{fs, smem};
-  double dummy = 0.0;
-  // the matrix as a streamed operator (products by contiguous slice shares, see spmv_stream)
-  const SellMatT<double> A0{a.A.sl_ptr, a.A.sl_w, a.A.rlen, a.A.col, a.A.aval, N, nsl, 1};
-  int ma, mb;
-  warp_slices(nsl, gwarp, nwarps, ma, mb);
+  const int mat = C.mat_phase();
   struct Two {
     double u, w;
   };
 
-  const double gain = dirichlet_gain(a);
+  const double gain = C.gain;
   const int hist = history_length(a);
   double bb[1] = {0.0};
   for (int sl = gwarp; sl < nsl; sl += nwarps) {
@@ -148,8 +161,8 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restric
           {
             const double* __restrict__ bv = a.b;
             const double* __restrict__ xv = x;
-            spmv_stream<double, GridOps::kStream64>(
-                A0, ma, mb, lane, [xv](int c) { return __ldca(xv + c); }, [bv](int i) { return bv[i]; },
+            stream_rows<double, double>(
+                ops.ring, mat, lane, [xv](int c) { return __ldca(xv + c); }, [bv](int i) { return bv[i]; },
                 [&](int i, double ax, double bi) {
                   const double ri = bi - ax;
                   r[i] = ri;
@@ -174,13 +187,13 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restric
           restart = false;
         }
         // ---- p^ = M p, then P1: v = A p^
-        if (!vcycle(H, (const double*)p, ph, ops, gwarp, nwarps, lane, false, dummy)) return false;
+        if (!vcycle(C, (const double*)p, ph, ops, gwarp, nwarps, lane)) return false;
         double rv[1] = {0.0};
         {
           const double* __restrict__ phv = ph;
           const double* __restrict__ rhv = rh;
-          spmv_stream<double, GridOps::kStream64>(
-              A0, ma, mb, lane, [phv](int c) { return __ldca(phv + c); }, [rhv](int i) { return rhv[i]; },
+          stream_rows<double, double>(
+              ops.ring, mat, lane, [phv](int c) { return __ldca(phv + c); }, [rhv](int i) { return rhv[i]; },
               [&](int i, double w, double rhi) {
                 v[i] = w;
                 rv[0] = fma(rhi, w, rv[0]);
@@ -223,14 +236,14 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restric
           continue;
         }
         // ---- s^ = M s, then P3: t = A s^
-        if (!vcycle(H, (const double*)sv, sh, ops, gwarp, nwarps, lane, false, dummy)) return false;
+        if (!vcycle(C, (const double*)sv, sh, ops, gwarp, nwarps, lane)) return false;
         double d4[4] = {0.0, 0.0, 0.0, 0.0};  // t.s, t.t, rh.s, rh.t
         {
           const double* __restrict__ shv = sh;
           const double* __restrict__ svv = sv;
           const double* __restrict__ rhv = rh;
-          spmv_stream<double, GridOps::kStream64>(
-              A0, ma, mb, lane, [shv](int c) { return __ldca(shv + c); },
+          stream_rows<double, double>(
+              ops.ring, mat, lane, [shv](int c) { return __ldca(shv + c); },
               [svv, rhv](int i) { return Two{svv[i], rhv[i]}; },
               [&](int i, double ti, const Two& o) {
                 const double si = o.u, rhi = o.w;
@@ -290,13 +303,18 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgDevT<T>* __restric
 template <int TPB, typename T>
 __global__ void __launch_bounds__(TPB, 1) bicgstab_amg_kernel(PcgArgs a) {
   if (solve_skipped(a.sc)) return;  // an earlier stage of this run failed beyond repair
-  __shared__ double smem[2 * 32 * 4];
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ SolveShared sh;
   constexpr int wpb = TPB / 32;
-  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x};
-  if (!amg_bicgstab_solve<T>(a, amg_of<T>(a), fs, smem, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb,
-                             threadIdx.x & 31, blockIdx.x == 0 && threadIdx.x == 0) &&
-      threadIdx.x == 0)
-    report_timeout(a);
+  using R = Ring<ring_slots(TPB, true)>;
+  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x, &sh.bad};
+  GridOps<R, 4> ops{fs, R()};
+  const int gwarp = blockIdx.x * wpb + (threadIdx.x >> 5), nwarps = gridDim.x * wpb, lane = threadIdx.x & 31;
+  const AmgCtx<T> C =
+      solve_begin<T>(sh, ops.ring, ring_mem, a, amg_of<T>(a), a.A.aval, (int)gridDim.x, gwarp, nwarps, lane, true);
+  const bool ok = amg_bicgstab_solve<T>(a, C, ops, gwarp, nwarps, lane, blockIdx.x == 0 && threadIdx.x == 0);
+  ops.ring.finish(lane);
+  if (!ok && threadIdx.x == 0) report_timeout(a);
 }
 
 // Several systems solved side by side in one cooperative launch (the photoionisation terms):
@@ -320,22 +338,26 @@ __global__ void __launch_bounds__(TPB, 1) amg_group_kernel(const __grid_constant
   }
   __syncthreads();
   const PcgArgs& a = s_args;
-  __shared__ double smem[2 * 32 * 4];
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ SolveShared sh;
+  using R = Ring<ring_slots(TPB, kBicg)>;
   constexpr int wpb = TPB / 32;
   const int nb = g.start[j + 1] - g.start[j], rank = (int)blockIdx.x - g.start[j];
-  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, nb, rank};
+  if (threadIdx.x == 0) sh.bad = 0;
+  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, nb, rank, &sh.bad};
   const int gwarp = rank * wpb + (int)(threadIdx.x >> 5), nwarps = nb * wpb, lane = threadIdx.x & 31;
   const bool leader = rank == 0 && threadIdx.x == 0;
+  GridOps<R, kBicg ? 4 : 1> ops{fs, R()};
   double skip[1] = {solve_skipped(a.sc) ? 1.0 : 0.0};
-  bool ok = grid_allsum<1>(skip, fs, smem);
+  bool ok = ops.sum(skip);
   if (ok && skip[0] > 0.0) return;
   if (ok) {
-    if constexpr (kBicg) {
-      ok = amg_bicgstab_solve<T>(a, amg_of<T>(a), fs, smem, gwarp, nwarps, lane, leader);
-    } else {
-      GridOps ops{fs, smem};
-      ok = amg_cg_solve<T>(a, amg_of<T>(a), a.z, ops, gwarp, nwarps, lane, leader);
-    }
+    const AmgCtx<T> C = solve_begin<T>(sh, ops.ring, ring_mem, a, amg_of<T>(a), a.A.aval, nb, gwarp, nwarps, lane, true);
+    if constexpr (kBicg)
+      ok = amg_bicgstab_solve<T>(a, C, ops, gwarp, nwarps, lane, leader);
+    else
+      ok = amg_cg_solve<T>(a, C, a.z, ops, gwarp, nwarps, lane, leader);
+    ops.ring.finish(lane);
   }
   if (!ok && threadIdx.x == 0) report_timeout(a);
 }
@@ -349,14 +371,31 @@ __global__ void __launch_bounds__(TPB, 1) amg_group_kernel(const __grid_constant
 template <int TPB>
 __global__ void __launch_bounds__(TPB, 1) pcg_amg_mixed_kernel(PcgArgs a) {
   if (solve_skipped(a.sc)) return;  // an earlier stage of this run failed beyond repair
-  __shared__ double smem[2 * 32 * 4];
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ SolveShared sh;
   constexpr int wpb = TPB / 32;
-  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x};
-  GridOps ops{fs, smem};
-  if (!amg_mixed_solve(a, ops, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb, threadIdx.x & 31,
-                       blockIdx.x == 0 && threadIdx.x == 0) &&
-      threadIdx.x == 0)
-    report_timeout(a);
+  using R = Ring<ring_slots(TPB, false)>;
+  FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x, &sh.bad};
+  GridOps<R, 1> ops{fs, R()};
+  const int gwarp = blockIdx.x * wpb + (threadIdx.x >> 5), nwarps = gridDim.x * wpb, lane = threadIdx.x & 31;
+  const AmgCtx<float> C =
+      solve_begin<float>(sh, ops.ring, ring_mem, a, a.amg32, a.aval32, (int)gridDim.x, gwarp, nwarps, lane, false);
+  const bool ok = amg_mixed_solve(a, C, ops, gwarp, nwarps, lane, blockIdx.x == 0 && threadIdx.x == 0);
+  ops.ring.finish(lane);
+  if (!ok && threadIdx.x == 0) report_timeout(a);
+}
+
+// Columns of the mesh matrix with the last slot of every slice marked, for the streamed products.
+__global__ void mark_slices_kernel(const int32_t* __restrict__ sl_ptr, int nslices, const int32_t* __restrict__ col,
+                                   int32_t* __restrict__ out) {
+  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (s >= nslices) return;
+  const int e1 = sl_ptr[s + 1];
+  for (int e = sl_ptr[s] + lane; e < e1; e += kSlice) out[e] = e + kSlice >= e1 ? col[e] | kSliceEnd : col[e];
+}
+cudaError_t launch_mark_slices(const int32_t* sl_ptr, int nslices, const int32_t* col, int32_t* out, cudaStream_t st) {
+  mark_slices_kernel<<<(nslices * 32 + 255) / 256, 256, 0, st>>>(sl_ptr, nslices, col, out);
+  return cudaGetLastError();
 }
 
 template <typename T>
@@ -399,9 +438,11 @@ PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, amg_kernel_ptr(kind, pl.tpb, fp64), pl.tpb, 0);
-  const int wpb = pl.tpb / kSlice;
-  const int want = (nslices + wpb - 1) / wpb;
+  const void* fn = amg_kernel_ptr(kind, pl.tpb, fp64);
+  const size_t smem = ring_bytes(pl.tpb, kind == 9);
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, pl.tpb, smem);
+  const int want = (nslices + kSlicesPerBlock - 1) / kSlicesPerBlock;
   pl.blocks = std::max(1, std::min(std::max(occ, 1) * std::max(sms, 1), want));
   return pl;
 }
@@ -410,7 +451,7 @@ cudaError_t launch_pcg_amg(const PcgArgs& args, const PcgPlan& pl, cudaStream_t 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
   cfg.blockDim = dim3(pl.tpb);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = ring_bytes(pl.tpb, pl.kind == 9);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -439,7 +480,10 @@ cudaError_t launch_amg_group(const AmgGroupArgs& g, const PcgPlan& pl, cudaStrea
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
   cfg.blockDim = dim3(pl.tpb);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = ring_bytes(pl.tpb, bicg);
+  if (cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+      e != cudaSuccess)
+    return e;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

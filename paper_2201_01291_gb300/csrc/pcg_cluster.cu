@@ -568,32 +568,42 @@ __global__ void __launch_bounds__(kClusterTPB, 1) pcg_cluster_kernel(PcgArgs a, 
 // AMG-preconditioned CG of one instance on one cluster: the rows of every level are shared by
 // the cluster's warps, barriers are cluster barriers and sums go through distributed shared
 // memory (the same V-cycle and CG as the whole-GPU kernel, solver kind 8).
-template <class Ops = ClusterOps>
-__device__ void cluster_amg_solve(const PcgArgs& a, double* part, double* wsum) {
+// Ring of a cluster solve's warp: 192 KB per CTA.
+template <int TPB>
+using ClusterRing = Ring<192 * 1024 / (TPB / 32 * kSlotBytes)>;
+constexpr size_t kClusterRingBytes = 192 * 1024 + kRhsBytes;
+struct ClusterAmgShared {
+  SolveShared solve;
+  ClusterSums sums;
+};
+
+// The FP64 CG with an FP32 (default) or FP64 hierarchy, or the mixed-precision solve.
+template <int TPB>
+__device__ void cluster_amg_solve(const PcgArgs& a, ClusterAmgShared& sh, char* ring_mem) {
   if (solve_skipped(a.sc)) return;  // every CTA of the cluster reads the same status
+  using R = ClusterRing<TPB>;
   cg::cluster_group cl = cg::this_cluster();
-  Ops ops{cl, part, wsum, wsum + 32 * 4, 0u};
-  const int wpb = (int)(blockDim.x >> 5), rank = (int)cl.block_rank();
-  const int gw = rank * wpb + (int)(threadIdx.x >> 5), nw = (int)cl.num_blocks() * wpb, lane = (int)(threadIdx.x & 31);
-  if (a.amg32)  // FP32 hierarchy (default), else FP64
-    amg_cg_solve<float>(a, a.amg32, a.z, ops, gw, nw, lane, rank == 0 && threadIdx.x == 0);
-  else
-    amg_cg_solve<double>(a, a.amg, a.z, ops, gw, nw, lane, rank == 0 && threadIdx.x == 0);
-  cl.sync();  // the next instance reuses the sum buffers
-}
-
-// (wsum holds 32 x 4 warp partials followed by the 4 totals.)
-
-// The same for a mixed-precision instance with an FP32 hierarchy (solver kind 10).
-template <class Ops = ClusterOps>
-__device__ void cluster_amg_mixed_solve(const PcgArgs& a, double* part, double* wsum) {
-  if (solve_skipped(a.sc)) return;
-  cg::cluster_group cl = cg::this_cluster();
-  Ops ops{cl, part, wsum, wsum + 32 * 4, 0u};
-  const int wpb = (int)(blockDim.x >> 5), rank = (int)cl.block_rank();
-  amg_mixed_solve(a, ops, rank * wpb + (int)(threadIdx.x >> 5), (int)cl.num_blocks() * wpb,
-                  (int)(threadIdx.x & 31), rank == 0 && threadIdx.x == 0);
-  cl.sync();
+  ClusterOps<R> ops{cl, sh.sums, R(), 0u};
+  constexpr int wpb = TPB / 32;
+  const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
+  const int gw = rank * wpb + (int)(threadIdx.x >> 5), nw = C * wpb, lane = (int)(threadIdx.x & 31);
+  const bool leader = rank == 0 && threadIdx.x == 0;
+  if (a.amg_mixed) {
+    const AmgCtx<float> ctx =
+        solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.aval32, C, gw, nw, lane, false);
+    amg_mixed_solve(a, ctx, ops, gw, nw, lane, leader);
+  } else if (a.amg32) {
+    const AmgCtx<float> ctx =
+        solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.A.aval, C, gw, nw, lane, true);
+    amg_cg_solve<float>(a, ctx, a.z, ops, gw, nw, lane, leader);
+  } else {
+    const AmgCtx<double> ctx =
+        solve_begin<double>(sh.solve, ops.ring, ring_mem, a, a.amg, a.A.aval, C, gw, nw, lane, true);
+    amg_cg_solve<double>(a, ctx, a.z, ops, gw, nw, lane, leader);
+  }
+  ops.ring.finish(lane);
+  if (sh.solve.bad && lane == 0) atomicCAS(&a.sc->status, AVIP_OK, AVIP_ETIMEOUT);  // (a copy never arrived)
+  cl.sync();  // the next instance reuses the shared memory
 }
 
 // Batched, persistent: every resident cluster solves instances order[c], order[c + nclusters],
@@ -604,8 +614,11 @@ __global__ void __launch_bounds__(kClusterTPB, 1) pcg_cluster_batch_kernel(const
                                                                             const ClusterLayout* __restrict__ lays,
                                                                             const int32_t* __restrict__ order,
                                                                             int count) {
-  __shared__ ClusterShared sh;
-  __shared__ double s_amg_part[2 * 4], s_amg_wsum[32 * 4 + 4];
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ union {  // one instance at a time
+    ClusterShared jacobi;
+    ClusterAmgShared amg;
+  } sh;
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks();
   const int cid = blockIdx.x / C, ncl = gridDim.x / C;
@@ -613,14 +626,12 @@ __global__ void __launch_bounds__(kClusterTPB, 1) pcg_cluster_batch_kernel(const
     const int k = order[j];
     const PcgArgs a = args[k];
     const ClusterLayout L = lays[k];
-    if ((a.amg || a.amg32) && !a.amg_mixed)
-      cluster_amg_solve(a, s_amg_part, s_amg_wsum);
-    else if (a.amg32)
-      cluster_amg_mixed_solve(a, s_amg_part, s_amg_wsum);
+    if (a.amg || a.amg32)
+      cluster_amg_solve<kClusterTPB>(a, sh.amg, ring_mem);
     else if (L.mixed)
-      cluster_solve_mixed(a, L, sh);
+      cluster_solve_mixed(a, L, sh.jacobi);
     else
-      cluster_solve(a, L, sh);
+      cluster_solve(a, L, sh.jacobi);
   }
 }
 
@@ -768,17 +779,14 @@ cudaError_t launch_pcg_cluster(const PcgArgs& args, const PcgPlan& pl, const Clu
 // 16-CTA cluster: 150k nodes 218 -> 185 us per CG iteration, mixed 188 -> 155; 4k nodes 26.3 ->
 // 28.5, so small meshes keep 512).
 constexpr int kAmgClusterWideRows = 20000;
-template <int TPB, class Ops>
+template <int TPB>
 __global__ void __launch_bounds__(TPB, 1) pcg_amg_cluster_kernel(PcgArgs a) {
-  __shared__ double s_amg_part[2 * 4], s_amg_wsum[32 * 4 + 4];
-  if (a.amg_mixed)
-    cluster_amg_mixed_solve<Ops>(a, s_amg_part, s_amg_wsum);
-  else
-    cluster_amg_solve<Ops>(a, s_amg_part, s_amg_wsum);
+  extern __shared__ __align__(128) char ring_mem[];
+  __shared__ ClusterAmgShared sh;
+  cluster_amg_solve<TPB>(a, sh, ring_mem);
 }
 static const void* amg_cluster_kernel_ptr(int tpb) {
-  return tpb == 768 ? (const void*)pcg_amg_cluster_kernel<768, ClusterOpsT<6, 4>>
-                    : (const void*)pcg_amg_cluster_kernel<kClusterTPB, ClusterOps>;
+  return tpb == 768 ? (const void*)pcg_amg_cluster_kernel<768> : (const void*)pcg_amg_cluster_kernel<kClusterTPB>;
 }
 
 // Cluster of the standalone AMG cluster kernel for a mesh of n rows: `want` CTAs (2, 4, 8 or
@@ -790,11 +798,13 @@ PcgPlan amg_cluster_plan(int want, int n) {
   const int tpb = n > kAmgClusterWideRows ? 768 : kClusterTPB;
   const void* fn = amg_cluster_kernel_ptr(tpb);
   cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterRingBytes);
   for (int c : {want, 16, 8}) {
     if (c <= 0) continue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
     cfg.blockDim = dim3(tpb);
+    cfg.dynamicSmemBytes = kClusterRingBytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = c;
@@ -807,7 +817,7 @@ PcgPlan amg_cluster_plan(int want, int n) {
       pl.kind = 11;
       pl.tpb = tpb;
       pl.blocks = c;
-      pl.maxs = 0;
+      pl.maxs = (int)kClusterRingBytes;
       return pl;
     }
     cudaGetLastError();
@@ -819,6 +829,7 @@ cudaError_t launch_pcg_amg_cluster(const PcgArgs& args, const PcgPlan& pl, cudaS
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
   cfg.blockDim = dim3(pl.tpb);
+  cfg.dynamicSmemBytes = kClusterRingBytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -830,6 +841,9 @@ cudaError_t launch_pcg_amg_cluster(const PcgArgs& args, const PcgPlan& pl, cudaS
   void* kargs[] = {const_cast<PcgArgs*>(&args)};
   return cudaLaunchKernelExC(&cfg, amg_cluster_kernel_ptr(pl.tpb), kargs);
 }
+
+// Dynamic shared memory of a batch with AMG instances.
+size_t cluster_ring_bytes() { return kClusterRingBytes; }
 
 // Clusters of size C that can be resident at once with `smem` bytes per CTA.
 int cluster_batch_capacity(int C, size_t smem) {
