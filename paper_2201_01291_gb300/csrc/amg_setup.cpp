@@ -424,17 +424,18 @@ void sell_from_csr(const Csr& A, SellHost& S, int lpr) {
   }
 }
 
-int lanes_per_row(const Csr& A) {
+int lanes_per_row(const Csr& A, bool mixed) {
   const double avg = A.n > 0 ? (double)A.rp[A.n] / A.n : 0.0;
   int lpr = 1;
-  while (lpr < kSlice && avg > 8.0 * lpr && (int64_t)A.n * lpr < (int64_t)kManySlices * kSlice) lpr *= 2;
+  while (lpr < kSlice && avg > 8.0 * lpr && (mixed || (int64_t)A.n * lpr < (int64_t)kManySlices * kSlice))
+    lpr *= 2;
   return lpr;
 }
 
-int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
+int amg_setup(const HostMesh& m, bool mixed, AmgHost& H, char* err, size_t errlen) {
   // the axisymmetric matrix is not symmetric: no symmetrisation, LU instead of Cholesky
   const bool symmetric = m.geometry != AVIP_GEOM_AXISYMMETRIC;
-  const int32_t coarse_max = m.N <= kDirectRows ? m.N : std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
+  const int32_t coarse_max = !mixed && m.N <= kDirectRows ? m.N : std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
   auto fail = [&](const char* msg) {
     if (err && errlen) std::snprintf(err, errlen, "%s", msg);
     return AVIP_EINVAL;

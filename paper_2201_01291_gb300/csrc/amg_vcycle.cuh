@@ -84,10 +84,12 @@ __device__ __forceinline__ int dense_choice(const AmgDevT<T>& H, int nctas) {
 // and the calling warp's ring started at the matrix phase (the solve begins with a true residual)
 // or at the finest down phase.  TA: type of the streamed matrix values.  Every thread of the
 // participating blocks calls it.
+// keep: the dense operator is the coarsest inverse whatever the number of CTAs (the mixed-precision
+// solves' arithmetic, see block_group_sum).
 template <typename T, typename TA, class R>
 __device__ AmgCtx<T> solve_begin(SolveShared& sh, R& ring, char* dyn, const PcgArgs& a,
                                  const AmgDevT<T>* __restrict__ Hg, const TA* aval, int nctas, int gwarp, int nwarps,
-                                 int lane, bool matrix_first) {
+                                 int lane, bool matrix_first, bool keep = false) {
   static_assert(sizeof(AmgDevT<T>) == sizeof(AmgDevT<double>), "one shared copy for both types");
   const unsigned long long* src = reinterpret_cast<const unsigned long long*>(Hg);
   for (int k = threadIdx.x; k < (int)(sizeof(AmgDevT<T>) / 8); k += blockDim.x) sh.H[k] = src[k];
@@ -100,7 +102,7 @@ __device__ AmgCtx<T> solve_begin(SolveShared& sh, R& ring, char* dyn, const PcgA
   C.gain = sh.gain;
   C.rhs = reinterpret_cast<T*>(dyn + (blockDim.x >> 5) * R::kWarpBytes);
   C.H = reinterpret_cast<const AmgDevT<T>*>(sh.H);
-  C.D = C.H->dense[dense_choice(*C.H, nctas)];
+  C.D = C.H->dense[keep ? 1 : dense_choice(*C.H, nctas)];
   const int dl = C.D.level, p = (int)threadIdx.x;
   if (p <= 2 * dl + 1) {
     PhaseDesc d;
@@ -510,13 +512,16 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgCtx<T>& C, double* __res
 
 
 // Mixed-precision solve with the FP32 hierarchy (kind 10 and the batched mixed form): FP64
-// outer residual and correction, FP32 inner CG preconditioned by the FP32 V-cycle.
+// outer residual and correction, FP32 inner CG preconditioned by the FP32 V-cycle.  As in
+// amg_cg_solve the update r - alpha q, e += alpha p of an iteration is folded into the finest down
+// phase of the next.
 template <class Ops>
 __device__ bool amg_mixed_solve(const PcgArgs& a, const AmgCtx<float>& C, Ops& ops, int gwarp, int nwarps, int lane,
                                 bool leader) {
-  const int N = a.A.N, nsl = a.A.nslices;
+  const int N = a.A.N, nsl = a.A.nslices, dl = C.D.level;
   const double* nb = a.nbuf + (size_t)a.sc->parity * AVIP_MAX_SPECIES * a.Npad;
-  float* __restrict__ r32 = a.r32;
+  float* rc = a.r32;   // current inner residual
+  float* rn = a.rq32;  // the other buffer
   float* __restrict__ e32 = a.e32;
   float* __restrict__ p32 = a.p32;
   float* __restrict__ q32 = a.q32;
@@ -524,7 +529,7 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, const AmgCtx<float>& C, Ops& o
 
   const double gain = C.gain;
   const int hist = history_length(a);
-  double bb[1] = {0.0};
+  double bb = 0.0;
   for (int s = gwarp; s < nsl; s += nwarps) {
     const int i = s * kSlice + lane;
     if (i >= N) continue;
@@ -541,156 +546,232 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, const AmgCtx<float>& C, Ops& o
     } else {
       b = a.b[i];
     }
-    if (a.rhs_scale[i] != 0.0) bb[0] = fma(b, b, bb[0]);  // free rows only: a Dirichlet row holds its value exactly
+    if (a.rhs_scale[i] != 0.0) bb = fma(b, b, bb);  // free rows only: a Dirichlet row holds its value exactly
     else a.x[i] = b;  // a Dirichlet unit row takes its (possibly ramped) value exactly
   }
-  if (!ops.sum(bb)) return false;
+  double bs[2];  // b.b and the stopping threshold on r.r
+  bool zero;
   {
-    const double thresh = a.rtol * a.rtol * bb[0];
-    int it = 0, outer = 0, status = AVIP_OK;
-    double rr64 = 0.0;
-    while (true) {
-      // ---- FP64 residual of the FP64 iterate (x complete)
-      double r2[1] = {0.0};
-      for (int s = gwarp; s < nsl; s += nwarps) {
-        const int i = s * kSlice + lane;
-        if (i >= N) continue;
-        const double r = a.b[i] - sell_row_dot(a.A, s, lane, i, a.x);
-        a.r[i] = r;
-        r2[0] = fma(r, r, r2[0]);
-      }
-      double rs[3];  // r.r, its root and 1 / root
-      bool small;
-      if (!ops.template sum_epi<3>(r2[0], rs, small, [thresh](double t, double* o) {
-            o[0] = t;
-            o[1] = sqrt(t);
-            o[2] = 1.0 / o[1];
-            return t <= thresh;
-          }))
-        return false;
-      rr64 = rs[0];
-      if (!isfinite(rr64)) {
-        status = AVIP_ENAN;
-        break;
-      }
-      if (small || bb[0] == 0.0) break;
-      if (it >= a.max_iter) {
-        status = AVIP_ENOTCONV;
-        break;
-      }
-      ++outer;
-      const int it_outer = it;
-      const double rnorm = rs[1], rscale = rs[2];
-      // ---- FP32 right-hand side r / ||r||, e = 0
-      double g0[1];
-      {
-        DotAcc<float> k;
-        for (int s = gwarp; s < nsl; s += nwarps) {
-          const int i = s * kSlice + lane;
-          if (i >= N) continue;
-          const float r = (float)(a.r[i] * rscale);
-          r32[i] = r;
-          e32[i] = 0.f;
-          k.add(r, r);
-        }
-        g0[0] = k.value();
-      }
-      if (!ops.sum(g0)) return false;
-      const double inner_thresh = a.inner_rtol * a.inner_rtol * g0[0];
-      double rz = 0.0;
-      bool fresh = true, go_on = g0[0] > inner_thresh;
-      while (go_on && it < a.max_iter) {
-        double rzb[2];  // r.z, beta
-        bool positive;
-        const double rz_old = rz;
-        const bool first = fresh;
-        if (!vcycle(C, (const float*)r32, z32, ops, gwarp, nwarps, lane, rzb, positive,
-                    [rz_old, first](double t, double* o) {
-                      o[0] = t;
-                      o[1] = first ? 0.0 : t / rz_old;
-                      return t > 0.0 && isfinite(t);
-                    }))
-          return false;
-        if (!positive) break;  // refine with what the inner solve has
-        const float beta = (float)rzb[1];
-        rz = rzb[0];
-        fresh = false;
-        DotAcc<float> kpq;
-        struct PreA {
-          float z, q, p;
-        };
-        stream_rows<float, float>(
-            ops.ring, C.mat_phase(), lane, [z32](int c) { return __ldca(z32 + c); },
-            [=](int i) { return PreA{__ldca(z32 + i), q32[i], p32[i]}; },
-            [&](int i, float w, const PreA& o) {
-              const float qn = first ? w : fmaf(beta, o.q, w);  // (restart: old p, q unused)
-              const float pn = first ? o.z : fmaf(beta, o.p, o.z);
-              q32[i] = qn;
-              p32[i] = pn;
-              kpq.add(pn, qn);
-            });
-        double al[1];
-        bool more;
-        const double rz_now = rz;
-        if (!ops.template sum_epi<1>(kpq.value(), al, more, [rz_now](double t, double* o) {
-              o[0] = rz_now / t;
-              return false;
-            }))
-          return false;
-        const float alpha = (float)al[0];
-        DotAcc<float> krr;
-        for (int s = gwarp; s < nsl; s += nwarps) {
-          const int i = s * kSlice + lane;
-          if (i >= N) continue;
-          e32[i] = fmaf(alpha, p32[i], e32[i]);
-          const float r = fmaf(-alpha, q32[i], r32[i]);
-          r32[i] = r;
-          krr.add(r, r);
-        }
-        if (!ops.template sum_epi<1>(krr.value(), al, more, [inner_thresh](double t, double* o) {
-              o[0] = t;
-              return t > inner_thresh;
-            }))
-          return false;
-        go_on = more;
-        ++it;
-      }
-      if (it == it_outer) {  // the inner solve could not start: no progress is possible
-        status = AVIP_ENOTCONV;
-        break;
-      }
-      // ---- FP64 correction x += ||r|| e
-      for (int s = gwarp; s < nsl; s += nwarps) {
-        const int i = s * kSlice + lane;
-        if (i >= N) continue;
-        a.x[i] = fma(rnorm, (double)e32[i], a.x[i]);
-      }
-      double z0[1] = {0.0};
-      if (!ops.sum(z0)) return false;  // x complete before the next residual
-    }
+    const double rtol = a.rtol;
+    if (!ops.template sum_epi<2>(bb, bs, zero, [rtol](double t, double* o) {
+          o[0] = t;
+          o[1] = rtol * rtol * t;
+          return t == 0.0;
+        }))
+      return false;
+  }
+  const double thresh = bs[1];
+  int it = 0, outer = 0, status = AVIP_OK;
+  double rr64 = 0.0;
+  while (true) {
+    // ---- FP64 residual of the FP64 iterate (x complete)
+    double r2 = 0.0;
     for (int s = gwarp; s < nsl; s += nwarps) {
       const int i = s * kSlice + lane;
-      if (i < N) a.phi[i] = a.dsqinv[i] * (bb[0] == 0.0 ? a.b[i] : a.x[i]);  // free b == 0: x = b
+      if (i >= N) continue;
+      const double r = a.b[i] - sell_row_dot(a.A, s, lane, i, a.x);
+      a.r[i] = r;
+      r2 = fma(r, r, r2);
     }
-    if (leader) {
-      a.res->pcg_iters = it;
-      advance_history(a);
-      a.res->pcg_outer = outer;
-      a.res->pcg_status = status;
-      a.res->pcg_relres = bb[0] > 0.0 ? sqrt(rr64 / bb[0]) : 0.0;
-      a.res->pcg_bnorm = sqrt(bb[0]);
-      if (status != AVIP_OK && a.sc->status == AVIP_OK) a.sc->status = status;
+    double rs[3];  // r.r, its root and 1 / root
+    bool small;
+    if (!ops.template sum_epi<3>(r2, rs, small, [thresh](double t, double* o) {
+          o[0] = t;
+          o[1] = sqrt(t);
+          o[2] = 1.0 / o[1];
+          return t <= thresh;
+        }))
+      return false;
+    rr64 = rs[0];
+    if (!isfinite(rr64)) {
+      status = AVIP_ENAN;
+      break;
     }
-    return true;
+    if (small || zero) break;
+    if (it >= a.max_iter) {
+      status = AVIP_ENOTCONV;
+      break;
+    }
+    ++outer;
+    const int it_outer = it;
+    const double rnorm = rs[1], rscale = rs[2];
+    // ---- FP32 right-hand side r / ||r||, e = 0
+    double g0[2];  // its square norm, the inner stopping threshold
+    bool go;
+    {
+      DotAcc<float> k;
+      for (int s = gwarp; s < nsl; s += nwarps) {
+        const int i = s * kSlice + lane;
+        if (i >= N) continue;
+        const float r = (float)(a.r[i] * rscale);
+        rc[i] = r;
+        e32[i] = 0.f;
+        k.add(r, r);
+      }
+      const double in_rtol = a.inner_rtol;
+      if (!ops.template sum_epi<2>(k.value(), g0, go, [in_rtol](double t, double* o) {
+            o[0] = t;
+            o[1] = in_rtol * in_rtol * t;
+            return t > o[1];
+          }))
+        return false;
+    }
+    const double inner_thresh = g0[1];
+    double rz = 0.0;
+    float alpha = 0.f;
+    bool fresh = true;
+    while (go) {
+      // ---- finest down phase on the residual, updated by the last step unless fresh
+      {
+        const float* __restrict__ rv = rc;
+        const float al = alpha;
+        const bool upd = !fresh;
+        auto res = [rv, q32, al, upd](int c) {
+          return upd ? fmaf(-al, __ldca(q32 + c), __ldca(rv + c)) : __ldca(rv + c);
+        };
+        DotAcc<float> krr;
+        struct Pre {
+          float r, q, e, p;
+        };
+        struct Hook {
+          const float *rv, *qv, *pv;
+          float *ev, *rnv;
+          DotAcc<float>* krr;
+          float al;
+          bool upd;
+          __device__ Pre begin(int i) const {
+            if (!upd) return Pre{0.f, 0.f, 0.f, 0.f};
+            return Pre{__ldca(rv + i), __ldca(qv + i), ev[i], pv[i]};
+          }
+          __device__ void end(int i, const Pre& p) const {
+            if (!upd) return;
+            const float v = fmaf(-al, p.q, p.r);
+            rnv[i] = v;
+            ev[i] = fmaf(al, p.p, p.e);
+            krr->add(v, v);
+          }
+        } hook{rv, q32, p32, e32, rn, &krr, al, upd};
+        if (dl == 0) {
+          for (int s = gwarp; s < nsl; s += nwarps) {
+            const int i = s * kSlice + lane;
+            if (i < N) hook.end(i, hook.begin(i));
+          }
+        } else {
+          amg_down(C, ops, 0, res, hook, gwarp, nwarps, lane);
+        }
+        if (upd) {
+          double none[1];
+          bool done;
+          if (!ops.template sum_epi<1>(krr.value(), none, done, [inner_thresh](double t, double* o) {
+                o[0] = t;
+                return !(t > inner_thresh);
+              }))
+            return false;
+          ++it;
+          float* t = rc;
+          rc = rn;
+          rn = t;
+          if (done || it >= a.max_iter) break;
+        } else if (!ops.barrier()) {
+          return false;
+        }
+      }
+      // ---- the levels below, then the finest up phase: z = U0 xp0 + Pf0 x1, r.z
+      double rzb[2];  // r.z, beta
+      bool positive;
+      {
+        DotAcc<double> acc;
+        struct Out {
+          const float* rv;
+          float* z;
+          DotAcc<double>* acc;
+          __device__ float begin(int i) const { return __ldca(rv + i); }
+          __device__ void end(int i, float v, float ri) const {
+            z[i] = v;
+            acc->add((double)ri, (double)v);
+          }
+        } out{rc, z32, &acc};
+        if (dl == 0) {
+          const float* __restrict__ rv = rc;
+          amg_dense(C, ops, [rv](int k) { return __ldca(rv + k); },
+                    [&](int row, float v) { out.end(row, v, out.begin(row)); }, lane);
+        } else {
+          if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
+          amg_up(C, ops, 0, out, lane);
+        }
+        const double rz_old = rz;
+        const bool first = fresh;
+        if (!ops.template sum_epi<2>(acc.value(), rzb, positive, [rz_old, first](double t, double* o) {
+              o[0] = t;
+              o[1] = first ? 0.0 : t / rz_old;
+              return t > 0.0 && isfinite(t);
+            }))
+          return false;
+      }
+      if (!positive) break;  // refine with what the inner solve has
+      const float beta = (float)rzb[1];
+      const bool first = fresh;
+      rz = rzb[0];
+      fresh = false;
+      // ---- w = A z, q = w + beta q, p = z + beta p, p.q -> alpha
+      DotAcc<float> kpq;
+      struct PreA {
+        float z, q, p;
+      };
+      stream_rows<float, float>(
+          ops.ring, C.mat_phase(), lane, [z32](int c) { return __ldca(z32 + c); },
+          [=](int i) { return PreA{__ldca(z32 + i), q32[i], p32[i]}; },
+          [&](int i, float w, const PreA& o) {
+            const float qn = first ? w : fmaf(beta, o.q, w);  // (restart: old p, q unused)
+            const float pn = first ? o.z : fmaf(beta, o.p, o.z);
+            q32[i] = qn;
+            p32[i] = pn;
+            kpq.add(pn, qn);
+          });
+      double al[1];
+      bool unused;
+      const double rz_now = rz;
+      if (!ops.template sum_epi<1>(kpq.value(), al, unused, [rz_now](double t, double* o) {
+            o[0] = rz_now / t;
+            return false;
+          }))
+        return false;
+      alpha = (float)al[0];
+    }
+    if (it == it_outer) {  // the inner solve could not start: no progress is possible
+      status = AVIP_ENOTCONV;
+      break;
+    }
+    // ---- FP64 correction x += ||r|| e
+    for (int s = gwarp; s < nsl; s += nwarps) {
+      const int i = s * kSlice + lane;
+      if (i >= N) continue;
+      a.x[i] = fma(rnorm, (double)e32[i], a.x[i]);
+    }
+    if (!ops.barrier()) return false;  // x complete before the next residual
   }
+  for (int s = gwarp; s < nsl; s += nwarps) {
+    const int i = s * kSlice + lane;
+    if (i < N) a.phi[i] = a.dsqinv[i] * (zero ? a.b[i] : a.x[i]);  // free b == 0: x = b
+  }
+  if (leader) {
+    a.res->pcg_iters = it;
+    advance_history(a);
+    a.res->pcg_outer = outer;
+    a.res->pcg_status = status;
+    a.res->pcg_relres = bs[0] > 0.0 ? sqrt(rr64 / bs[0]) : 0.0;
+    a.res->pcg_bnorm = sqrt(bs[0]);
+    if (status != AVIP_OK && a.sc->status == AVIP_OK) a.sc->status = status;
+  }
+  return true;
 }
 
 
 // Grid-wide synchronisation of a cooperative launch (counter barrier of grid_sync.cuh); MAXV: most
-// values of one sum.  sum_epi evaluates `epi(total, out)` on one thread per block: a division or
+// values of one sum; kKeep: sums in the order the mixed-precision solves keep (block_group_sum).  sum_epi evaluates `epi(total, out)` on one thread per block: a division or
 // comparison that every thread repeats costs a 1024-thread block 600 cycles per FP64 instruction
 // (a division 5,000), one thread 64.  It returns a flag, and up to three derived scalars in out.
-template <class R, int MAXV>
+template <class R, int MAXV, bool kKeep = false>
 struct GridOps {
   FlagSync& fs;
   R ring;
@@ -698,7 +779,7 @@ struct GridOps {
   template <int NE, class Epi>
   __device__ bool sum_epi(double v, double (&out)[NE], bool& flag, Epi epi) {
     double s[1] = {v}, e[NE + 1];
-    if (!grid_allsum<1, NE + 1, MAXV>(s, e, fs, nullptr,
+    if (!grid_allsum<1, NE + 1, MAXV, kKeep>(s, e, fs, nullptr,
                                       [&epi](const double* t, double* o) { o[NE] = epi(t[0], o) ? 1.0 : 0.0; }))
       return false;
 #pragma unroll
@@ -708,7 +789,7 @@ struct GridOps {
   }
   __device__ bool sum(double (&v)[1]) {
     double e[1];
-    return grid_allsum<1, 0, MAXV>(v, e, fs, nullptr, NoEpilogue());
+    return grid_allsum<1, 0, MAXV, kKeep>(v, e, fs, nullptr, NoEpilogue());
   }
 };
 
@@ -724,7 +805,7 @@ struct ClusterSums {
   double res[4];
   int flag;
 };
-template <class R>
+template <class R, bool kKeep = false>
 struct ClusterOps {
   cooperative_groups::cluster_group cl;
   ClusterSums& sh;
@@ -749,7 +830,20 @@ struct ClusterOps {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = (int)cl.num_blocks();
     double* part = sh.part[seq++ & 1];
     double s[1] = {v}, bt[1];
-    block_group_sum<1>(s, bt, sh.thr, sh.grp);
+    if constexpr (kKeep) {
+      // the mixed-precision solves' order (see block_group_sum): a tree in every warp, then the
+      // warps in turn
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+      if (lane == 0) sh.thr[warp] = s[0];
+      __syncthreads();
+      if (warp == 0) {
+        bt[0] = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) bt[0] += sh.thr[w];
+      }
+    } else {
+      block_group_sum<1>(s, bt, sh.thr, sh.grp);
+    }
     if (warp == 0 && lane < C) *cl.map_shared_rank(part + cl.block_rank(), lane) = bt[0];
     cluster_sync();
     if (warp == 0) {

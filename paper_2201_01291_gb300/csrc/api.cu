@@ -121,6 +121,7 @@ struct avip_mesh {
 namespace {
 
 thread_local char g_err[256];
+constexpr int kClusterMixedMinRows = 500;  // mixed precision: Jacobi-PCG on one cluster up to this size (kind 6)
 constexpr int kClusterAutoRows = 20000;  // one-cluster solvers up to this many nodes
 
 void* dev_alloc(avip_mesh* h, size_t bytes) {
@@ -444,7 +445,7 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
   D.nlev = (int32_t)H.lv.size();
   auto put = [&](const Csr& M, SellMatT<T>& dst) {
     SellHost S;
-    sell_from_csr(M, S, lanes_per_row(M));
+    sell_from_csr(M, S, lanes_per_row(M, h->opts.precision == AVIP_PREC_MIXED));
     int32_t *slp = nullptr, *col = nullptr;
     T* val = nullptr;
     std::vector<T> v(S.val.begin(), S.val.end());
@@ -668,7 +669,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // or three iterations replace the 70 to 90 of the Jacobi form.
   PcgPlan amg_cluster;
   amg_cluster.kind = 0;
-  if (!bicg && (h->opts.pcg_kind == 11 || (h->opts.pcg_kind == 0 && m.N <= kClusterAutoRows)))
+  if (!bicg && (h->opts.pcg_kind == 11 || (h->opts.pcg_kind == 0 && m.N <= kClusterAutoRows &&
+                 !(h->opts.precision == AVIP_PREC_MIXED && m.N <= kClusterMixedMinRows))))
     amg_cluster = amg_cluster_plan(h->opts.cluster_size, m.N);
   // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above the cluster size
   const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (h->opts.pcg_kind == 0 && m.N > kClusterAutoRows));
@@ -696,7 +698,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
                    (h->opts.pcg_kind == 8 ||
                     (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
     AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -725,7 +727,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
       (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
     AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -737,7 +739,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   }
   if (amg_cluster.kind == 11) {
     AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -972,7 +974,7 @@ int photo_set(avip_mesh_t h, int32_t n_terms, const double* a, const double* kap
       hm.aval = std::move(val);
       hm.dsq.assign(dh.begin(), dh.begin() + m.N);
       AmgHost H;
-      if (amg_setup(hm, H, g_err, sizeof(g_err)) != AVIP_OK) return AVIP_EINVAL;
+      if (amg_setup(hm, false, H, g_err, sizeof(g_err)) != AVIP_OK) return AVIP_EINVAL;
       if (h->amg)
         ok = upload_amg_t<double>(h, H, t.amg, false);
       else

@@ -95,8 +95,9 @@ struct AmgHost {
 // four phases of 2 us and more for the levels it replaces.
 constexpr int kAmgDenseRows = 1536;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
-// composite operators of every non-coarsest level.
-int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen);
+// composite operators of every non-coarsest level.  mixed: for a mixed-precision handle, whose
+// solves keep one arithmetic (block_group_sum in grid_sync.cuh): no direct inverse of small meshes.
+int amg_setup(const HostMesh& m, bool mixed, AmgHost& out, char* err, size_t errlen);
 
 // SELL-32 form of a CSR matrix with `lpr` lanes per row (1, 2, 4, 8, 16 or 32): a slice holds
 // 32 / lpr consecutive rows; step k of a slice is 32 contiguous elements, entries k*lpr ..
@@ -115,7 +116,8 @@ void sell_from_csr(const Csr& A, SellHost& out, int lpr = 1);
 // at most 8 stored entries per lane on an average row, or fewer lanes when that gives a slice to
 // every warp of the whole-GPU solvers already (a row's epilogue runs on one of its lanes only, and
 // the finest level's has FP64 operations).
-int lanes_per_row(const Csr& A);
+// `mixed` (see amg_setup): always the former.
+int lanes_per_row(const Csr& A, bool mixed);
 // Elements a streamed array must be readable past its end (a ring slot is always filled).
 constexpr size_t kStreamPad = 16 * kSlice;
 

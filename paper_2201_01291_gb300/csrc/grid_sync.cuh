@@ -129,13 +129,18 @@ __device__ __forceinline__ AllsumScratch<MAXV>& allsum_scratch() {
 // not (one per ~19 cycles and SM; latency 64), so a single warp adding 32 values per lane takes
 // 2,200 cycles.  Every thread stores its values, four warps per value (one per sub-partition) add
 // a quarter of them each and finish with a shuffle tree, and warp 0 adds the four group sums.
-template <int NV>
+//
+// kOneGroup keeps the order of a single adding warp.  The mixed-precision solves take it: their FP32
+// inner solves and the FP32 drift-diffusion stage turn a last-bit difference of one of these sums
+// into differences of 1e-9 of the densities within ten steps, so that mixed-precision results are
+// kept bit for bit when a kernel is reworked; it costs them 1,200 cycles per sum.
+template <int NV, bool kOneGroup = false>
 __device__ __forceinline__ void block_group_sum(const double (&v)[NV], double (&bt)[NV], double* thr, double* grp) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) thr[k * 1024 + threadIdx.x] = v[k];
   __syncthreads();
-  const int G = nw >= 4 * NV ? 4 : 1;  // groups per value
+  const int G = !kOneGroup && nw >= 4 * NV ? 4 : 1;  // groups per value
   if (warp < G * NV) {
     const int k = warp / G, j = warp % G;
     double t = 0.0;
@@ -174,7 +179,7 @@ __device__ __forceinline__ void red_add_release_u32(unsigned* p, unsigned v) {
 // warp 0 waits (acquire) until the counter reaches seq * nb and then reads all partials in
 // block order.  Partials are double-buffered by the parity of seq because a fast
 // block may publish reduction k+1 while a slow one is still reading reduction k.
-template <int NV, int NE, int MAXV = 4, typename Epi>
+template <int NV, int NE, int MAXV = 4, bool kOneGroup = false, typename Epi>
 __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 0 ? NE : 1], FlagSync& fs,
                                             double* smem, Epi epi) {
   static_assert(NV <= MAXV && MAXV <= 4 && NE <= 4, "grid_allsum: at most 4 sums and 4 derived scalars");
@@ -187,7 +192,7 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 
   int& s_ok = scr.ok;
   (void)smem;
   double bt[NV];
-  block_group_sum<NV>(v, bt, scr.thr, scr.grp);
+  block_group_sum<NV, kOneGroup>(v, bt, scr.thr, scr.grp);
   if (warp == 0) {
     int ok = 1;
     if (nb > 1) {

@@ -376,10 +376,10 @@ __global__ void __launch_bounds__(TPB, 1) pcg_amg_mixed_kernel(PcgArgs a) {
   constexpr int wpb = TPB / 32;
   using R = Ring<ring_slots(TPB, false)>;
   FlagSync fs{a.flags, a.parts, a.sync, 0u, a.spin_ns, (int)gridDim.x, (int)blockIdx.x, &sh.bad};
-  GridOps<R, 1> ops{fs, R()};
+  GridOps<R, 1, true> ops{fs, R()};
   const int gwarp = blockIdx.x * wpb + (threadIdx.x >> 5), nwarps = gridDim.x * wpb, lane = threadIdx.x & 31;
-  const AmgCtx<float> C =
-      solve_begin<float>(sh, ops.ring, ring_mem, a, a.amg32, a.aval32, (int)gridDim.x, gwarp, nwarps, lane, false);
+  const AmgCtx<float> C = solve_begin<float>(sh, ops.ring, ring_mem, a, a.amg32, a.aval32, (int)gridDim.x, gwarp,
+                                             nwarps, lane, false, true);
   const bool ok = amg_mixed_solve(a, C, ops, gwarp, nwarps, lane, blockIdx.x == 0 && threadIdx.x == 0);
   ops.ring.finish(lane);
   if (!ok && threadIdx.x == 0) report_timeout(a);
@@ -442,7 +442,9 @@ PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64) {
   const size_t smem = ring_bytes(pl.tpb, kind == 9);
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, pl.tpb, smem);
-  const int want = (nslices + kSlicesPerBlock - 1) / kSlicesPerBlock;
+  // (the mixed-precision form keeps the partition of its FP32 sums: a slice per warp)
+  const int per_block = kind == 10 ? pl.tpb / kSlice : kSlicesPerBlock;
+  const int want = (nslices + per_block - 1) / per_block;
   pl.blocks = std::max(1, std::min(std::max(occ, 1) * std::max(sms, 1), want));
   return pl;
 }

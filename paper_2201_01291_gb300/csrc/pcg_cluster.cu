@@ -583,25 +583,29 @@ __device__ void cluster_amg_solve(const PcgArgs& a, ClusterAmgShared& sh, char* 
   if (solve_skipped(a.sc)) return;  // every CTA of the cluster reads the same status
   using R = ClusterRing<TPB>;
   cg::cluster_group cl = cg::this_cluster();
-  ClusterOps<R> ops{cl, sh.sums, R(), 0u};
   constexpr int wpb = TPB / 32;
   const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
   const int gw = rank * wpb + (int)(threadIdx.x >> 5), nw = C * wpb, lane = (int)(threadIdx.x & 31);
   const bool leader = rank == 0 && threadIdx.x == 0;
   if (a.amg_mixed) {
+    ClusterOps<R, true> ops{cl, sh.sums, R(), 0u};
     const AmgCtx<float> ctx =
-        solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.aval32, C, gw, nw, lane, false);
+        solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.aval32, C, gw, nw, lane, false, true);
     amg_mixed_solve(a, ctx, ops, gw, nw, lane, leader);
+    ops.ring.finish(lane);
   } else if (a.amg32) {
+    ClusterOps<R> ops{cl, sh.sums, R(), 0u};
     const AmgCtx<float> ctx =
         solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.A.aval, C, gw, nw, lane, true);
     amg_cg_solve<float>(a, ctx, a.z, ops, gw, nw, lane, leader);
+    ops.ring.finish(lane);
   } else {
+    ClusterOps<R> ops{cl, sh.sums, R(), 0u};
     const AmgCtx<double> ctx =
         solve_begin<double>(sh.solve, ops.ring, ring_mem, a, a.amg, a.A.aval, C, gw, nw, lane, true);
     amg_cg_solve<double>(a, ctx, a.z, ops, gw, nw, lane, leader);
+    ops.ring.finish(lane);
   }
-  ops.ring.finish(lane);
   if (sh.solve.bad && lane == 0) atomicCAS(&a.sc->status, AVIP_OK, AVIP_ETIMEOUT);  // (a copy never arrived)
   cl.sync();  // the next instance reuses the shared memory
 }
