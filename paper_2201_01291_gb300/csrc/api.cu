@@ -60,6 +60,8 @@ struct avip_mesh {
   double *x = nullptr, *y = nullptr, *vol = nullptr, *dsq = nullptr, *dsqinv = nullptr, *lift = nullptr,
          *rhs_scale = nullptr;
   double* cw = nullptr;
+  float* cw32 = nullptr;
+  float4* vf = nullptr;
   int32_t *e_lo = nullptr, *e_hi = nullptr, *slot_eid = nullptr;  // edge list (flux once per edge)
   double *e_sx = nullptr, *e_sy = nullptr, *eflux = nullptr;
   double *phi1 = nullptr, *phi2 = nullptr, *phi3 = nullptr;  // the three previous potentials (predictor)
@@ -262,6 +264,8 @@ DDArgs dd_args(const avip_mesh* h) {
   a.photo_S = h->photo_S;
   a.cell = h->cell;
   a.cw = h->cw;
+  a.cw32 = h->cw32;
+  a.vf = h->vf;
   a.e_lo = h->e_lo;
   a.e_hi = h->e_hi;
   a.e_sx = h->e_sx;
@@ -640,7 +644,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   bool ok = upload(h, h->sl_ptr, m.sl_ptr) && upload(h, h->sl_w, m.sl_w) && upload(h, h->rlen, m.rlen) &&
             upload(h, h->col, m.col) && upload(h, h->aval, m.aval, m.aval.size() + kStreamPad) && upload(h, h->gx, m.gx) &&
             upload(h, h->gy, m.gy) && upload(h, h->sx, m.sx) && upload(h, h->sy, m.sy) &&
-            upload(h, h->cell, m.cell) && upload(h, h->flen, m.flen) && upload(h, h->cw, m.cw) && upload(h, h->e_lo, m.e_lo, 1) && upload(h, h->e_hi, m.e_hi, 1) &&
+            upload(h, h->cell, m.cell) && upload(h, h->flen, m.flen) && upload(h, h->cw, m.cw) && upload(h, h->cw32, std::vector<float>(m.cw.begin(), m.cw.end())) &&
+            zalloc(h, h->vf, (size_t)AVIP_MAX_SPECIES * Np) && upload(h, h->e_lo, m.e_lo, 1) && upload(h, h->e_hi, m.e_hi, 1) &&
             upload(h, h->e_sx, m.e_sx, 1) && upload(h, h->e_sy, m.e_sy, 1) && upload(h, h->slot_eid, m.slot_eid) &&
             zalloc(h, h->eflux, (size_t)AVIP_MAX_SPECIES * std::max<size_t>(m.e_lo.size(), 1)) && upload(h, h->x, m.x, Np) &&
             upload(h, h->y, m.y, Np) && upload(h, h->vol, m.vol, Np) && upload(h, h->ivol, inverse_volumes(m.vol), Np) && upload(h, h->dsq, m.dsq, Np) && upload(h, h->dsqinv, m.dsqinv, Np) &&
@@ -1292,6 +1297,7 @@ cudaError_t launch_dd_batch(const DDArgs* args, const int32_t* node_pref, const 
                             int node_blocks, int cell_blocks, int threads, cudaStream_t st);
 cudaError_t launch_run_reset_batch(const DDArgs* args, int count, cudaStream_t st);
 int dd_threads();
+int dt_cells_blocks(int cells, int threads);
 }  // namespace avip
 
 struct avip_batch {
@@ -1383,7 +1389,7 @@ bool batch_set_dd(avip_batch* b, int T) {
   std::vector<int32_t> npref(count + 1, 0), cpref(count + 1, 0);
   for (int k = 0; k < count; ++k) {
     npref[k + 1] = npref[k] + (b->m[k]->hm.N + T - 1) / T;
-    cpref[k + 1] = cpref[k] + (b->m[k]->hm.T + T - 1) / T;
+    cpref[k + 1] = cpref[k] + dt_cells_blocks(b->m[k]->hm.T, T);
   }
   if (cudaMemcpyAsync(b->d_npref, npref.data(), npref.size() * sizeof(int32_t), cudaMemcpyHostToDevice, b->stream) !=
           cudaSuccess ||

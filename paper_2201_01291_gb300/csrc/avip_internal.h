@@ -15,6 +15,8 @@
 #include <cstdint>
 #include <vector>
 
+#include <vector_types.h>
+
 #include "../../include/avip.h"
 
 namespace avip {
@@ -423,6 +425,8 @@ struct DDArgs {
   double* photo_S;        // per node: S_ph = sum_j S_ph,j
   const int32_t* cell;    // SoA v0[T], v1[T], v2[T] (, v3[T] when nvmax == 4; -1 for triangles)
   const double* cw;       // per cell 1 / (n_v dx_min)
+  const float* cw32;      // the same rounded to FP32 (screening of the time-step limits)
+  float4* vf;             // per species per node, FP32: vx, vy, n mu, 0 (screening)
   // edge fluxes computed once per edge (FP64 single-instance path; eflux == nullptr: each
   // row evaluates the fluxes of its edges itself)
   const int32_t* e_lo;

@@ -43,19 +43,25 @@ __device__ __forceinline__ double limiter(double r, double beta, int kind) {
   return fmax(0.0, fmax(fmin(beta * r, 1.0), fmin(r, beta)));
 }
 
+// Smallest positive v of the block into *dst (the bits of positive doubles order like integers):
+// two integer warp reductions, no FP64 comparison (each costs the SM 19 cycles per warp).
 __device__ __forceinline__ void block_min_to_global(double v, unsigned long long* dst) {
-  __shared__ double sm[32];
+  __shared__ unsigned long long sm[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (lane == 0) sm[warp] = v;
+  constexpr unsigned long long kInf = 0x7ff0000000000000ULL;
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long key = bits == 0 || bits > kInf ? kInf : bits;  // zero, negative, NaN: no candidate
+  auto warp_min = [](unsigned long long k) {
+    const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(k >> 32));
+    const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0xffffffffu);
+    return (unsigned long long)hi << 32 | lo;
+  };
+  const unsigned long long w = warp_min(key);
+  if (lane == 0) sm[warp] = w;
   __syncthreads();
   if (warp == 0) {
-    double t = lane < nw ? sm[lane] : INFINITY;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t = fmin(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if (lane == 0 && t < INFINITY && t > 0.0)
-      atomicMin(dst, (unsigned long long)__double_as_longlong(t));
+    const unsigned long long t = warp_min(lane < nw ? sm[lane] : kInf);
+    if (lane == 0 && t < kInf) atomicMin(dst, t);
   }
 }
 
@@ -133,7 +139,9 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
         double2* d = reinterpret_cast<double2*>(a.ndat + ((size_t)s * a.Npad + i) * 4);
         d[0] = make_double2(gnx[s], gny[s]);
         d[1] = make_double2(vx, vy);
-        a.nm[(size_t)s * a.Npad + i] = n[(size_t)s * a.Npad + i] * mu[s];
+        const double nmu = n[(size_t)s * a.Npad + i] * mu[s];
+        a.nm[(size_t)s * a.Npad + i] = nmu;
+        a.vf[(size_t)s * a.Npad + i] = make_float4((float)vx, (float)vy, (float)nmu, 0.f);
       }
     }
     double src[AVIP_MAX_SPECIES];
@@ -204,54 +212,135 @@ __global__ void __launch_bounds__(kDDThreads, 3) node_fields_kernel(DDArgs a, in
 // largest conductivity over its cells and species, and divides once at the end:
 // min_c cfl dx / |V| = cfl / max_c |V| / dx, likewise for the dielectric limit.  The Fourier
 // limit, fourier dx^2 / D over cells and species, depends on the mesh only (ph.dt_fourier).
-__device__ __forceinline__ void dt_cells_body(const DDArgs& a, int bid, int nblocks) {
-  // the largest (|V_cell| / dx)^2 is carried instead of |V_cell| / dx, so that each thread
-  // takes one square root at the end rather than one per cell and species (FP64 square roots
-  // dominated this kernel's FP64 issue)
-  double v2max = 0.0, smax = 0.0;
+//
+// The two maxima are screened in FP32: every cell's |V_cell| / dx and conductivity get a lower and an
+// upper bound from FP32 copies of the nodal values (a.vf, written by the nodal kernel: vx, vy,
+// n mu) and a bound of the FP32 rounding, and only the cells whose upper bound reaches the
+// block's largest lower bound, in blocks that can still lower the global minimum, are evaluated
+// in FP64.  The cell that sets the time step always is, so the result is the FP64 one bit for
+// bit.  On GB300 the FP64 pipe bounded this kernel (16 operations per cell and species; 997,002
+// triangles, 2 species: 93 us).
+constexpr int kDtCells = 4;  // cells per thread
+__device__ __forceinline__ void dt_cell_fp64(const DDArgs& a, int c, double& v2max, double& smax) {
   const int ns = a.ph.ns;
-  for (int c = bid * blockDim.x + threadIdx.x; c < a.T; c += nblocks * blockDim.x) {
-    const int n0 = a.cell[c], n1 = a.cell[a.T + c], n2 = a.cell[2 * a.T + c];
-    const int n3 = a.nvmax == 4 ? a.cell[3 * a.T + c] : -1;  // -1: triangle
-    const bool quad = n3 >= 0;
-    const double w = a.cw[c];
-    const double w2 = w * w;
-    const double inv_nv = quad ? 0.25 : (1.0 / 3.0);
-    double sigma = 0.0;
-#pragma unroll
-    for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
-      if (s < ns) {
-        double vx, vy;
-        if (a.ph.dd_fp32) {  // FP32 velocities, FP64 candidate and reduction
-          const float* d = a.ndat32 + (size_t)s * a.Npad * 4;
-          vx = (double)d[4 * n0 + 2] + (double)d[4 * n1 + 2] + (double)d[4 * n2 + 2];
-          vy = (double)d[4 * n0 + 3] + (double)d[4 * n1 + 3] + (double)d[4 * n2 + 3];
-          if (quad) {
-            vx += (double)d[4 * n3 + 2];
-            vy += (double)d[4 * n3 + 3];
-          }
-        } else {
-          const double* d = a.ndat + (size_t)s * a.Npad * 4;
-          vx = d[4 * n0 + 2] + d[4 * n1 + 2] + d[4 * n2 + 2];
-          vy = d[4 * n0 + 3] + d[4 * n1 + 3] + d[4 * n2 + 3];
-          if (quad) {
-            vx += d[4 * n3 + 2];
-            vy += d[4 * n3 + 3];
-          }
-        }
-        v2max = fmax(v2max, (vx * vx + vy * vy) * w2);
-        const double* nm = a.nm + (size_t)s * a.Npad;
-        double cell = nm[n0] + nm[n1] + nm[n2];
-        if (quad) cell += nm[n3];
-        sigma += fabs(a.ph.sp[s].q * kECharge * cell);
+  const int n0 = a.cell[c], n1 = a.cell[a.T + c], n2 = a.cell[2 * a.T + c];
+  const int n3 = a.nvmax == 4 ? a.cell[3 * a.T + c] : -1;  // -1: triangle
+  const bool quad = n3 >= 0;
+  const double w = a.cw[c], w2 = w * w;
+  const double inv_nv = quad ? 0.25 : (1.0 / 3.0);
+  double sigma = 0.0;
+  for (int s = 0; s < ns; ++s) {
+    double vx, vy;
+    if (a.ph.dd_fp32) {  // FP32 velocities, FP64 candidate and reduction
+      const float* d = a.ndat32 + (size_t)s * a.Npad * 4;
+      vx = (double)d[4 * n0 + 2] + (double)d[4 * n1 + 2] + (double)d[4 * n2 + 2];
+      vy = (double)d[4 * n0 + 3] + (double)d[4 * n1 + 3] + (double)d[4 * n2 + 3];
+      if (quad) {
+        vx += (double)d[4 * n3 + 2];
+        vy += (double)d[4 * n3 + 3];
+      }
+    } else {
+      const double* d = a.ndat + (size_t)s * a.Npad * 4;
+      vx = d[4 * n0 + 2] + d[4 * n1 + 2] + d[4 * n2 + 2];
+      vy = d[4 * n0 + 3] + d[4 * n1 + 3] + d[4 * n2 + 3];
+      if (quad) {
+        vx += d[4 * n3 + 2];
+        vy += d[4 * n3 + 3];
       }
     }
-    smax = fmax(smax, sigma * inv_nv);
+    v2max = fmax(v2max, (vx * vx + vy * vy) * w2);
+    const double* nm = a.nm + (size_t)s * a.Npad;
+    double cell = nm[n0] + nm[n1] + nm[n2];
+    if (quad) cell += nm[n3];
+    sigma += fabs(a.ph.sp[s].q * kECharge * cell);
   }
-  double cand = a.ph.dt_fourier;
-  if (v2max > 0.0) cand = fmin(cand, a.ph.cfl / sqrt(v2max));
-  if (smax > 0.0) cand = fmin(cand, a.ph.a_diel * kEps0 / smax);
-  block_min_to_global(cand, &a.sc->dt_bits);
+  smax = fmax(smax, sigma * inv_nv);
+}
+
+__device__ __forceinline__ void dt_cells_body(const DDArgs& a, int bid, int nblocks) {
+  __shared__ unsigned long long s_max[2];  // bits of the block's FP64 maxima
+  __shared__ unsigned s_lo[2];             // bits of the block's largest FP32 lower bounds
+  __shared__ float s_cur;
+  const int ns = a.ph.ns, stride = nblocks * blockDim.x;
+  constexpr float kEps = 1e-6f;  // FP32 rounding of the sums below, relative to the sum of magnitudes
+  if (threadIdx.x < 2) {
+    s_max[threadIdx.x] = 0;
+    s_lo[threadIdx.x] = 0;
+  }
+  // the running minimum over the blocks already done, rounded up (it only falls)
+  double cur = 0.0;
+  if (threadIdx.x == 0) cur = __longlong_as_double(*(volatile long long*)&a.sc->dt_bits);
+  __syncthreads();
+  for (int base = bid * blockDim.x + threadIdx.x; base - (int)threadIdx.x < a.T; base += kDtCells * stride) {
+    float vhi[kDtCells], shi[kDtCells];  // upper bounds of (|V_cell| / dx) and of the conductivity
+    float vlo = 0.f, slo = 0.f;
+#pragma unroll
+    for (int k = 0; k < kDtCells; ++k) {
+      const int c = base + k * stride;
+      vhi[k] = shi[k] = -1.f;
+      if (c >= a.T || c < base) continue;
+      const int n0 = __ldg(a.cell + c), n1 = __ldg(a.cell + a.T + c), n2 = __ldg(a.cell + 2 * a.T + c);
+      const int n3 = a.nvmax == 4 ? __ldg(a.cell + 3 * a.T + c) : -1;
+      const float w = __ldg(a.cw32 + c);
+      float v = 0.f, vl = 0.f, sig = 0.f, sige = 0.f;
+      for (int s = 0; s < ns; ++s) {
+        const float4* f = a.vf + (size_t)s * a.Npad;
+        const float4 p0 = f[n0], p1 = f[n1], p2 = f[n2];
+        float4 p3 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (n3 >= 0) p3 = f[n3];
+        const float vx = fabsf((p0.x + p1.x) + (p2.x + p3.x)), vy = fabsf((p0.y + p1.y) + (p2.y + p3.y));
+        const float ex = kEps * ((fabsf(p0.x) + fabsf(p1.x)) + (fabsf(p2.x) + fabsf(p3.x)));
+        const float ey = kEps * ((fabsf(p0.y) + fabsf(p1.y)) + (fabsf(p2.y) + fabsf(p3.y)));
+        const float hx = vx + ex, hy = vy + ey, lx = fmaxf(vx - ex, 0.f), ly = fmaxf(vy - ey, 0.f);
+        // !(x <= v): a NaN becomes an upper bound that no test excludes
+        const float h2 = (hx * hx + hy * hy) * (w * w);
+        if (!(h2 <= v)) v = h2;
+        vl = fmaxf(vl, (lx * lx + ly * ly) * (w * w));
+        sig += fabsf((p0.z + p1.z) + (p2.z + p3.z));
+        sige += kEps * ((fabsf(p0.z) + fabsf(p1.z)) + (fabsf(p2.z) + fabsf(p3.z)));
+      }
+      const float inv_nv = n3 >= 0 ? 0.25f : 1.f / 3.f;
+      vhi[k] = v * (1.f + 4.f * kEps);
+      vlo = fmaxf(vlo, vl * (1.f - 4.f * kEps));
+      shi[k] = (sig + sige) * inv_nv * (1.f + 4.f * kEps);
+      slo = fmaxf(slo, fmaxf(sig - sige, 0.f) * inv_nv * (1.f - 4.f * kEps));
+    }
+    // the block's largest lower bounds (bits of nonnegative floats order like integers)
+    const unsigned bv = __reduce_max_sync(0xffffffffu, __float_as_uint(vlo));
+    const unsigned bs = __reduce_max_sync(0xffffffffu, __float_as_uint(slo));
+    if ((threadIdx.x & 31) == 0) {
+      if (bv) atomicMax(&s_lo[0], bv);
+      if (bs) atomicMax(&s_lo[1], bs);
+    }
+    if (threadIdx.x == 0) s_cur = __double2float_ru(cur);
+    __syncthreads();
+    const float now = s_cur, cfl = (float)a.ph.cfl, diel = (float)a.ph.a_diel * (float)(kEps0 / kECharge);
+    const float vthr = __uint_as_float(s_lo[0]), sthr = __uint_as_float(s_lo[1]);
+#pragma unroll
+    for (int k = 0; k < kDtCells; ++k) {
+      const int c = base + k * stride;
+      if (c >= a.T || c < base) continue;
+      const bool ev = !(vhi[k] < vthr) && !(cfl * rsqrtf(vhi[k]) * (1.f - 1e-5f) > now);
+      const bool es = !(shi[k] < sthr) && !(diel / shi[k] * (1.f - 1e-5f) > now);
+      if (ev || es) {
+        double v2 = 0.0, sm = 0.0;
+        dt_cell_fp64(a, c, v2, sm);
+        if (v2 > 0.0) atomicMax(&s_max[0], (unsigned long long)__double_as_longlong(v2));
+        if (sm > 0.0) atomicMax(&s_max[1], (unsigned long long)__double_as_longlong(sm));
+      }
+    }
+  }
+  __syncthreads();
+  // one thread per limit, in different warps (a square root or a division takes 650 cycles)
+  if ((threadIdx.x & 31) == 0 && threadIdx.x < 96) {
+    const int k = threadIdx.x >> 5;
+    double cand = a.ph.dt_fourier;
+    if (k < 2) {
+      const double m = __longlong_as_double((long long)s_max[k]);
+      cand = !(m > 0.0) ? INFINITY : k == 0 ? a.ph.cfl / sqrt(m) : a.ph.a_diel * kEps0 / m;
+    }
+    if (cand > 0.0 && cand < INFINITY) atomicMin(&a.sc->dt_bits, (unsigned long long)__double_as_longlong(cand));
+  }
 }
 
 __global__ void __launch_bounds__(kDDThreads) dt_cells_kernel(DDArgs a) { dt_cells_body(a, blockIdx.x, gridDim.x); }
@@ -616,9 +705,11 @@ __device__ __forceinline__ void node_fields32_body(const DDArgs& a, int with_dt,
         const SpeciesParams& sp = a.ph.sp[s];
         mu[s] = mobility32(sp, Emag);
         const float sg = sp.q > 0 ? 1.0f : -1.0f;
-        reinterpret_cast<float4*>(a.ndat32)[(size_t)s * a.Npad + i] =
-            make_float4(gnx[s], gny[s], sg * mu[s] * Ex, sg * mu[s] * Ey);
-        a.nm[(size_t)s * a.Npad + i] = n[(size_t)s * a.Npad + i] * (double)mu[s];
+        const float vx = sg * mu[s] * Ex, vy = sg * mu[s] * Ey;
+        reinterpret_cast<float4*>(a.ndat32)[(size_t)s * a.Npad + i] = make_float4(gnx[s], gny[s], vx, vy);
+        const double nmu = n[(size_t)s * a.Npad + i] * (double)mu[s];
+        a.nm[(size_t)s * a.Npad + i] = nmu;
+        a.vf[(size_t)s * a.Npad + i] = make_float4(vx, vy, (float)nmu, 0.f);
       } else {
         mu[s] = 0.0f;
       }
@@ -882,9 +973,14 @@ cudaError_t launch_photo_add(const DDArgs& a, int with_dt, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Blocks of the cell time step: up to kDtCells cells per thread, one on small meshes (fewer than
+// 4 blocks per SM otherwise).
+int dt_cells_blocks(int cells, int threads) {
+  const int most = (cells + threads - 1) / threads, least = (cells + kDtCells * threads - 1) / (kDtCells * threads);
+  return most < 4 * 152 ? most : least < 4 * 152 ? 4 * 152 : least;
+}
 cudaError_t launch_dt_cells(const DDArgs& a, cudaStream_t st) {
-  // a few cells per thread: 8 resident blocks on each of the 152 SMs
-  const int blocks = nblk(a.T) < 152 * 8 ? nblk(a.T) : 152 * 8;
+  const int blocks = dt_cells_blocks(a.T, kDDThreads);
   dt_cells_kernel<<<blocks, kDDThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
