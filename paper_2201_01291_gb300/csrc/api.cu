@@ -63,7 +63,7 @@ struct avip_mesh {
   float* cw32 = nullptr;
   float4* vf = nullptr;
   int32_t *e_lo = nullptr, *e_hi = nullptr, *slot_eid = nullptr;  // edge list (flux once per edge)
-  double *e_sx = nullptr, *e_sy = nullptr, *eflux = nullptr;
+  double *e_hx = nullptr, *e_hy = nullptr, *e_dx = nullptr, *e_dy = nullptr, *eflux = nullptr;
   double *phi1 = nullptr, *phi2 = nullptr, *phi3 = nullptr;  // the three previous potentials (predictor)
   double *phi = nullptr, *xs = nullptr, *b = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
   double *nbuf = nullptr, *ndat = nullptr, *nm = nullptr, *src = nullptr, *Ex = nullptr, *Ey = nullptr;
@@ -268,8 +268,10 @@ DDArgs dd_args(const avip_mesh* h) {
   a.vf = h->vf;
   a.e_lo = h->e_lo;
   a.e_hi = h->e_hi;
-  a.e_sx = h->e_sx;
-  a.e_sy = h->e_sy;
+  a.e_hx = h->e_hx;
+  a.e_hy = h->e_hy;
+  a.e_dx = h->e_dx;
+  a.e_dy = h->e_dy;
   a.slot_eid = h->slot_eid;
   a.eflux = h->eflux;
   a.E = (int32_t)h->hm.e_lo.size();
@@ -429,6 +431,13 @@ int read_scalars(avip_mesh* h, DevScalars& out) {
   cudaError_t e = cudaMemcpyAsync(&out, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   return cuda_status(e);
+}
+
+// Half of every entry (exact).
+std::vector<double> halved(const std::vector<double>& v) {
+  std::vector<double> r(v.size());
+  for (size_t i = 0; i < v.size(); ++i) r[i] = 0.5 * v[i];
+  return r;
 }
 
 bool ready(const avip_mesh* h) { return h && h->ph.ns > 0 && h->species_declared == h->ph.ns; }
@@ -646,7 +655,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
             upload(h, h->gy, m.gy) && upload(h, h->sx, m.sx) && upload(h, h->sy, m.sy) &&
             upload(h, h->cell, m.cell) && upload(h, h->flen, m.flen) && upload(h, h->cw, m.cw) && upload(h, h->cw32, std::vector<float>(m.cw.begin(), m.cw.end())) &&
             zalloc(h, h->vf, (size_t)AVIP_MAX_SPECIES * Np) && upload(h, h->e_lo, m.e_lo, 1) && upload(h, h->e_hi, m.e_hi, 1) &&
-            upload(h, h->e_sx, m.e_sx, 1) && upload(h, h->e_sy, m.e_sy, 1) && upload(h, h->slot_eid, m.slot_eid) &&
+            upload(h, h->e_hx, halved(m.e_sx), 1) && upload(h, h->e_hy, halved(m.e_sy), 1) && upload(h, h->e_dx, m.e_dx, 1) &&
+            upload(h, h->e_dy, m.e_dy, 1) && upload(h, h->slot_eid, m.slot_eid) &&
             zalloc(h, h->eflux, (size_t)AVIP_MAX_SPECIES * std::max<size_t>(m.e_lo.size(), 1)) && upload(h, h->x, m.x, Np) &&
             upload(h, h->y, m.y, Np) && upload(h, h->vol, m.vol, Np) && upload(h, h->ivol, inverse_volumes(m.vol), Np) && upload(h, h->dsq, m.dsq, Np) && upload(h, h->dsqinv, m.dsqinv, Np) &&
             upload(h, h->lift, m.lift, Np) && upload(h, h->rhs_scale, m.rhs_scale, Np);
@@ -869,6 +879,7 @@ int species_set(avip_mesh_t h, int32_t s, int32_t charge, int32_t mob_model, con
   sp.mob_log_ref = mob_model == AVIP_MOB_POWER ? std::log(mob_params[1]) : 0.0;
   sp.mob_model = mob_model;
   sp.bnd_mode = bnd_mode;
+  sp.immobile = mob_model == AVIP_MOB_CONST && mob_params[0] == 0.0 && D == 0.0 ? 1 : 0;
   if (s == h->species_declared) h->species_declared++;
   h->ph.ns = h->species_declared;
   // density into the current parity buffer

@@ -52,6 +52,7 @@ struct HostMesh {
   // element of an edge slot the edge id, bit 31 set when the row is the edge's hi end
   std::vector<int32_t> e_lo, e_hi, slot_eid;
   std::vector<double> e_sx, e_sy;
+  std::vector<double> e_dx, e_dy;     // per edge x_hi - x_lo
   std::vector<double> lift;           // N: free rows -sum_{k in D} K_ik phi_D,k ; Dirichlet rows phi_D (scaled by 1/sqrt(K_ii))
   std::vector<double> rhs_scale;      // N: free rows e V_i / eps0 ; Dirichlet rows 0 (scaled by 1/sqrt(K_ii))
 };
@@ -190,6 +191,8 @@ struct SpeciesParams {
   double mob_log_ref;  // log(mob[1]) for AVIP_MOB_POWER (set on the host)
   int32_t mob_model;
   int32_t bnd_mode;
+  int32_t immobile;    // constant zero mobility and D = 0: no flux, so no gradient is needed
+  int32_t pad;
 };
 
 struct Physics {
@@ -431,8 +434,10 @@ struct DDArgs {
   // row evaluates the fluxes of its edges itself)
   const int32_t* e_lo;
   const int32_t* e_hi;
-  const double* e_sx;
-  const double* e_sy;
+  const double* e_hx;     // half of the edge normal S_lo->hi, and x_hi - x_lo
+  const double* e_hy;
+  const double* e_dx;
+  const double* e_dy;
   const int32_t* slot_eid;
   double* eflux;          // [species][E]: flux from lo to hi
   int32_t E;

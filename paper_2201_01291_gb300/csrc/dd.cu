@@ -106,7 +106,7 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
       }
 #pragma unroll
       for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
-        if (s < ns) {
+        if (s < ns && !a.ph.sp[s].immobile) {
           double uj[kG];
 #pragma unroll
           for (int u = 0; u < kG; ++u) uj[u] = n[(size_t)s * a.Npad + c[u]];
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kDDThreads) dt_cells_kernel(DDArgs a) { dt_cel
 
 // ------------------------------------------------------------------------ fluxes + update
 struct EdgeEnd {
-  double u, gx, gy, vx, vy, x, y;
+  double u, gx, gy, vx, vy;
 };
 
 // Bernoulli function B(x) = x / (e^x - 1) for x >= 0 (B(0) = 1; 0 once e^x overflows).
@@ -393,38 +393,65 @@ __device__ __forceinline__ double sg_flux(double ulo, double uhi, const SgGeo& G
   return fpar + fperp;
 }
 
-// Flux from `lo` to `hi` through the dual face with normal (Sx, Sy) oriented lo -> hi:
+// The sign and magnitude tests of the flux on the bit patterns: an FP64 comparison costs as much as
+// an FP64 multiply-add (19 cycles per warp and SM), integer ones next to nothing.
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
+__device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ double flip_sign(double x, bool flip) {
+  return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
+}
+
+// Sum of the block's values into *dst in a fixed order: the warps' values through shared memory to
+// one warp, which adds a column each and finishes with a shuffle tree (nw + 4 warp-wide FP64 adds
+// instead of the 5 nw + 5 of a tree in every warp).
+__device__ __forceinline__ void block_charge(double q, double* dst) {
+  __shared__ double thr[kDDThreads];
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  thr[threadIdx.x] = q;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = thr[lane];
+    for (int w = 1; w < nw; ++w) t += thr[w * 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) *dst = t;
+  }
+}
+
+// Flux from `lo` to `hi` through the dual face with normal 2 (Hx, Hy) oriented lo -> hi:
 // limited Lax-Wendroff convective part with a virtual upwind node plus central diffusion, or
-// (sg != nullptr) the Scharfetter-Gummel flux.
+// (sg != nullptr) the Scharfetter-Gummel flux.  (dx, dy) = x_hi - x_lo, dt4 = dt / 4.
 //
 // The edge means V_ij = (V_i + V_j)/2 and grad_ij = (grad_i + grad_j)/2 are kept as sums and the
-// halves folded into the products that use them: scaling by a power of two is exact in floating
-// point, so this adds no rounding, for four FP64 multiplications fewer per edge and species (the
-// FP64 issue rate bounds this kernel on GB300).
-__device__ __forceinline__ double edge_flux(const EdgeEnd& lo, const EdgeEnd& hi, double Sx, double Sy,
-                                            double D, double dt, double beta, int lim, const SgGeo* sg) {
+// halves folded into the half normals and into psi / 2: scaling by a power of two is exact, so
+// this adds no rounding.  23 FP64 operations per edge and species (33 with the halves, the sign
+// and range tests and the coordinate differences in FP64): the FP64 issue rate bounds the kernel
+// on GB300.
+__device__ __forceinline__ double edge_flux(const EdgeEnd& lo, const EdgeEnd& hi, double dx, double dy, double Hx,
+                                            double Hy, double D, double dt4, double beta, int lim, const SgGeo* sg) {
   if (sg)
     return sg_flux(lo.u, hi.u, *sg, 0.5 * (lo.vx + hi.vx), 0.5 * (lo.vy + hi.vy), 0.5 * (lo.gx + hi.gx),
                    0.5 * (lo.gy + hi.gy), D);
   const double sVx = lo.vx + hi.vx, sVy = lo.vy + hi.vy;  // 2 V_ij
   const double sgx = lo.gx + hi.gx, sgy = lo.gy + hi.gy;  // 2 grad_ij
-  const double av = 0.5 * (sVx * Sx + sVy * Sy);          // V_ij . S
-  const bool up_lo = av >= 0.0;
-  const EdgeEnd& U = up_lo ? lo : hi;
-  const EdgeEnd& W = up_lo ? hi : lo;
-  const double delta = W.u - U.u;
-  double psi = 0.0;
-  if (delta != 0.0) {
-    const double dx = W.x - U.x, dy = W.y - U.y;
-    // the ratio of the upwind to the local difference
-    const double r = (2.0 * (U.gx * dx + U.gy * dy) - delta) * recip_nr(delta);
-    psi = (lim == AVIP_LIM_SWEBY && beta == 1.0) ? fmax(0.0, fmin(r, 1.0))  // min-mod: the same value
-                                                 : limiter(r, beta, lim);
+  const double av = fma(sVx, Hx, sVy * Hy);               // V_ij . S
+  const bool up_hi = negative(av);                        // (-0: no flux either way)
+  const double uU = up_hi ? hi.u : lo.u;
+  const double gU = fma(up_hi ? hi.gx : lo.gx, dx, (up_hi ? hi.gy : lo.gy) * dy);  // grad_U . (x_hi - x_lo)
+  const double d = hi.u - lo.u;
+  const double delta = flip_sign(d, up_hi);               // u_W - u_U
+  const double num = fma(flip_sign(2.0, up_hi), gU, -delta);  // 2 grad_U . (x_W - x_U) - delta = r delta
+  double hpsi = 0.0;                                      // psi / 2
+  const long long ad = abs_bits(delta), an = abs_bits(num);
+  if (lim == AVIP_LIM_SWEBY && beta == 1.0) {  // min-mod: psi = clamp(r, 0, 1)
+    const bool same = ((__double2hiint(delta) ^ __double2hiint(num)) >= 0);
+    if (ad != 0 && same) hpsi = an >= ad ? 0.5 : (0.5 * num) * recip_nr(delta);
+  } else if (ad != 0) {
+    hpsi = 0.5 * limiter(num * recip_nr(delta), beta, lim);
   }
-  const double lw = 0.5 * delta - (0.125 * dt) * (sgx * sVx + sgy * sVy);  // delta/2 - dt/2 grad_ij.V_ij
-  const double fc = (U.u + lw * psi) * av;
-  const double fd = -(0.5 * D) * (sgx * Sx + sgy * Sy);                    // -D grad_ij.S
-  return fc + fd;
+  const double lw = fma(-dt4, fma(sgx, sVx, sgy * sVy), delta);  // delta - dt grad_ij.V_ij
+  const double us = fma(lw, hpsi, uU);
+  return fma(us, av, -D * fma(sgx, Hx, sgy * Hy));               // minus D grad_ij . S
 }
 
 // kGather: the edge fluxes were evaluated once per edge (edge_flux_kernel) and are gathered;
@@ -436,6 +463,7 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
   const int N = a.A.N;
   const int ns = a.ph.ns;
   const double dt = a.ph.dt_fixed > 0.0 ? a.ph.dt_fixed : __longlong_as_double((long long)a.sc->dt_bits);
+  const double dt4 = 0.25 * dt;
   double qsum = 0.0;
   if (i < N) {
     const int par = a.sc->parity;
@@ -444,16 +472,20 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
     const int slice = i / kSlice, lane = i % kSlice;
     const int base = __ldg(a.A.sl_ptr + slice) + lane;
     const int rl = __ldg(a.flen + i);  // edge slots only
-    const double xi = a.x[i], yi = a.y[i];
+    const double xi = kGather ? 0.0 : a.x[i], yi = kGather ? 0.0 : a.y[i];
     double R[AVIP_MAX_SPECIES];
     EdgeEnd me[AVIP_MAX_SPECIES];
 #pragma unroll
     for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
       R[s] = 0.0;
       if (s < ns) {
-        const double2* d = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + i) * 4);
-        const double2 g = d[0], v = d[1];
-        me[s] = EdgeEnd{n[(size_t)s * a.Npad + i], g.x, g.y, v.x, v.y, xi, yi};
+        double2 g = make_double2(0.0, 0.0), v = g;
+        if (!kGather) {  // (the gathering form reads the record of a boundary row only)
+          const double2* d = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + i) * 4);
+          g = d[0];
+          v = d[1];
+        }
+        me[s] = EdgeEnd{n[(size_t)s * a.Npad + i], g.x, g.y, v.x, v.y};
       }
     }
     if (kGather) {
@@ -466,13 +498,13 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
         for (int u = 0; u < kG; ++u) v[u] = k0 + u < rl ? __ldg(a.slot_eid + base + (k0 + u) * kSlice) : 0;
 #pragma unroll
         for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
-          if (s < ns) {
+          if (s < ns && !a.ph.sp[s].immobile) {
             double F[kG];
 #pragma unroll
             for (int u = 0; u < kG; ++u) F[u] = k0 + u < rl ? a.eflux[(size_t)s * a.E + (v[u] & 0x7fffffff)] : 0.0;
 #pragma unroll
             for (int u = 0; u < kG; ++u)
-              if (k0 + u < rl) R[s] = v[u] >= 0 ? R[s] - F[u] : R[s] + F[u];
+              if (k0 + u < rl) R[s] += flip_sign(F[u], v[u] >= 0);  // (the row is the lo end: flux out)
           }
         }
       }
@@ -482,62 +514,56 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
       const int j = __ldg(a.A.col + e);
       const double Sx = __ldg(a.A.sx + e), Sy = __ldg(a.A.sy + e);
       const bool lo_is_me = i < j;
-      const double xj = a.x[j], yj = a.y[j];
+      // canonical lo -> hi: the stored normal and the difference below are oriented i -> j
+      const double dx = flip_sign(a.x[j] - xi, !lo_is_me), dy = flip_sign(a.y[j] - yi, !lo_is_me);
+      const double Hx = flip_sign(0.5 * Sx, !lo_is_me), Hy = flip_sign(0.5 * Sy, !lo_is_me);
       SgGeo geo;
       const bool use_sg = a.ph.scheme == AVIP_FLUX_SG;
-      if (use_sg)  // canonical lo -> hi, like the flux itself
-        geo = lo_is_me ? sg_geometry(xj - xi, yj - yi, Sx, Sy) : sg_geometry(xi - xj, yi - yj, -Sx, -Sy);
+      if (use_sg) geo = sg_geometry(dx, dy, 2.0 * Hx, 2.0 * Hy);
 #pragma unroll
       for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
-        if (s < ns) {
+        if (s < ns && !a.ph.sp[s].immobile) {
           const double2* d = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + j) * 4);
           const double2 g = d[0], v = d[1];
-          const EdgeEnd other{n[(size_t)s * a.Npad + j], g.x, g.y, v.x, v.y, xj, yj};
+          const EdgeEnd other{n[(size_t)s * a.Npad + j], g.x, g.y, v.x, v.y};
           const EdgeEnd& lo = lo_is_me ? me[s] : other;
           const EdgeEnd& hi = lo_is_me ? other : me[s];
-          // the stored normal is oriented i -> j; the canonical one lo -> hi
-          const double sgn = lo_is_me ? 1.0 : -1.0;
-          const double F = edge_flux(lo, hi, sgn * Sx, sgn * Sy, a.ph.sp[s].D, dt, a.ph.beta, a.ph.limiter,
+          const double F = edge_flux(lo, hi, dx, dy, Hx, Hy, a.ph.sp[s].D, dt4, a.ph.beta, a.ph.limiter,
                                      use_sg ? &geo : nullptr);
-          R[s] = lo_is_me ? R[s] - F : R[s] + F;
+          R[s] += flip_sign(F, lo_is_me);
         }
       }
     }
     // boundary closure through the boundary nodal normal kept in the diagonal slot
+    // (an interior row's S_i^b is exactly zero and its closure term with it)
     const double Sbx = __ldg(a.A.sx + base), Sby = __ldg(a.A.sy + base);
+    const bool rim = (abs_bits(Sbx) | abs_bits(Sby)) != 0;
     const double Vi = a.vol[i], iVi = a.ivol[i];
     bool bad = false;
 #pragma unroll
     for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
       if (s < ns) {
         const SpeciesParams& sp = a.ph.sp[s];
-        double Fx = me[s].u * me[s].vx, Fy = me[s].u * me[s].vy;
-        if (sp.bnd_mode == AVIP_BND_OUTFLOW) {
-          Fx -= sp.D * me[s].gx;
-          Fy -= sp.D * me[s].gy;
+        double rs = R[s];
+        if (rim) {
+          const double2* d = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + i) * 4);
+          const double2 g = d[0], v = d[1];
+          double Fx = me[s].u * v.x, Fy = me[s].u * v.y;
+          if (sp.bnd_mode == AVIP_BND_OUTFLOW) {
+            Fx -= sp.D * g.x;
+            Fy -= sp.D * g.y;
+          }
+          rs -= Fx * Sbx + Fy * Sby;
         }
-        const double rs = R[s] - (Fx * Sbx + Fy * Sby);
         const double un = me[s].u + dt * fma(rs, iVi, a.src[(size_t)s * a.Npad + i]);
         nn[(size_t)s * a.Npad + i] = un;
-        bad |= !isfinite(un);
-        qsum += sp.q * (Vi * un);
+        bad |= (__double2hiint(un) & 0x7ff00000) == 0x7ff00000;
+        qsum = fma(flip_sign(Vi, negative(sp.q)), un, qsum);  // charge numbers are -1 or +1
       }
     }
     if (bad) atomicCAS(&a.sc->status, AVIP_OK, AVIP_ENAN);
   }
-  // per-block charge partial (fixed order)
-  __shared__ double sm[32];
-  const int ln = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) qsum += __shfl_xor_sync(0xffffffffu, qsum, o);
-  if (ln == 0) sm[warp] = qsum;
-  __syncthreads();
-  if (warp == 0) {
-    double t = ln < nw ? sm[ln] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (ln == 0) a.partials[bid] = t;
-  }
+  block_charge(qsum, a.partials + bid);
   if (bid == 0 && threadIdx.x == 0) a.sc->dt = dt;
 }
 
@@ -553,24 +579,24 @@ __global__ void __launch_bounds__(kDDThreads) edge_flux_kernel(DDArgs a) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= a.E) return;
   const int ns = a.ph.ns;
-  const double dt = a.ph.dt_fixed > 0.0 ? a.ph.dt_fixed : __longlong_as_double((long long)a.sc->dt_bits);
+  const double dt4 = 0.25 * (a.ph.dt_fixed > 0.0 ? a.ph.dt_fixed : __longlong_as_double((long long)a.sc->dt_bits));
   const double* n = a.nbuf + (size_t)a.sc->parity * AVIP_MAX_SPECIES * a.Npad;
   const int lo = __ldg(a.e_lo + e), hi = __ldg(a.e_hi + e);
-  const double Sx = __ldg(a.e_sx + e), Sy = __ldg(a.e_sy + e);
-  const double xl = a.x[lo], yl = a.y[lo], xh = a.x[hi], yh = a.y[hi];
+  const double Hx = __ldg(a.e_hx + e), Hy = __ldg(a.e_hy + e);  // half normal
+  const double dx = __ldg(a.e_dx + e), dy = __ldg(a.e_dy + e);
   const bool use_sg = a.ph.scheme == AVIP_FLUX_SG;
   SgGeo geo;
-  if (use_sg) geo = sg_geometry(xh - xl, yh - yl, Sx, Sy);
+  if (use_sg) geo = sg_geometry(dx, dy, 2.0 * Hx, 2.0 * Hy);
 #pragma unroll
   for (int s = 0; s < AVIP_MAX_SPECIES; ++s) {
-    if (s < ns) {
+    if (s < ns && !a.ph.sp[s].immobile) {
       const double2* dl = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + lo) * 4);
       const double2* dh = reinterpret_cast<const double2*>(a.ndat + ((size_t)s * a.Npad + hi) * 4);
       const double2 gl = dl[0], vl = dl[1], gh = dh[0], vh = dh[1];
-      const EdgeEnd L{n[(size_t)s * a.Npad + lo], gl.x, gl.y, vl.x, vl.y, xl, yl};
-      const EdgeEnd H{n[(size_t)s * a.Npad + hi], gh.x, gh.y, vh.x, vh.y, xh, yh};
+      const EdgeEnd L{n[(size_t)s * a.Npad + lo], gl.x, gl.y, vl.x, vl.y};
+      const EdgeEnd H{n[(size_t)s * a.Npad + hi], gh.x, gh.y, vh.x, vh.y};
       a.eflux[(size_t)s * a.E + e] =
-          edge_flux(L, H, Sx, Sy, a.ph.sp[s].D, dt, a.ph.beta, a.ph.limiter, use_sg ? &geo : nullptr);
+          edge_flux(L, H, dx, dy, Hx, Hy, a.ph.sp[s].D, dt4, a.ph.beta, a.ph.limiter, use_sg ? &geo : nullptr);
     }
   }
 }
@@ -886,18 +912,7 @@ __device__ __forceinline__ void flux_update32_body(const DDArgs& a, int bid) {
     }
     if (bad) atomicCAS(&a.sc->status, AVIP_OK, AVIP_ENAN);
   }
-  __shared__ double sm[32];
-  const int ln = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) qsum += __shfl_xor_sync(0xffffffffu, qsum, o);
-  if (ln == 0) sm[warp] = qsum;
-  __syncthreads();
-  if (warp == 0) {
-    double t = ln < nw ? sm[ln] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (ln == 0) a.partials[bid] = t;
-  }
+  block_charge(qsum, a.partials + bid);
   if (bid == 0 && threadIdx.x == 0) a.sc->dt = dt;
 }
 

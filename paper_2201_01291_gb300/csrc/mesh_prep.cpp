@@ -478,6 +478,8 @@ int prepare_mesh(const double* xy, int32_t n_nodes, const int32_t* tris, int32_t
     m.e_hi.resize(E);
     m.e_sx.resize(E);
     m.e_sy.resize(E);
+    m.e_dx.resize(E);
+    m.e_dy.resize(E);
     m.slot_eid.assign(off, 0);
     for (int32_t i = 0; i < N; ++i) {
       int32_t e = first[i];
@@ -488,6 +490,8 @@ int prepare_mesh(const double* xy, int32_t n_nodes, const int32_t* tris, int32_t
           m.e_hi[e] = j;
           m.e_sx[e] = Sx[rowptr[i] + k];
           m.e_sy[e] = Sy[rowptr[i] + k];
+          m.e_dx[e] = m.x[j] - m.x[i];
+          m.e_dy[e] = m.y[j] - m.y[i];
           ++e;
         }
       }
