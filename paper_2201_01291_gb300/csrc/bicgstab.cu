@@ -246,8 +246,9 @@ PcgPlan bicgstab_plan(int nslices, int requested_tpb) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bicgstab_fp64_kernel, kBcgTPB, 0);
-  const int wpb = kBcgTPB / kSlice;
-  const int want = (nslices + wpb - 1) / wpb;
+  // four slices per block: an SM issues one FP64 warp instruction per 19 cycles, so a slice per warp
+  // of a 24-warp block (the former partition) left each block FP64-bound on a few SMs
+  const int want = (nslices + 3) / 4;
   pl.blocks = std::max(1, std::min(std::max(occ, 1) * std::max(sms, 1), want));
   return pl;
 }
