@@ -61,7 +61,6 @@ constexpr double kTheta = 0.08;
 constexpr double kJacobiOmega = 1.7;  // omega = kJacobiOmega / lambda_max(D^-1 A)
 constexpr int kCoarseMin = 256, kCoarseMax = 1500;
 constexpr int kManySlices = 152 * 24;  // warps of a whole-GPU solve
-constexpr int kDirectRows = 512;  // meshes up to this size: the inverse of the matrix itself
 
 // y = A x (CSR)
 void csr_mv(const Csr& A, const std::vector<double>& x, std::vector<double>& y) {
@@ -432,10 +431,10 @@ int lanes_per_row(const Csr& A, bool mixed) {
   return lpr;
 }
 
-int amg_setup(const HostMesh& m, bool mixed, AmgHost& H, char* err, size_t errlen) {
+int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
   // the axisymmetric matrix is not symmetric: no symmetrisation, LU instead of Cholesky
   const bool symmetric = m.geometry != AVIP_GEOM_AXISYMMETRIC;
-  const int32_t coarse_max = !mixed && m.N <= kDirectRows ? m.N : std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
+  const int32_t coarse_max = std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
   auto fail = [&](const char* msg) {
     if (err && errlen) std::snprintf(err, errlen, "%s", msg);
     return AVIP_EINVAL;

@@ -61,7 +61,8 @@ struct SolveShared {
   int bad;                          // a warp's copy did not arrive (Ring::wait)
 };
 // Dynamic shared memory of a solve: the rings, then the dense product's right-hand side.
-constexpr size_t kRhsBytes = sizeof(double) * kAmgDenseRows;
+constexpr size_t kRhsBytes = sizeof(float) * kInverseRows;
+static_assert(kRhsBytes >= sizeof(double) * kAmgDenseRows, "an FP64 hierarchy has no inverse of the finest matrix");
 template <typename T>
 struct AmgCtx {
   const AmgDevT<T>* H;  // shared memory
@@ -71,13 +72,18 @@ struct AmgCtx {
   __device__ __forceinline__ int mat_phase() const { return 2 * D.level + 1; }
 };
 
-// The larger dense level as long as a CTA's share of it stays within 256 KB per product (2.5 us of
-// L2 bandwidth); the coarsest inverse on fewer CTAs.
-constexpr size_t kDenseBytesPerCta = 256 * 1024;
+// The finest dense operator whose share per CTA and product stays within a bound: 576 KB for the
+// inverse of the matrix (11,000 cycles of L2 bandwidth, which save every other level and three
+// quarters of the iterations), 256 KB for the V-cycle's tail, which saves a few phases; the
+// coarsest inverse on fewer CTAs.
+constexpr size_t kInverseBytesPerCta = 576 * 1024, kDenseBytesPerCta = 256 * 1024;
 template <typename T>
 __device__ __forceinline__ int dense_choice(const AmgDevT<T>& H, int nctas) {
-  const size_t bytes = (size_t)H.L[H.dense[0].level].n * H.dense[0].steps * kSlice * sizeof(T);
-  return bytes <= kDenseBytesPerCta * (size_t)nctas ? 0 : 1;
+  auto bytes = [&](int k) {
+    return (size_t)H.L[H.dense[k].level].n * H.dense[k].steps * kSlice * sizeof(T);
+  };
+  if (H.dense[0].m && bytes(0) <= kInverseBytesPerCta * (size_t)nctas) return 0;
+  return bytes(1) <= kDenseBytesPerCta * (size_t)nctas ? 1 : 2;
 }
 
 // Start of a solve: the hierarchy's descriptors copied to shared memory, the phase table written
@@ -102,7 +108,7 @@ __device__ AmgCtx<T> solve_begin(SolveShared& sh, R& ring, char* dyn, const PcgA
   C.gain = sh.gain;
   C.rhs = reinterpret_cast<T*>(dyn + (blockDim.x >> 5) * R::kWarpBytes);
   C.H = reinterpret_cast<const AmgDevT<T>*>(sh.H);
-  C.D = C.H->dense[keep ? 1 : dense_choice(*C.H, nctas)];
+  C.D = C.H->dense[keep ? 2 : dense_choice(*C.H, nctas)];
   const int dl = C.D.level, p = (int)threadIdx.x;
   if (p <= 2 * dl + 1) {
     PhaseDesc d;

@@ -42,6 +42,9 @@ cudaError_t launch_state_take(const StateArgs& s, cudaStream_t st);
 cudaError_t launch_state_check(const StateArgs& s, cudaStream_t st);
 cudaError_t launch_state_put(const StateArgs& s, cudaStream_t st);
 int flux_partials_max(int N);
+int dense_inverse_rows(int N);
+size_t dense_inverse_scratch(int N);
+cudaError_t launch_dense_inverse(const SellView& A, float* M, float* scratch, cudaStream_t st);
 }  // namespace avip
 
 using namespace avip;
@@ -127,6 +130,10 @@ constexpr int kClusterMixedMinRows = 500;  // mixed precision: Jacobi-PCG on one
 // BiCGStab preconditioned by the AMG V-cycle above this many nodes, Jacobi-scaled below: at 10,201
 // nodes its two V-cycles per iteration replace 290 iterations per step by 8.5 (8.7 -> 0.42 ms)
 constexpr int kBicgstabAmgRows = 3000;
+// Planar FP64 meshes of up to kInverseRows nodes have the inverse of the matrix as their
+// preconditioner: one cluster applies it up to kClusterInverseRows (5.8 MB over 16 CTAs), the whole
+// GPU above.
+constexpr int kClusterInverseRows = 1200;
 constexpr int kClusterAutoRows = 20000;  // one-cluster solvers up to this many nodes
 
 void* dev_alloc(avip_mesh* h, size_t bytes) {
@@ -455,7 +462,8 @@ void invalidate_graph(avip_mesh* h) {
 // non-coarsest level the composite operators Q, Rf, U, Pf in SELL-32 and the vectors xp (and,
 // below the finest level, x and b); the coarsest level's x, b and its dense inverse.
 template <typename T>
-bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record = true) {
+bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record = true,
+                  const float* inverse = nullptr) {
   AmgDevT<T> D;
   std::memset(&D, 0, sizeof(D));
   D.nlev = (int32_t)H.lv.size();
@@ -517,11 +525,12 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
     }
     if (l > 0) ok = ok && zalloc(h, dl.b, npad);
   }
-  ok = ok && put_dense(H.cinv, D.nlev - 1, D.dense[1]);
+  ok = ok && put_dense(H.cinv, D.nlev - 1, D.dense[2]);
   if (H.dlev == D.nlev - 1)
-    D.dense[0] = D.dense[1];
+    D.dense[1] = D.dense[2];
   else
-    ok = ok && put_dense(H.dmat, H.dlev, D.dense[0]);
+    ok = ok && put_dense(H.dmat, H.dlev, D.dense[1]);
+  if (inverse) D.dense[0] = AmgDenseT<T>{(const T*)inverse, 0, dense_inverse_rows(H.lv[0].A.n) / kSlice};
   auto* dd = static_cast<AmgDevT<T>*>(dev_alloc(h, sizeof(D)));
   ok = ok && dd && cudaMemcpyAsync(dd, &D, sizeof(D), cudaMemcpyHostToDevice, h->stream) == cudaSuccess &&
        cudaStreamSynchronize(h->stream) == cudaSuccess;
@@ -538,7 +547,7 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
 
 // Upload the hierarchy in the handle's preconditioner precision (FP64 values when asked for and
 // the solve is not the mixed-precision one) with its preconditioned-residual vector.
-bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np) {
+bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np, bool with_inverse = false) {
   if (!zalloc(h, h->colS, h->hm.col.size() + kStreamPad) ||
       launch_mark_slices(h->sl_ptr, h->hm.nslices, h->col, h->colS, h->stream) != cudaSuccess)
     return false;
@@ -546,7 +555,15 @@ bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np) {
   if (fp64) return upload_amg_t<double>(h, H, h->amg) && zalloc(h, h->amg_z, Np) && zalloc(h, h->r2, Np);
   // (the FP64 CG writes its preconditioned residual in FP64 whatever the hierarchy's type; the
   // mixed-precision solve keeps its own FP32 one)
-  return upload_amg_t<float>(h, H, h->amg32) && zalloc(h, h->z32, Np) && zalloc(h, h->amg_z, Np) &&
+  float* inverse = nullptr;
+  if (with_inverse) {
+    const size_t np = (size_t)dense_inverse_rows(h->hm.N);
+    float* scratch = nullptr;
+    if (!zalloc(h, inverse, np * np + kStreamPad) || !zalloc(h, scratch, dense_inverse_scratch(h->hm.N)) ||
+        launch_dense_inverse(sell_view(h), inverse, scratch, h->stream) != cudaSuccess)
+      return false;
+  }
+  return upload_amg_t<float>(h, H, h->amg32, true, inverse) && zalloc(h, h->z32, Np) && zalloc(h, h->amg_z, Np) &&
          zalloc(h, h->r2, Np) && zalloc(h, h->rq32, 3 * Np);
 }
 
@@ -687,15 +704,19 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // or three iterations replace the 70 to 90 of the Jacobi form.
   PcgPlan amg_cluster;
   amg_cluster.kind = 0;
-  if (!bicg && (h->opts.pcg_kind == 11 || (h->opts.pcg_kind == 0 && m.N <= kClusterAutoRows &&
-                 !(h->opts.precision == AVIP_PREC_MIXED && m.N <= kClusterMixedMinRows))))
+  const bool fp64 = h->opts.precision == AVIP_PREC_FP64;
+  // the inverse of the matrix as the preconditioner (dense_inverse.cu)
+  const bool inverse = !bicg && h->opts.pcg_kind == 0 && fp64 && !h->opts.precond_fp64 && m.N <= kInverseRows;
+  if (!bicg && (h->opts.pcg_kind == 11 ||
+                (h->opts.pcg_kind == 0 && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
+                 (fp64 || m.N > kClusterMixedMinRows))))
     amg_cluster = amg_cluster_plan(h->opts.cluster_size, m.N);
   // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above the cluster size
   const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (h->opts.pcg_kind == 0 && m.N > kBicgstabAmgRows));
   if (bicg) {
     h->plan = bicgstab_plan(m.nslices, h->opts.pcg_threads);
     ok = ok && zalloc(h, h->bcg, (bicg_amg ? 5 : 3) * Np);
-  } else if ((h->opts.pcg_kind == 0 && amg_cluster.kind != 11) || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
+  } else if ((h->opts.pcg_kind == 0 && amg_cluster.kind != 11 && !inverse) || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
     // small meshes: one thread-block cluster with everything in shared memory
     // (the Jacobi form, when asked for or when the AMG form below cannot be scheduled)
     const int mixed = h->opts.precision == AVIP_PREC_MIXED ? 1 : 0;
@@ -716,15 +737,15 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
                    (h->opts.pcg_kind == 8 ||
                     (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
     AmgHost H;
-    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
       delete h;
       return rc;
     }
-    ok = ok && upload_amg(h, H, Np);
-    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, bicg ? 9 : 8, h->amg ? 1 : 0);
+    ok = ok && upload_amg(h, H, Np, inverse);
+    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, bicg ? 9 : 8, h->amg ? 1 : 0, inverse ? m.N : 0);
   }
   if (h->opts.precision == AVIP_PREC_MIXED) {
     std::vector<float> a32(m.aval.begin(), m.aval.end());
@@ -745,7 +766,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
       (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
     AmgHost H;
-    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -757,14 +778,14 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   }
   if (amg_cluster.kind == 11) {
     AmgHost H;
-    int rc = amg_setup(m, h->opts.precision == AVIP_PREC_MIXED, H, g_err, sizeof(g_err));
+    int rc = amg_setup(m, H, g_err, sizeof(g_err));
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
       delete h;
       return rc;
     }
-    ok = ok && upload_amg(h, H, Np);
+    ok = ok && upload_amg(h, H, Np, inverse);
     h->plan = amg_cluster;
   }
   h->nparts = flux_blocks(m.N);
@@ -993,7 +1014,7 @@ int photo_set(avip_mesh_t h, int32_t n_terms, const double* a, const double* kap
       hm.aval = std::move(val);
       hm.dsq.assign(dh.begin(), dh.begin() + m.N);
       AmgHost H;
-      if (amg_setup(hm, false, H, g_err, sizeof(g_err)) != AVIP_OK) return AVIP_EINVAL;
+      if (amg_setup(hm, H, g_err, sizeof(g_err)) != AVIP_OK) return AVIP_EINVAL;
       if (h->amg)
         ok = upload_amg_t<double>(h, H, t.amg, false);
       else

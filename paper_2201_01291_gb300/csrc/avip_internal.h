@@ -97,10 +97,12 @@ struct AmgHost {
 // in FP32, 62 KB per SM of a whole-GPU solve and so about 0.6 us of L2 bandwidth, against two to
 // four phases of 2 us and more for the levels it replaces.
 constexpr int kAmgDenseRows = 1536;
+// Planar FP64 meshes up to this size get the inverse of the matrix itself (dense_inverse.cu): 4,608
+// rows are 85 MB in FP32, which stay in the 129 MB L2 from one product to the next.
+constexpr int kInverseRows = 4608;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
-// composite operators of every non-coarsest level.  mixed: for a mixed-precision handle, whose
-// solves keep one arithmetic (block_group_sum in grid_sync.cuh): no direct inverse of small meshes.
-int amg_setup(const HostMesh& m, bool mixed, AmgHost& out, char* err, size_t errlen);
+// composite operators of every non-coarsest level.
+int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen);
 
 // SELL-32 form of a CSR matrix with `lpr` lanes per row (1, 2, 4, 8, 16 or 32): a slice holds
 // 32 / lpr consecutive rows; step k of a slice is 32 contiguous elements, entries k*lpr ..
@@ -119,7 +121,7 @@ void sell_from_csr(const Csr& A, SellHost& out, int lpr = 1);
 // at most 8 stored entries per lane on an average row, or fewer lanes when that gives a slice to
 // every warp of the whole-GPU solvers already (a row's epilogue runs on one of its lanes only, and
 // the finest level's has FP64 operations).
-// `mixed` (see amg_setup): always the former.
+// `mixed`: always the former (the mixed-precision solves keep one arithmetic, see block_group_sum).
 int lanes_per_row(const Csr& A, bool mixed);
 // Elements a streamed array must be readable past its end (a ring slot is always filled).
 constexpr size_t kStreamPad = 16 * kSlice;
@@ -176,9 +178,10 @@ template <typename T>
 struct AmgDevT {
   int32_t nlev;         // levels including the coarsest
   int32_t pad;
-  // dense[0]: the V-cycle from the finest level of at most kAmgDenseRows rows down, as one
-  // matrix; dense[1]: the inverse of the coarsest matrix (solvers on few SMs, see dense_choice)
-  AmgDenseT<T> dense[2];
+  // dense[0]: the inverse of the finest matrix (small planar meshes, dense_inverse.cu; null
+  // otherwise); dense[1]: the V-cycle from the finest level of at most kAmgDenseRows rows down, as
+  // one matrix; dense[2]: the inverse of the coarsest matrix (see dense_choice)
+  AmgDenseT<T> dense[3];
   AmgLevelT<T> L[kAmgMaxLevels];
 };
 using AmgLevelDev = AmgLevelT<double>;
@@ -326,7 +329,7 @@ struct PcgPlan {
 PcgPlan pcg_plan(int nslices, int kind, int requested_tpb);
 PcgPlan pcg_mixed_plan(int nslices, int requested_tpb);
 PcgPlan bicgstab_plan(int nslices, int requested_tpb);
-PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64);  // kind 8 (CG), 9 (BiCGStab), 10 (mixed)
+PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64, int inverse_rows = 0);  // kind 8 (CG), 9 (BiCGStab), 10 (mixed)
 PcgPlan amg_cluster_plan(int want, int n);  // kind 11 for n rows (one cluster of `want` CTAs or 16 / 8; kind 0 if none fits)
 
 // Cluster-resident solve (kind 5): rows, halo and matrix slices per CTA of the cluster.

@@ -485,11 +485,13 @@ static const void* amg_kernel_ptr(int kind, int tpb, int fp64) {
 }
 
 // Grid: co-resident blocks (one per SM), no more than the finest level needs.
-PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64) {
+// inverse_rows > 0: the preconditioner is a dense inverse of that many rows; then the whole GPU, with
+// 1,024 threads where 768 would give some warps two rows and others one.
+PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64, int inverse_rows) {
   PcgPlan pl;
   pl.kind = kind;
   pl.maxs = fp64;  // FP64 hierarchy (1) or FP32 (0)
-  pl.tpb = amg_default_threads(kind, fp64);
+  pl.tpb = inverse_rows > 152 * 24 ? 1024 : amg_default_threads(kind, fp64);
   for (int t : kAmgSizes)
     if (t == requested_tpb) pl.tpb = t;
   int dev = 0, sms = 0, occ = 0;
@@ -501,7 +503,7 @@ PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64) {
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, pl.tpb, smem);
   // (the mixed-precision form keeps the partition of its FP32 sums: a slice per warp)
   const int per_block = kind == 10 ? pl.tpb / kSlice : kSlicesPerBlock;
-  const int want = (nslices + per_block - 1) / per_block;
+  const int want = inverse_rows > 0 ? (inverse_rows + 7) / 8 : (nslices + per_block - 1) / per_block;
   pl.blocks = std::max(1, std::min(std::max(occ, 1) * std::max(sms, 1), want));
   return pl;
 }

@@ -52,9 +52,12 @@ def estimate_bytes(problem) -> int:
 
 
 def solver_kind(problem) -> int:
-    """pcg_kind for a served request: the AMG solve on one cluster (11) for the mid-size meshes
-    the library would give the whole GPU, the library's choice (0) otherwise."""
-    return 11 if AUTO_CLUSTER_NODES < problem.n_nodes <= SHARED_MAX_NODES else 0
+    """pcg_kind for a served request: the AMG solve on one cluster (11) for the planar meshes up to
+    SHARED_MAX_NODES, some of which the library would give the whole GPU, the library's choice (0)
+    otherwise."""
+    if getattr(problem, "axisymmetric", False):
+        return 0
+    return 11 if problem.n_nodes <= SHARED_MAX_NODES else 0
 
 
 def cluster_ctas(problem) -> int:
