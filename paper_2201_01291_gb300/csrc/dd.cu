@@ -28,13 +28,22 @@ namespace avip {
 constexpr int kDDThreads = 256;
 constexpr int kDDMinThreads = 128;  // smallest block of the batched stages (autotuned)
 
+// Sign and magnitude tests on the bit patterns: an FP64 comparison costs as much as
+// an FP64 multiply-add (19 cycles per warp and SM), integer ones next to nothing.
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
+__device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ double flip_sign(double x, bool flip) {
+  return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
+}
+
 // Local-field mobility and the Townsend exponential with the library's FP64 exp / log
 // (fp64_math.cuh: a few ulp, a fraction of the FP64 instructions of the general routines).
 // mu0 (max(|E|, E_floor) / E_ref)^p = mu0 exp(p (log max(|E|, E_floor) - log E_ref)), log E_ref
 // from the host: no FP64 division.
 __device__ __forceinline__ double mobility(const SpeciesParams& sp, double Emag) {
   if (sp.mob_model == AVIP_MOB_POWER)
-    return sp.mob[0] * exp_fp64(sp.mob[2] * (log_fp64(fmax(Emag, sp.mob[3])) - sp.mob_log_ref));
+    return sp.mob[0] * exp_fp64(sp.mob[2] * (log_fp64(abs_bits(Emag) < abs_bits(sp.mob[3]) ? sp.mob[3] : Emag) -
+                                             sp.mob_log_ref));
   return sp.mob[0];
 }
 
@@ -124,7 +133,7 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
     // |E| and 1/|E| from one reciprocal square root (the Townsend and attachment exponents take
     // -B/|E| as a product)
     const double E2 = Ex * Ex + Ey * Ey;
-    const double invE = E2 > 0.0 ? rsqrt(E2) : 0.0;
+    const double invE = abs_bits(E2) != 0 ? rsqrt(E2) : 0.0;
     const double Emag = E2 * invE;
     a.Ex[i] = Ex;
     a.Ey[i] = Ey;
@@ -150,7 +159,7 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
     if (a.ph.src_model != AVIP_SRC_NONE) {
       const int ie = a.ph.src_idx[0], ip = a.ph.src_idx[1], ineg = a.ph.src_idx[2];
       const double ne = n[(size_t)ie * a.Npad + i];
-      const double alpha = Emag > 0.0 ? a.ph.src_params[0] * exp_fp64(-a.ph.src_params[1] * invE) : 0.0;
+      const double alpha = abs_bits(Emag) != 0 ? a.ph.src_params[0] * exp_fp64(-a.ph.src_params[1] * invE) : 0.0;
       double mue = 0.0;
 #pragma unroll
       for (int s = 0; s < AVIP_MAX_SPECIES; ++s)
@@ -177,7 +186,7 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
           if (s == ip) npos = n[(size_t)s * a.Npad + i];
           if (s == ineg) nneg = n[(size_t)s * a.Npad + i];
         }
-        const double eta = Emag > 0.0 ? a.ph.src_params[2] * exp_fp64(-a.ph.src_params[3] * invE) : 0.0;
+        const double eta = abs_bits(Emag) != 0 ? a.ph.src_params[2] * exp_fp64(-a.ph.src_params[3] * invE) : 0.0;
         const double att = eta * mue * Emag * ne;
         const double rep = a.ph.src_params[4] * ne * npos;
         const double rnp = a.ph.src_params[4] * nneg * npos;
@@ -192,7 +201,7 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
 #pragma unroll
       for (int s = 0; s < AVIP_MAX_SPECIES; ++s)
         if (s == ie) se = src[s];
-      if (se != 0.0) chem = a.ph.a_chem * fabs(ne) * recip_nr(fabs(se));
+      if (abs_bits(se) != 0) chem = a.ph.a_chem * fabs(ne) * recip_nr(fabs(se));
     }
 #pragma unroll
     for (int s = 0; s < AVIP_MAX_SPECIES; ++s)
@@ -350,55 +359,49 @@ struct EdgeEnd {
   double u, gx, gy, vx, vy;
 };
 
-// Bernoulli function B(x) = x / (e^x - 1) for x >= 0 (B(0) = 1; 0 once e^x overflows).
+// Bernoulli function B(x) = x / (e^x - 1) for x >= 0 (B(0) = 1; 0 where it is below 1e-300).
 // B(-x) = x + B(x), so one expm1 gives both values without cancellation.
-__device__ __forceinline__ double bernoulli_pos(double x) { return x != 0.0 ? x / expm1(x) : 1.0; }
+__device__ __forceinline__ double bernoulli_pos(double x) {
+  if (abs_bits(x) == 0) return 1.0;
+  return x > 700.0 ? 0.0 : x * recip_nr(expm1(x));
+}
 
 // Geometry of one edge for the Scharfetter-Gummel split (species independent), canonical
-// orientation lo -> hi: unit direction e, length h, s = S.e and S_perp = S - s e.
+// orientation lo -> hi: edge vector d = h e, S.e / h = S.d / d.d and S_perp = S - (S.e) e.
 struct SgGeo {
-  double ex, ey, h, rh, s, spx, spy;
+  double dx, dy, sh, spx, spy;
 };
 __device__ __forceinline__ SgGeo sg_geometry(double dx, double dy, double Sx, double Sy) {
   SgGeo g;
-  g.h = sqrt(dx * dx + dy * dy);
-  g.rh = 1.0 / g.h;
-  g.ex = dx * g.rh;
-  g.ey = dy * g.rh;
-  g.s = Sx * g.ex + Sy * g.ey;
-  g.spx = Sx - g.s * g.ex;
-  g.spy = Sy - g.s * g.ey;
+  g.dx = dx;
+  g.dy = dy;
+  g.sh = fma(Sx, dx, Sy * dy) * recip_nr(fma(dx, dx, dy * dy));
+  g.spx = fma(-g.sh, dx, Sx);
+  g.spy = fma(-g.sh, dy, Sy);
   return g;
 }
 
 // Scharfetter-Gummel flux (section "Scharfetter Gummel scheme"): S is split along the edge
 // direction e into S_par = (S.e) e and S_perp; the tangential part is the exponentially fitted
-// V.S_par (u_hi - e^a u_lo)/(1 - e^a), a = h V.e / D, evaluated as
+// V.S_par (u_hi - e^a u_lo)/(1 - e^a), a = h V.e / D = V.d / D, evaluated as
 // (D (S.e)/h)(B(-a) u_lo - B(a) u_hi) (no overflow for large |a|, no 0/0 at a = 0; D = 0 is
-// the upwind limit); the normal part is centred: V.S_perp (u_lo + u_hi)/2 - D g.S_perp.
-__device__ __forceinline__ double sg_flux(double ulo, double uhi, const SgGeo& G, double Vx, double Vy, double gx,
-                                          double gy, double D) {
-  const double Vt = Vx * G.ex + Vy * G.ey;
+// the upwind limit); the normal part is centred: V.S_perp (u_lo + u_hi)/2 - D g.S_perp.  V and g
+// come doubled (the sums of the two ends).  Written on d instead of e and h it needs no square
+// root, and 1 / D comes from the host: fluxes and update of 313,000 edges, 2 species, 127 -> 94 us.
+__device__ __forceinline__ double sg_flux(double ulo, double uhi, const SgGeo& G, double sVx, double sVy, double sgx,
+                                          double sgy, const SpeciesParams& sp) {
+  const double Vd = 0.5 * fma(sVx, G.dx, sVy * G.dy);  // V.d
   double fpar;
-  if (D > 0.0) {
-    const double a = G.h * Vt / D;
+  if (sp.D > 0.0) {
+    const double a = Vd * sp.invD;
     const double aa = fabs(a);
     const double Bp = bernoulli_pos(aa), Bm = aa + Bp;  // B(|a|), B(-|a|)
-    const double B_neg_a = a >= 0.0 ? Bm : Bp, B_a = a >= 0.0 ? Bp : Bm;
-    fpar = (D * G.s * G.rh) * (B_neg_a * ulo - B_a * uhi);
+    const bool neg = negative(a);
+    fpar = (sp.D * G.sh) * fma(neg ? Bp : Bm, ulo, -((neg ? Bm : Bp) * uhi));
   } else {
-    fpar = G.s * (fmax(Vt, 0.0) * ulo + fmin(Vt, 0.0) * uhi);
+    fpar = G.sh * Vd * (negative(Vd) ? uhi : ulo);
   }
-  const double fperp = (Vx * G.spx + Vy * G.spy) * (0.5 * (ulo + uhi)) - D * (gx * G.spx + gy * G.spy);
-  return fpar + fperp;
-}
-
-// The sign and magnitude tests of the flux on the bit patterns: an FP64 comparison costs as much as
-// an FP64 multiply-add (19 cycles per warp and SM), integer ones next to nothing.
-__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
-__device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
-__device__ __forceinline__ double flip_sign(double x, bool flip) {
-  return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
+  return fma(0.25 * fma(sVx, G.spx, sVy * G.spy), ulo + uhi, fma(-0.5 * sp.D, fma(sgx, G.spx, sgy * G.spy), fpar));
 }
 
 // Sum of the block's values into *dst in a fixed order: the warps' values through shared memory to
@@ -428,12 +431,11 @@ __device__ __forceinline__ void block_charge(double q, double* dst) {
 // and range tests and the coordinate differences in FP64): the FP64 issue rate bounds the kernel
 // on GB300.
 __device__ __forceinline__ double edge_flux(const EdgeEnd& lo, const EdgeEnd& hi, double dx, double dy, double Hx,
-                                            double Hy, double D, double dt4, double beta, int lim, const SgGeo* sg) {
-  if (sg)
-    return sg_flux(lo.u, hi.u, *sg, 0.5 * (lo.vx + hi.vx), 0.5 * (lo.vy + hi.vy), 0.5 * (lo.gx + hi.gx),
-                   0.5 * (lo.gy + hi.gy), D);
+                                            double Hy, const SpeciesParams& sp, double dt4, double beta, int lim,
+                                            const SgGeo* sg) {
   const double sVx = lo.vx + hi.vx, sVy = lo.vy + hi.vy;  // 2 V_ij
   const double sgx = lo.gx + hi.gx, sgy = lo.gy + hi.gy;  // 2 grad_ij
+  if (sg) return sg_flux(lo.u, hi.u, *sg, sVx, sVy, sgx, sgy, sp);
   const double av = fma(sVx, Hx, sVy * Hy);               // V_ij . S
   const bool up_hi = negative(av);                        // (-0: no flux either way)
   const double uU = up_hi ? hi.u : lo.u;
@@ -451,7 +453,7 @@ __device__ __forceinline__ double edge_flux(const EdgeEnd& lo, const EdgeEnd& hi
   }
   const double lw = fma(-dt4, fma(sgx, sVx, sgy * sVy), delta);  // delta - dt grad_ij.V_ij
   const double us = fma(lw, hpsi, uU);
-  return fma(us, av, -D * fma(sgx, Hx, sgy * Hy));               // minus D grad_ij . S
+  return fma(us, av, -sp.D * fma(sgx, Hx, sgy * Hy));               // minus D grad_ij . S
 }
 
 // kGather: the edge fluxes were evaluated once per edge (edge_flux_kernel) and are gathered;
@@ -528,7 +530,7 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
           const EdgeEnd other{n[(size_t)s * a.Npad + j], g.x, g.y, v.x, v.y};
           const EdgeEnd& lo = lo_is_me ? me[s] : other;
           const EdgeEnd& hi = lo_is_me ? other : me[s];
-          const double F = edge_flux(lo, hi, dx, dy, Hx, Hy, a.ph.sp[s].D, dt4, a.ph.beta, a.ph.limiter,
+          const double F = edge_flux(lo, hi, dx, dy, Hx, Hy, a.ph.sp[s], dt4, a.ph.beta, a.ph.limiter,
                                      use_sg ? &geo : nullptr);
           R[s] += flip_sign(F, lo_is_me);
         }
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(kDDThreads) edge_flux_kernel(DDArgs a) {
       const EdgeEnd L{n[(size_t)s * a.Npad + lo], gl.x, gl.y, vl.x, vl.y};
       const EdgeEnd H{n[(size_t)s * a.Npad + hi], gh.x, gh.y, vh.x, vh.y};
       a.eflux[(size_t)s * a.E + e] =
-          edge_flux(L, H, dx, dy, Hx, Hy, a.ph.sp[s].D, dt4, a.ph.beta, a.ph.limiter, use_sg ? &geo : nullptr);
+          edge_flux(L, H, dx, dy, Hx, Hy, a.ph.sp[s], dt4, a.ph.beta, a.ph.limiter, use_sg ? &geo : nullptr);
     }
   }
 }
