@@ -1065,9 +1065,6 @@ int poisson_solve(avip_mesh_t h, int32_t* iters_out, double* relres_out) {
 static int run_impl(avip_mesh_t h, int32_t nsteps, double dt, avip_stats* stats, bool use_graph) {
   if (!ready(h)) return h ? AVIP_ESTATE : AVIP_EINVAL;
   if (nsteps < 0) return AVIP_EINVAL;
-  DevScalars s0;
-  int rc = read_scalars(h, s0);
-  if (rc) return rc;
   const double saved_dt = h->ph.dt_fixed;
   if (dt > 0.0) {
     if (h->ph.dt_fixed != dt) invalidate_graph(h);
@@ -1107,7 +1104,7 @@ static int run_impl(avip_mesh_t h, int32_t nsteps, double dt, avip_stats* stats,
   if (dt > 0.0 && saved_dt != dt) invalidate_graph(h);
   if (e != cudaSuccess) return cuda_status(e);
   DevScalars sc;
-  rc = read_scalars(h, sc);
+  const int rc = read_scalars(h, sc);
   if (rc) return rc;
   if (stats) {
     stats->steps = sc.run_steps;
@@ -1118,7 +1115,7 @@ static int run_impl(avip_mesh_t h, int32_t nsteps, double dt, avip_stats* stats,
     stats->dt_max = sc.run_dt_max;
     stats->t = sc.t;
     stats->charge = sc.charge;
-    stats->charge_start = s0.charge;
+    stats->charge_start = sc.charge_start;
     stats->relres_max = sc.run_relres_max;
   }
   if (sc.status == AVIP_ETIMEOUT) {
@@ -1145,9 +1142,6 @@ int run_steps_timed(avip_mesh_t h, int32_t nsteps, double* kernel_ms, avip_stats
   if (!ready(h)) return h ? AVIP_ESTATE : AVIP_EINVAL;
   if (nsteps < 0 || !kernel_ms) return AVIP_EINVAL;
   for (int k = 0; k < AVIP_TIMED_KERNELS; ++k) kernel_ms[k] = 0.0;
-  DevScalars s0;
-  int rc = read_scalars(h, s0);
-  if (rc) return rc;
   constexpr int kEv = 8;  // per step: 6 boundaries of the timed stages, 2 around photoionisation
   std::vector<cudaEvent_t> ev((size_t)nsteps * kEv, nullptr);
   cudaError_t e = cudaSuccess;
@@ -1196,7 +1190,7 @@ int run_steps_timed(avip_mesh_t h, int32_t nsteps, double* kernel_ms, avip_stats
     if (x) cudaEventDestroy(x);
   if (e != cudaSuccess) return cuda_status(e);
   DevScalars sc;
-  rc = read_scalars(h, sc);
+  const int rc = read_scalars(h, sc);
   if (rc) return rc;
   if (stats) {
     stats->steps = sc.run_steps;
@@ -1207,7 +1201,7 @@ int run_steps_timed(avip_mesh_t h, int32_t nsteps, double* kernel_ms, avip_stats
     stats->dt_max = sc.run_dt_max;
     stats->t = sc.t;
     stats->charge = sc.charge;
-    stats->charge_start = s0.charge;
+    stats->charge_start = sc.charge_start;
     stats->relres_max = sc.run_relres_max;
   }
   return sc.status;
@@ -1682,11 +1676,6 @@ int batch_set_dd_threads(avip_batch_t b, int32_t threads) {
 int batch_run_steps(avip_batch_t b, int32_t nsteps, avip_stats* stats) {
   if (!b || nsteps < 0) return AVIP_EINVAL;
   const int n = (int)b->m.size();
-  std::vector<DevScalars> s0(n);
-  for (int k = 0; k < n; ++k) {
-    cudaError_t e = cudaMemcpyAsync(&s0[k], b->m[k]->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, b->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-  }
   cudaError_t e = launch_run_reset_batch(b->d_dargs, n, b->stream);
   if (e == cudaSuccess && !b->graph && nsteps > 1) {
     cudaGraph_t g = nullptr;
@@ -1723,7 +1712,7 @@ int batch_run_steps(avip_batch_t b, int32_t nsteps, avip_stats* stats) {
       stats[k].dt_max = sc[k].run_dt_max;
       stats[k].t = sc[k].t;
       stats[k].charge = sc[k].charge;
-      stats[k].charge_start = s0[k].charge;
+      stats[k].charge_start = sc[k].charge_start;
       stats[k].relres_max = sc[k].run_relres_max;
     }
     if (status == AVIP_OK && sc[k].status != AVIP_OK) status = sc[k].status;

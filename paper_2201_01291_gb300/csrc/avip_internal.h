@@ -243,6 +243,7 @@ struct DevScalars {
   int32_t pcg_outer;            // refinement steps of the last mixed-precision solve
   int32_t phi_hist;             // earlier potentials kept for the predictor (0 .. 3)
   double run_dt_min, run_dt_max, run_relres_max;
+  double charge_start;          // Q when the current run began
 };
 
 // Jacobi-PCG is run on the symmetrically scaled system

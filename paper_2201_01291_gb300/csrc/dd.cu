@@ -659,6 +659,7 @@ __global__ void finalize_kernel(DevScalars* sc, const double* partials, int npar
 }
 
 __global__ void run_reset_kernel(DevScalars* sc) {
+  sc->charge_start = sc->charge;
   sc->run_steps = 0;
   sc->run_iters_total = 0;
   sc->run_iters_max = 0;
@@ -966,6 +967,7 @@ __global__ void run_reset_batch_kernel(const DDArgs* __restrict__ args, int coun
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   DevScalars* sc = args[k].sc;
+  sc->charge_start = sc->charge;
   sc->run_steps = 0;
   sc->run_iters_total = 0;
   sc->run_iters_max = 0;
