@@ -210,7 +210,14 @@ __device__ __forceinline__ void node_fields_body(const DDArgs& a, int with_dt, i
   if (with_dt) block_min_to_global(chem, &a.sc->dt_bits);
 }
 
+// The kernels of a single-instance step are launched with programmatic stream serialisation: each is
+// put on the SMs while its predecessor drains and waits here, before it reads anything, until the
+// predecessor has completed and its writes are visible.  Hides the launch of four of the step's
+// kernels, which dominate it on small meshes.
+__device__ __forceinline__ void after_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __global__ void __launch_bounds__(kDDThreads, 3) node_fields_kernel(DDArgs a, int with_dt) {
+  after_predecessor();
   node_fields_body(a, with_dt, blockIdx.x);
 }
 
@@ -352,7 +359,10 @@ __device__ __forceinline__ void dt_cells_body(const DDArgs& a, int bid, int nblo
   }
 }
 
-__global__ void __launch_bounds__(kDDThreads) dt_cells_kernel(DDArgs a) { dt_cells_body(a, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(kDDThreads) dt_cells_kernel(DDArgs a) {
+  after_predecessor();
+  dt_cells_body(a, blockIdx.x, gridDim.x);
+}
 
 // ------------------------------------------------------------------------ fluxes + update
 struct EdgeEnd {
@@ -571,6 +581,7 @@ __device__ __forceinline__ void flux_update_body_t(const DDArgs& a, int bid) {
 
 template <bool kGather>
 __global__ void __launch_bounds__(kDDThreads, kGather ? 3 : 2) flux_update_kernel(DDArgs a) {
+  after_predecessor();
   flux_update_body_t<kGather>(a, blockIdx.x);
 }
 
@@ -578,6 +589,7 @@ __global__ void __launch_bounds__(kDDThreads, kGather ? 3 : 2) flux_update_kerne
 // face, the same function of the same operands as in flux_update_body's per-row evaluation, so
 // both ends receive identical values.
 __global__ void __launch_bounds__(kDDThreads) edge_flux_kernel(DDArgs a) {
+  after_predecessor();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= a.E) return;
   const int ns = a.ph.ns;
@@ -655,6 +667,7 @@ __global__ void __launch_bounds__(kDDThreads) photo_add_kernel(DDArgs a, int wit
 }
 
 __global__ void finalize_kernel(DevScalars* sc, const double* partials, int nparts) {
+  after_predecessor();
   finalize_body(sc, partials, nparts);
 }
 
@@ -802,6 +815,7 @@ __device__ __forceinline__ void node_fields32_body(const DDArgs& a, int with_dt,
 }
 
 __global__ void __launch_bounds__(kDDThreads) node_fields32_kernel(DDArgs a, int with_dt) {
+  after_predecessor();
   node_fields32_body(a, with_dt, blockIdx.x);
 }
 
@@ -919,7 +933,10 @@ __device__ __forceinline__ void flux_update32_body(const DDArgs& a, int bid) {
   if (bid == 0 && threadIdx.x == 0) a.sc->dt = dt;
 }
 
-__global__ void __launch_bounds__(kDDThreads, 3) flux_update32_kernel(DDArgs a) { flux_update32_body(a, blockIdx.x); }
+__global__ void __launch_bounds__(kDDThreads, 3) flux_update32_kernel(DDArgs a) {
+  after_predecessor();
+  flux_update32_body(a, blockIdx.x);
+}
 
 // ------------------------------------------------------------------------ batched forms
 // One launch covers every instance of a batch: block b belongs to the instance k with
@@ -980,12 +997,23 @@ __global__ void run_reset_batch_kernel(const DDArgs* __restrict__ args, int coun
 // ------------------------------------------------------------------------ host launchers
 static inline int nblk(int n) { return (n + kDDThreads - 1) / kDDThreads; }
 
+// Launch with programmatic stream serialisation (see after_predecessor).
+template <typename... P, typename... A>
+static cudaError_t launch_after(void (*kernel)(P...), int blocks, int threads, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 cudaError_t launch_node_fields(const DDArgs& a, int with_dt, cudaStream_t st) {
-  if (a.ph.dd_fp32)
-    node_fields32_kernel<<<nblk(a.A.N), kDDThreads, 0, st>>>(a, with_dt);
-  else
-    node_fields_kernel<<<nblk(a.A.N), kDDThreads, 0, st>>>(a, with_dt);
-  return cudaGetLastError();
+  return launch_after(a.ph.dd_fp32 ? node_fields32_kernel : node_fields_kernel, nblk(a.A.N), kDDThreads, st, a, with_dt);
 }
 cudaError_t launch_photo_add(const DDArgs& a, int with_dt, cudaStream_t st) {
   photo_add_kernel<<<nblk(a.A.N), kDDThreads, 0, st>>>(a, with_dt);
@@ -1000,25 +1028,16 @@ int dt_cells_blocks(int cells, int threads) {
 }
 cudaError_t launch_dt_cells(const DDArgs& a, cudaStream_t st) {
   const int blocks = dt_cells_blocks(a.T, kDDThreads);
-  dt_cells_kernel<<<blocks, kDDThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_after(dt_cells_kernel, blocks, kDDThreads, st, a);
 }
 cudaError_t launch_flux_update(const DDArgs& a, cudaStream_t st) {
-  if (a.ph.dd_fp32) {
-    flux_update32_kernel<<<nblk(a.A.N), kDDThreads, 0, st>>>(a);
-  } else {
-    if (a.eflux && a.E > 0) {
-      edge_flux_kernel<<<nblk(a.E), kDDThreads, 0, st>>>(a);
-      flux_update_kernel<true><<<nblk(a.A.N), kDDThreads, 0, st>>>(a);
-    } else {
-      flux_update_kernel<false><<<nblk(a.A.N), kDDThreads, 0, st>>>(a);
-    }
-  }
-  return cudaGetLastError();
+  if (a.ph.dd_fp32) return launch_after(flux_update32_kernel, nblk(a.A.N), kDDThreads, st, a);
+  if (!(a.eflux && a.E > 0)) return launch_after(flux_update_kernel<false>, nblk(a.A.N), kDDThreads, st, a);
+  const cudaError_t e = launch_after(edge_flux_kernel, nblk(a.E), kDDThreads, st, a);
+  return e != cudaSuccess ? e : launch_after(flux_update_kernel<true>, nblk(a.A.N), kDDThreads, st, a);
 }
 cudaError_t launch_finalize(DevScalars* sc, const double* partials, int nparts, cudaStream_t st) {
-  finalize_kernel<<<1, 256, 0, st>>>(sc, partials, nparts);
-  return cudaGetLastError();
+  return launch_after(finalize_kernel, 1, 256, st, sc, partials, nparts);
 }
 cudaError_t launch_run_reset(DevScalars* sc, cudaStream_t st) {
   run_reset_kernel<<<1, 1, 0, st>>>(sc);
