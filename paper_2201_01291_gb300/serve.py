@@ -8,9 +8,8 @@ yet.  The request then keeps its whole state resident on the device (one mesh ha
 own CUDA stream) until its last step, and releases slot and memory when done, which admits the
 requests waiting behind it.  Admitted requests advance in chunks of steps on worker threads;
 the CUDA work of concurrent requests overlaps on the device: every request of up to
-SHARED_MAX_NODES nodes solves its Poisson problem on one thread-block cluster (the Jacobi or
-AMG-preconditioned cluster solvers, 16 CTAs for the AMG ones), so up to nine of them run side by
-side on the 152 SMs.
+SHARED_MAX_NODES nodes solves its Poisson problem on one thread-block cluster (the cluster
+solvers, 16 CTAs for the AMG-preconditioned ones), so up to nine of them run side by side on the 152 SMs.
 Larger requests use the whole-GPU cooperative kernel and run their chunks exclusively, because
 a cooperative launch must have its whole grid resident.
 
@@ -38,7 +37,8 @@ from . import avip
 BYTES_PER_NODE = 1400
 BYTES_PER_TRI = 24
 SHARED_MAX_NODES = 300000  # requests up to this size solve on one thread-block cluster (shared)
-AUTO_CLUSTER_NODES = 20000  # below this the library's automatic choice is already a cluster solver
+AUTO_CLUSTER_NODES = 20000  # up to this the library's automatic choice is a cluster solver (mixed)
+AUTO_CLUSTER_NODES_FP64 = 1200  # FP64: above it the inverse of the matrix takes the whole GPU
 CLUSTER_KINDS = (5, 6, 11)  # solver kinds that occupy one thread-block cluster, not the whole GPU
 FREE_MARGIN = 512 << 20  # device memory kept free for the CUDA runtime and the caching allocator
 # CTAs of a served request's cluster, by size.  On the 100-request sample of the served
@@ -51,13 +51,13 @@ def estimate_bytes(problem) -> int:
     return int(problem.n_nodes * BYTES_PER_NODE + problem.n_tris * BYTES_PER_TRI) + (1 << 20)
 
 
-def solver_kind(problem) -> int:
-    """pcg_kind for a served request: the AMG solve on one cluster (11) for the planar meshes up to
-    SHARED_MAX_NODES, some of which the library would give the whole GPU, the library's choice (0)
-    otherwise."""
+def solver_kind(problem, precision: int = avip.PREC_MIXED) -> int:
+    """pcg_kind for a served request: the AMG solve on one cluster (11) for the planar meshes the
+    library would give the whole GPU, up to SHARED_MAX_NODES, the library's choice (0) otherwise."""
     if getattr(problem, "axisymmetric", False):
         return 0
-    return 11 if problem.n_nodes <= SHARED_MAX_NODES else 0
+    auto = AUTO_CLUSTER_NODES if precision == avip.PREC_MIXED else AUTO_CLUSTER_NODES_FP64
+    return 11 if auto < problem.n_nodes <= SHARED_MAX_NODES else 0
 
 
 def cluster_ctas(problem) -> int:
@@ -144,7 +144,7 @@ class Server:
     def _work(self, req: Request, t0: float, release, built):
         m = None
         try:
-            m = avip.Mesh(req.problem, rtol=self.rtol, pcg_kind=solver_kind(req.problem),
+            m = avip.Mesh(req.problem, rtol=self.rtol, pcg_kind=solver_kind(req.problem, self.precision),
                           cluster_size=self.cluster_size(req.problem), precision=self.precision)
             built()  # the handle's memory is now part of what the device reports as used
             # cluster-resident solves share the GPU; whole-GPU cooperative solves run exclusively
