@@ -7,8 +7,8 @@
  *      boundaries (section "Integrating the Poisson equation", Eq. poisson, Eq.
  *      poisson_discretization_cartesian, Eq. coeff_matriceA, "Boundary conditions"),
  *      solved on the device by conjugate gradients preconditioned by a smoothed-aggregation
- *      AMG V-cycle (planar meshes above 500 nodes; Jacobi-preconditioned CG below, and as an
- *      option), or by BiCGStab for the non-symmetric axisymmetric matrix (the paper names no
+ *      AMG V-cycle or, on small planar FP64 meshes (up to 4,608 nodes), by the inverse of the
+ *      matrix (Jacobi-preconditioned CG as an option), or by BiCGStab for the non-symmetric axisymmetric matrix (the paper names no
  *      linear solver);
  *   2. E = -grad(phi) with Green-Gauss cell gradients through nodal normals;
  *   3. edge-based limited Lax-Wendroff + central diffusion fluxes of every charged species
@@ -107,15 +107,18 @@ typedef struct avip_opts {
   double dt_fixed;                     /* > 0: use this time step instead of the automatic one */
   double inner_rtol;                   /* mixed precision: FP32 inner reduction per refinement */
   int32_t pcg_threads;                 /* solver block size (256/512/768/1024; 0 = the kind's default:
-                                          768, 1024 for the AMG-preconditioned CG) */
+                                          768; 512 for one cluster up to 20,000 nodes) */
   int32_t pcg_kind;                    /* solver kernel: 0 auto, 1 streaming, 2 register-resident,
                                           5 cluster, 7 BiCGStab (the only one for AXISYMMETRIC),
                                           8 CG preconditioned by an AMG V-cycle (auto for planar
-                                          FP64 meshes above 20,000 nodes), 9 BiCGStab
-                                          preconditioned by it (auto for AXISYMMETRIC meshes
-                                          above 20,000 nodes), 10 the mixed-precision form of
-                                          8, 11 the AMG solve on one thread-block cluster (auto
-                                          for planar meshes of 501 to 20,000 nodes) */
+                                          FP64 meshes above 20,000 nodes; of 1,201 to 4,608
+                                          nodes with the matrix's inverse in its place),
+                                          9 BiCGStab preconditioned by it (auto for
+                                          AXISYMMETRIC meshes above 3,000 nodes, 7 below),
+                                          10 the mixed-precision form of 8, 11 the AMG solve on
+                                          one thread-block cluster (auto for planar meshes up
+                                          to 20,000 nodes: with the inverse up to 1,200, FP64;
+                                          in mixed precision from 501 nodes on, 6 below) */
   void* stream;                        /* cudaStream_t for all work; NULL = default stream    */
   avip_alloc_fn alloc;                 /* optional device allocator (both or neither)         */
   avip_free_fn free;

@@ -694,24 +694,23 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     delete h;
     return AVIP_ENOMEM;
   }
-  // persistent PCG grid: co-resident blocks, but no more than there are slices to share
   // persistent PCG grid (co-resident blocks): register-resident kernel when the mesh fits
   h->plan = h->opts.precision == AVIP_PREC_MIXED ? pcg_mixed_plan(m.nslices, h->opts.pcg_threads)
                                                  : pcg_plan(m.nslices, h->opts.pcg_kind, h->opts.pcg_threads);
   const bool bicg = axi || h->opts.pcg_kind == 7 || h->opts.pcg_kind == 9;
   // small and mid-size planar meshes (or kind 11 forced): the AMG-preconditioned solve on one
-  // cluster.  Below a few hundred nodes its hierarchy is the inverse of the matrix alone, and two
-  // or three iterations replace the 70 to 90 of the Jacobi form.
+  // cluster
   PcgPlan amg_cluster;
   amg_cluster.kind = 0;
   const bool fp64 = h->opts.precision == AVIP_PREC_FP64;
-  // the inverse of the matrix as the preconditioner (dense_inverse.cu)
+  // the inverse of the matrix as the preconditioner (dense_inverse.cu): one to three iterations
+  // replace the V-cycle's 8 to 9, or the 70 to 90 of the Jacobi form
   const bool inverse = !bicg && h->opts.pcg_kind == 0 && fp64 && !h->opts.precond_fp64 && m.N <= kInverseRows;
   if (!bicg && (h->opts.pcg_kind == 11 ||
                 (h->opts.pcg_kind == 0 && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
                  (fp64 || m.N > kClusterMixedMinRows))))
     amg_cluster = amg_cluster_plan(h->opts.cluster_size, m.N);
-  // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above the cluster size
+  // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above kBicgstabAmgRows
   const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (h->opts.pcg_kind == 0 && m.N > kBicgstabAmgRows));
   if (bicg) {
     h->plan = bicgstab_plan(m.nslices, h->opts.pcg_threads);

@@ -34,11 +34,11 @@
 namespace avip {
 
 namespace {
-// Block sizes (one block per SM).  Default: 1024 threads for CG with the FP32 hierarchy (kind
-// 8: 99.9 us per CG iteration on the pin-plane solve against 104.8 at 768), 768 otherwise
-// (BiCGStab and the mixed form are 1 % faster at 768; the FP64 hierarchy spills at 1024)
+// Block sizes (one block per SM).  768 threads by default: 80 registers hold every form without
+// spills, and the rings keep the loads in flight whatever the number of warps (CG on the pin-plane
+// mesh of 500,000 nodes: 85.8 us per iteration at 768, 98.6 at 1024, 101.8 at 512).
 constexpr int kAmgSizes[] = {768, 512, 1024};
-int amg_default_threads(int kind, int fp64) { return 768; }
+constexpr int kAmgThreads = 768;
 constexpr int kAmgMaxRestarts = 8;
 // Fewest slices (of 32 rows) worth a block of their own: the whole GPU from 1,216 slices (39,000
 // rows) on.
@@ -46,8 +46,10 @@ constexpr int kSlicesPerBlock = 4;
 
 }  // namespace
 
-// Slots of a warp's ring (stream.cuh): 192 KB per block for the CG and mixed forms, at most 160 KB
-// for BiCGStab, whose four-value sums take 32 KB of shared memory.
+// Slots of a warp's ring (stream.cuh): 144 KB per block for the CG and mixed forms (3 slots of 2 KB
+// per warp at 768 threads: 22 MB in flight over the GPU, several times what the HBM latency needs),
+// which leaves more of the SM's 256 KB to L1, where the gathers hit (96, 144 and 192 KB measure
+// within 1 %); 160 KB for BiCGStab.
 constexpr int ring_slots(int tpb, bool bicg) {
   return (bicg ? 160 : 144) * 1024 / (tpb / 32 * kSlotBytes);
 }
@@ -491,7 +493,7 @@ PcgPlan amg_plan(int nslices, int requested_tpb, int kind, int fp64, int inverse
   PcgPlan pl;
   pl.kind = kind;
   pl.maxs = fp64;  // FP64 hierarchy (1) or FP32 (0)
-  pl.tpb = inverse_rows > 152 * 24 ? 1024 : amg_default_threads(kind, fp64);
+  pl.tpb = inverse_rows > 152 * 24 ? 1024 : kAmgThreads;
   for (int t : kAmgSizes)
     if (t == requested_tpb) pl.tpb = t;
   int dev = 0, sms = 0, occ = 0;

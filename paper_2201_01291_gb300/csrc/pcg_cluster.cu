@@ -780,8 +780,8 @@ cudaError_t launch_pcg_cluster(const PcgArgs& args, const PcgPlan& pl, const Clu
 // whose solve is too short to occupy the whole GPU (FP64 CG with an FP32 or FP64 hierarchy, or
 // the mixed-precision solve).  Other work, such as other requests of a server, can run beside it.
 // 512 threads per CTA for small meshes, 768 above kAmgClusterWideRows rows (measured on one
-// 16-CTA cluster: 150k nodes 218 -> 185 us per CG iteration, mixed 188 -> 155; 4k nodes 26.3 ->
-// 28.5, so small meshes keep 512).
+// 16-CTA cluster before the products went through the rings: 150k nodes 218 -> 185 us per CG
+// iteration, mixed 188 -> 155; 4k nodes 26.3 -> 28.5, so small meshes keep 512).
 constexpr int kAmgClusterWideRows = 20000;
 template <int TPB>
 __global__ void __launch_bounds__(TPB, 1) pcg_amg_cluster_kernel(PcgArgs a) {
