@@ -219,6 +219,7 @@ KERNEL_NAMES = {1: "pcg_fp64_kernel (streaming)", 2: "pcg_fp64_res_kernel (regis
                 9: "bicgstab_amg_kernel (BiCGStab + AMG V-cycle, axisymmetric)",
                 10: "pcg_amg_mixed_kernel (FP32 CG + FP32 AMG V-cycle, FP64 refinement)",
                 11: "pcg_amg_cluster_kernel (AMG-preconditioned CG on one cluster)"}
+INVERSE_NODES = 4608  # planar FP64 meshes up to this size: the inverse of the matrix as the preconditioner
 
 # DRAM bytes per solver iteration measured by ncu on the pin-plane 500 x 1000 workload (the
 # counters of one captured launch divided by its iterations), keyed by solver kind; valid for the
@@ -227,9 +228,8 @@ NCU_DRAM_BYTES_PER_ITER = {
     # pcg_fp64_res_kernel: 300-iteration capture, L2-resident working set
     2: ((72.372224e6 + 2.023936e6) / 300.0, "ncu DRAM read+write of a 300-iteration capture scaled to the "
                                             "launch's iterations (L2-resident working set)"),
-    # pcg_amg_kernel<1024, float>: one 21-iteration solve (two-phase V-cycle, Jacobi smoother,
-    # spill-free streams)
-    8: ((3574.051e6 + 28.363e6) / 21.0, "ncu DRAM read+write of a 21-iteration solve scaled to the launch's "
+    # pcg_amg_kernel<768, float>: one 21-iteration solve (two-phase V-cycle, operators through the rings)
+    8: ((3840.931e6 + 13.555e6) / 21.0, "ncu DRAM read+write of a 21-iteration solve scaled to the launch's "
                                         "iterations (profiles/pcg_amg_kernel_pin_plane_500x1000.md)"),
 }
 
@@ -403,6 +403,10 @@ def run_ours(args, rank, world, local_rank):
     # ---- roofline of the dominant kernel (PCG)
     peaks = measured_peaks()
     kernel_name = KERNEL_NAMES.get(info["pcg_kind"], str(info["pcg_kind"]))
+    if (args.precision == "fp64" and not args.precond_fp64 and args.pcg_kind == 0 and info["pcg_kind"] in (8, 11)
+            and info["n_nodes"] <= INVERSE_NODES):
+        info["levels"] = info["levels"][:1]  # the inverse of the matrix takes the place of the V-cycle
+        kernel_name += ", preconditioned by the inverse of the matrix"
     if info["pcg_kind"] == 11:  # the one-cluster AMG solve moves the bytes of kind 8 or 10
         info = dict(info, pcg_kind=10 if args.precision == "mixed" else 8)
     byts, flops = pcg_traffic_model(info, iters, args.steps)
@@ -495,7 +499,7 @@ def run_batch(args, rank, world, local_rank):
     probs = W.random_instances(args.instances, seed=4 + 1000 * rank)
     prec = avip.PREC_MIXED if args.precision == "mixed" else avip.PREC_FP64
     # instances above 2,000 nodes solve with the cluster form of the AMG-preconditioned CG (kind 8,
-    # or kind 10 in mixed precision); the smaller ones with the shared-memory Jacobi-PCG
+    # or kind 10 in mixed precision); the smaller ones with the library's choice
     meshes = [avip.Mesh(p, rtol=args.rtol, precision=prec,
                         pcg_kind=(8 if prec == avip.PREC_FP64 else 10) if p.n_nodes > 2000 else 0) for p in probs]
     b = avip.Batch(meshes, cluster_size=0)
