@@ -555,9 +555,17 @@ int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
   H.dlev = (int32_t)H.lv.size() - 1;
   H.dmat = H.cinv;
   while (H.dlev > 0 && H.lv[H.dlev - 1].A.n <= kAmgDenseRows) {
+    const AmgHostLevel& L = H.lv[H.dlev - 1];
     std::vector<double> M;
-    dense_vcycle(H.lv[--H.dlev], H.dmat, M);
+    dense_vcycle(L, H.dmat, M);
+    // FP32 rounding of M, scaled by the level's diagonal, moves the spectrum of A M by about
+    // 2 sqrt(n) 2^-24 times its largest entry (on the diagonal): kept below 1/8, else the levels of
+    // this ill-conditioned matrix stay phases of their own
+    double top = 0.0;
+    for (int32_t i = 0; i < L.A.n; ++i) top = std::max(top, std::fabs(M[(size_t)i * L.A.n + i]) / L.dinv[i]);
+    if (!(top * 2.0 * std::sqrt((double)L.A.n) <= 0.125 * 16777216.0)) break;
     H.dmat.swap(M);
+    --H.dlev;
   }
   return AVIP_OK;
 }

@@ -44,7 +44,7 @@ cudaError_t launch_state_put(const StateArgs& s, cudaStream_t st);
 int flux_partials_max(int N);
 int dense_inverse_rows(int N);
 size_t dense_inverse_scratch(int N);
-cudaError_t launch_dense_inverse(const SellView& A, float* M, float* scratch, cudaStream_t st);
+cudaError_t launch_dense_inverse(const SellView& A, float* M, float* scratch, int* bad, cudaStream_t st);
 }  // namespace avip
 
 using namespace avip;
@@ -126,7 +126,9 @@ struct avip_mesh {
 namespace {
 
 thread_local char g_err[256];
-constexpr int kClusterMixedMinRows = 500;  // mixed precision: Jacobi-PCG on one cluster up to this size (kind 6)
+// Jacobi-PCG on one cluster up to this size (kind 6 in mixed precision; kind 5 in FP64 when the
+// inverse of the matrix is not usable)
+constexpr int kClusterJacobiRows = 500;
 // BiCGStab preconditioned by the AMG V-cycle above this many nodes, Jacobi-scaled below: at 10,201
 // nodes its two V-cycles per iteration replace 290 iterations per step by 8.5 (8.7 -> 0.42 ms)
 constexpr int kBicgstabAmgRows = 3000;
@@ -545,9 +547,24 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
   return ok;
 }
 
+// The FP32 inverse of the scaled matrix (dense_inverse.cu) in `inverse`, or null there when it is too
+// ill-conditioned for one; false if memory or a launch failed.
+bool build_inverse(avip_mesh* h, float*& inverse) {
+  const size_t np = (size_t)dense_inverse_rows(h->hm.N);
+  float *M = nullptr, *scratch = nullptr;
+  int *bad = nullptr, host_bad = 1;
+  if (!zalloc(h, M, np * np + kStreamPad) || !zalloc(h, scratch, dense_inverse_scratch(h->hm.N)) || !zalloc(h, bad, 1) ||
+      launch_dense_inverse(sell_view(h), M, scratch, bad, h->stream) != cudaSuccess ||
+      cudaMemcpyAsync(&host_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+      cudaStreamSynchronize(h->stream) != cudaSuccess)
+    return false;
+  inverse = host_bad ? nullptr : M;
+  return true;
+}
+
 // Upload the hierarchy in the handle's preconditioner precision (FP64 values when asked for and
 // the solve is not the mixed-precision one) with its preconditioned-residual vector.
-bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np, bool with_inverse = false) {
+bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np, float* inverse = nullptr) {
   if (!zalloc(h, h->colS, h->hm.col.size() + kStreamPad) ||
       launch_mark_slices(h->sl_ptr, h->hm.nslices, h->col, h->colS, h->stream) != cudaSuccess)
     return false;
@@ -555,14 +572,6 @@ bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np, bool with_inverse = f
   if (fp64) return upload_amg_t<double>(h, H, h->amg) && zalloc(h, h->amg_z, Np) && zalloc(h, h->r2, Np);
   // (the FP64 CG writes its preconditioned residual in FP64 whatever the hierarchy's type; the
   // mixed-precision solve keeps its own FP32 one)
-  float* inverse = nullptr;
-  if (with_inverse) {
-    const size_t np = (size_t)dense_inverse_rows(h->hm.N);
-    float* scratch = nullptr;
-    if (!zalloc(h, inverse, np * np + kStreamPad) || !zalloc(h, scratch, dense_inverse_scratch(h->hm.N)) ||
-        launch_dense_inverse(sell_view(h), inverse, scratch, h->stream) != cudaSuccess)
-      return false;
-  }
   return upload_amg_t<float>(h, H, h->amg32, true, inverse) && zalloc(h, h->z32, Np) && zalloc(h, h->amg_z, Np) &&
          zalloc(h, h->r2, Np) && zalloc(h, h->rq32, 3 * Np);
 }
@@ -705,17 +714,29 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   const bool fp64 = h->opts.precision == AVIP_PREC_FP64;
   // the inverse of the matrix as the preconditioner (dense_inverse.cu): one to three iterations
   // replace the V-cycle's 8 to 9, or the 70 to 90 of the Jacobi form
-  const bool inverse = !bicg && h->opts.pcg_kind == 0 && fp64 && !h->opts.precond_fp64 && m.N <= kInverseRows;
+  const bool automatic = h->opts.pcg_kind == 0;
+  float* inverse = nullptr;
+  if (!bicg && automatic && fp64 && !h->opts.precond_fp64 && m.N <= kInverseRows) ok = ok && build_inverse(h, inverse);
+  // the hierarchy, built here where the Jacobi form takes over if it cannot be
+  AmgHost H;
+  auto hierarchy = [&]() {
+    if (amg_setup(m, H, g_err, sizeof(g_err)) == AVIP_OK) return true;
+    H = AmgHost();
+    g_err[0] = 0;
+    return false;
+  };
+  if (inverse && m.N <= kClusterJacobiRows && !hierarchy()) inverse = nullptr;
   if (!bicg && (h->opts.pcg_kind == 11 ||
-                (h->opts.pcg_kind == 0 && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
-                 (fp64 || m.N > kClusterMixedMinRows))))
+                (automatic && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
+                 (inverse || m.N > kClusterJacobiRows))))
     amg_cluster = amg_cluster_plan(h->opts.cluster_size, m.N);
   // BiCGStab preconditioned by the AMG V-cycle: forced, or automatic above kBicgstabAmgRows
-  const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (h->opts.pcg_kind == 0 && m.N > kBicgstabAmgRows));
+  const bool bicg_amg = bicg && (h->opts.pcg_kind == 9 || (automatic && m.N > kBicgstabAmgRows &&
+                                                       (m.N > kClusterAutoRows || hierarchy())));
   if (bicg) {
     h->plan = bicgstab_plan(m.nslices, h->opts.pcg_threads);
     ok = ok && zalloc(h, h->bcg, (bicg_amg ? 5 : 3) * Np);
-  } else if ((h->opts.pcg_kind == 0 && amg_cluster.kind != 11 && !inverse) || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
+  } else if ((automatic && amg_cluster.kind != 11 && !inverse) || h->opts.pcg_kind == 5 || h->opts.pcg_kind == 6) {
     // small meshes: one thread-block cluster with everything in shared memory
     // (the Jacobi form, when asked for or when the AMG form below cannot be scheduled)
     const int mixed = h->opts.precision == AVIP_PREC_MIXED ? 1 : 0;
@@ -735,8 +756,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   if (bicg_amg || (!bicg && h->opts.precision == AVIP_PREC_FP64 &&
                    (h->opts.pcg_kind == 8 ||
                     (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
-    AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -764,8 +784,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // AMG V-cycle, FP64 iterative refinement of the residual
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
       (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
-    AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -776,8 +795,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
   }
   if (amg_cluster.kind == 11) {
-    AmgHost H;
-    int rc = amg_setup(m, H, g_err, sizeof(g_err));
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);

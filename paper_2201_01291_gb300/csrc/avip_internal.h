@@ -89,7 +89,8 @@ struct AmgHost {
   int32_t nc = 0;                // coarsest size
   std::vector<double> cinv;      // dense inverse of the coarsest matrix (row-major)
   // the V-cycle from level dlev down as one dense matrix (row-major; the coarsest inverse when
-  // dlev is the coarsest level), dlev the finest level of at most kAmgDenseRows rows
+  // dlev is the coarsest level), dlev the finest level of at most kAmgDenseRows rows (coarser where
+  // FP32 would not hold it)
   int32_t dlev = 0;
   std::vector<double> dmat;
 };

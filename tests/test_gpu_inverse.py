@@ -42,6 +42,31 @@ def test_direct_preconditioner_sizes(avip, nx, ny, kind):
         assert normwise(m2.density(s), n[s]) <= 1e-10
 
 
+@pytest.mark.parametrize("nx,ny,lx,kind", [(4, 100, 1e-4, 5), (25, 50, 3e-4, 11), (30, 45, 1e-3, 11)])
+def test_ill_conditioned_matrices_keep_their_solver(avip, nx, ny, lx, kind):
+    """Cells of aspect 50 and more between electrodes at the long ends: the FP32 inverse is
+    rejected (spectral bound above 1/2) and the solve converges as without it.  Error of the
+    scaled potential: at most the residual over the smallest eigenvalue (twice that, for the
+    rounding of the oracle's solution at these conditions)."""
+    rtol = 1e-10
+    p = W.plates_problem(nx, ny, lx, 1.0, 5e3, seed=nx + ny)
+    o = O.Oracle(p)
+    free = p.node_bc != 1
+    K = o.K.toarray()[free][:, free]
+    d = np.sqrt(np.diag(K))
+    phi = o.poisson(o.initial_state())
+    b = (K @ phi[free]) / d
+    A = K / np.outer(d, d)
+    M = np.linalg.inv(A.astype(np.float32)).astype(np.float64)
+    assert np.abs(A @ ((M + M.T) / 2) - np.eye(len(A))).sum(1).max() > 0.5
+    m = avip.Mesh(p, rtol=rtol)
+    assert m.info["pcg_kind"] == kind
+    it, rr = m.poisson_solve()
+    assert rr <= rtol
+    err = np.linalg.norm(d * (m.phi() - phi)[free])
+    assert err <= 2 * rtol * np.linalg.norm(b) / np.linalg.eigvalsh(A)[0]
+
+
 @pytest.mark.parametrize("quads,ns,seed", [(0.0, 2, 1), (0.0, 3, 2), (0.5, 2, 3), (1.0, 3, 4)])
 def test_time_step_screening(avip, quads, ns, seed):
     """The step equals the oracle's minimum with densities from 1e0 to 1e20, a few of them
