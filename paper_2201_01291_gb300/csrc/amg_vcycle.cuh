@@ -186,13 +186,27 @@ struct StoreOut {  // x_i = value
 };
 
 // The dense product x = M b of the phase dl, b given by src: every block first copies all of b to
-// shared memory (one load per thread), so that the product's inner loop has no memory latency.
+// shared memory, so that the product's inner loop has no memory latency.
 template <typename T, class Ops, class Src, class Out>
 __device__ __forceinline__ void amg_dense(const AmgCtx<T>& C, Ops& ops, Src src, Out out, int lane) {
   const int n = C.H->L[C.D.level].n, np = C.D.steps * kSlice;
-  for (int k = threadIdx.x; k < np; k += blockDim.x) C.rhs[k] = k < n ? src(k) : T(0);
+  for (int k0 = threadIdx.x; k0 < np; k0 += 4 * blockDim.x) {
+    T v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + q * blockDim.x;
+      v[q] = k < n ? src(k) : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + q * blockDim.x;
+      if (k < np) C.rhs[k] = v[q];
+    }
+  }
   __syncthreads();
-  stream_dense<T>(ops.ring, C.D.level, lane, C.rhs, out);
+  using P = decltype(out.begin(0));
+  stream_dense<T>(ops.ring, C.D.level, lane, C.rhs, [&out](int row) { return out.begin(row); },
+                  [&out](int row, T v, P p) { out.end(row, v, p); });
 }
 
 // The V-cycle below the finest level: down phases of levels 1 .. dl-1, the dense product, up
@@ -209,7 +223,7 @@ __device__ bool amg_inner(const AmgCtx<T>& C, Ops& ops, int gwarp, int nwarps, i
   {
     const T* __restrict__ cb = C.H->L[dl].b;
     T* __restrict__ cx = C.H->L[dl].x;
-    amg_dense(C, ops, [cb](int k) { return __ldca(cb + k); }, [cx](int row, T v) { cx[row] = v; }, lane);
+    amg_dense(C, ops, [cb](int k) { return __ldca(cb + k); }, StoreOut<T>{cx}, lane);
     if (!ops.barrier()) return false;
   }
   for (int l = dl - 1; l >= 1; --l) {
@@ -239,7 +253,7 @@ __device__ bool vcycle(const AmgCtx<T>& C, const TB* __restrict__ b0, TZ* __rest
     }
   } out{b0, z, &acc};
   if (C.D.level == 0) {
-    amg_dense(C, ops, src, [&](int row, T v) { out.end(row, v, out.begin(row)); }, lane);
+    amg_dense(C, ops, src, out, lane);
   } else {
     amg_down(C, ops, 0, src, NoHook(), gwarp, nwarps, lane);
     if (!ops.barrier()) return false;
@@ -439,8 +453,8 @@ __device__ bool amg_cg_solve(const PcgArgs& a, const AmgCtx<T>& C, double* __res
             }
           } out{rv, z, &acc};
           if (dl == 0) {
-            amg_dense(C, ops, [rv](int k) { return (T)__ldca(rv + k); },
-                      [&](int row, T v) { out.end(row, v, out.begin(row)); }, lane);
+            const T* __restrict__ tv = tc;  // r in the hierarchy's type
+            amg_dense(C, ops, [tv](int k) { return __ldca(tv + k); }, out, lane);
           } else {
             if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
             amg_up(C, ops, 0, out, lane);
@@ -699,8 +713,7 @@ __device__ bool amg_mixed_solve(const PcgArgs& a, const AmgCtx<float>& C, Ops& o
         } out{rc, z32, &acc};
         if (dl == 0) {
           const float* __restrict__ rv = rc;
-          amg_dense(C, ops, [rv](int k) { return __ldca(rv + k); },
-                    [&](int row, float v) { out.end(row, v, out.begin(row)); }, lane);
+          amg_dense(C, ops, [rv](int k) { return __ldca(rv + k); }, out, lane);
         } else {
           if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
           amg_up(C, ops, 0, out, lane);

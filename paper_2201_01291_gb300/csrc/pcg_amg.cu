@@ -270,17 +270,16 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
           continue;
         }
         // ---- the rest of s^ = M s, then P3: t = A s^
+        struct Out {
+          double* z;
+          __device__ NoPre begin(int) const { return NoPre(); }
+          __device__ void end(int i, T v, NoPre) const { z[i] = (double)v; }
+        } out{sh};
         if (dl == 0) {
           const double* __restrict__ svv = sv;
-          amg_dense(C, ops, [svv](int k) { return (T)__ldca(svv + k); }, [&](int row, T z) { sh[row] = (double)z; },
-                    lane);
+          amg_dense(C, ops, [svv](int k) { return (T)__ldca(svv + k); }, out, lane);
         } else {
           if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
-          struct Out {
-            double* z;
-            __device__ NoPre begin(int) const { return NoPre(); }
-            __device__ void end(int i, T v, NoPre) const { z[i] = (double)v; }
-          } out{sh};
           amg_up(C, ops, 0, out, lane);
         }
         if (!ops.barrier()) return false;

@@ -308,32 +308,67 @@ __device__ __forceinline__ void stream_rows(R& ring, int ph, int lane, G g, Begi
   ring.leave(ph);
 }
 
-// This warp's rows of the dense operator of phase ph: out(row, sum_k M[row, k] b[k]) on lane 0, b
-// (the whole right-hand side) in shared memory.
-template <typename T, class R, class Out>
-__device__ __forceinline__ void stream_dense(R& ring, int ph, int lane, const T* b, Out out) {
+// This warp's rows of the dense operator of phase ph: out(row, sum_k M[row, k] b[k], pre) on lane 0, b
+// (the whole right-hand side) in shared memory, pre = begin(row) evaluated when the row starts.  Rows
+// of at least a slot (the inverses of small matrices, the V-cycle's tail) take the slot's steps of
+// one row at a time, all loads before the sums; with a test of the row's end after every step the
+// loads of a step waited for the sums of the last one (65 x 65 nodes, 71 MB over the GPU: 75.4 ->
+// 65.4 us per solve of 1.34 iterations; 500,000 nodes, tail of 1,073 rows: 77.9 -> 76.4 us per
+// iteration).  Shorter rows, of which a slot holds several, keep that form.
+template <typename T, class R, class Begin, class Out>
+__device__ __forceinline__ void stream_dense(R& ring, int ph, int lane, const T* b, Begin begin, Out out) {
   const int nsteps = __shfl_sync(0xffffffffu, ring.ns, ph);
   if (nsteps == 0) return;
   int slot = ring.enter(ph, lane);
   constexpr int K = steps_per_slot<T, true>();
-  const int w = ring.tab[ph].lpr;
+  const int w = ring.tab[ph].lpr, nrows = ring.tab[ph].nslices;
   int row = __shfl_sync(0xffffffffu, ring.sa, ph), k = 0;
   T acc = T(0);
+  decltype(begin(0)) pre{};
+  if (lane == 0) pre = begin(row);
+  auto end_row = [&]() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+      out(row, acc, pre);
+      if (row + 1 < nrows) pre = begin(row + 1);
+    }
+    acc = T(0);
+    k = 0;
+    ++row;
+  };
 #pragma unroll 1
   for (int left = nsteps; left > 0; left -= K) {
     if (!ring.resident) ring.wait(slot);
     const T* vs = reinterpret_cast<const T*>(ring.buf + slot * kSlotBytes) + lane;
     const int cnt = min(K, left);
-#pragma unroll 4
-    for (int u = 0; u < cnt; ++u) {
-      acc = fma_t(vs[u * 32], b[k * 32 + lane], acc);
-      if (++k == w) {
+    if (w >= K) {
+#pragma unroll 1
+      for (int u = 0; u < cnt;) {
+        const int n = min(cnt - u, w - k);
+        const T *vp = vs + u * 32, *bp = b + k * 32 + lane;
+        if (n == K) {
+          T v[K], x[K];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) out(row, acc);
-        acc = T(0);
-        k = 0;
-        ++row;
+          for (int q = 0; q < K; ++q) {
+            v[q] = vp[q * 32];
+            x[q] = bp[q * 32];
+          }
+#pragma unroll
+          for (int q = 0; q < K; ++q) acc = fma_t(v[q], x[q], acc);
+        } else {
+#pragma unroll 4
+          for (int q = 0; q < n; ++q) acc = fma_t(vp[q * 32], bp[q * 32], acc);
+        }
+        u += n;
+        k += n;
+        if (k == w) end_row();
+      }
+    } else {
+#pragma unroll 4
+      for (int u = 0; u < cnt; ++u) {
+        acc = fma_t(vs[u * 32], b[k * 32 + lane], acc);
+        if (++k == w) end_row();
       }
     }
     slot = ring.advance(slot, lane);
