@@ -38,7 +38,9 @@ BYTES_PER_NODE = 1400
 BYTES_PER_TRI = 24
 SHARED_MAX_NODES = 300000  # requests up to this size solve on one thread-block cluster (shared)
 AUTO_CLUSTER_NODES = 20000  # up to this the library's automatic choice is a cluster solver (mixed)
-AUTO_CLUSTER_NODES_FP64 = 1200  # FP64: above it the inverse of the matrix takes the whole GPU
+# FP64: above this the library's automatic choice keeps an inverse of the matrix that estimate_bytes
+# does not count (4 bytes x nodes squared) and, from 1,201 nodes on, takes the whole GPU with it
+AUTO_CLUSTER_NODES_FP64 = 500
 CLUSTER_KINDS = (5, 6, 11)  # solver kinds that occupy one thread-block cluster, not the whole GPU
 FREE_MARGIN = 512 << 20  # device memory kept free for the CUDA runtime and the caching allocator
 # CTAs of a served request's cluster, by size.  On the 100-request sample of the served
@@ -53,7 +55,8 @@ def estimate_bytes(problem) -> int:
 
 def solver_kind(problem, precision: int = avip.PREC_MIXED) -> int:
     """pcg_kind for a served request: the AMG solve on one cluster (11) for the planar meshes the
-    library would give the whole GPU, up to SHARED_MAX_NODES, the library's choice (0) otherwise."""
+    library would give the whole GPU or an inverse, up to SHARED_MAX_NODES, the library's choice (0)
+    otherwise."""
     if getattr(problem, "axisymmetric", False):
         return 0
     auto = AUTO_CLUSTER_NODES if precision == avip.PREC_MIXED else AUTO_CLUSTER_NODES_FP64
