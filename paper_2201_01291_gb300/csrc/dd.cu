@@ -48,8 +48,19 @@ __device__ __forceinline__ double mobility(const SpeciesParams& sp, double Emag)
 }
 
 __device__ __forceinline__ double limiter(double r, double beta, int kind) {
-  if (kind == AVIP_LIM_VANLEER) return (r + fabs(r)) / (1.0 + fabs(r));
+  if (kind == AVIP_LIM_VANLEER) {
+    if (abs_bits(r) == 0x7ff0000000000000LL) return negative(r) ? 0.0 : 2.0;  // (an overflowed ratio)
+    return (r + fabs(r)) / (1.0 + fabs(r));
+  }
   return fmax(0.0, fmax(fmin(beta * r, 1.0), fmin(r, beta)));
+}
+
+// num / delta, delta != 0: through the Newton reciprocal, or the division where delta is subnormal.  An
+// explicit front that runs into a zero background decays through the subnormals, and 1 / delta
+// overflows below 2^-1024.
+__device__ __forceinline__ double slope_ratio(double num, double delta) {
+  if (abs_bits(delta) < 0x0010000000000000LL) return num / delta;
+  return num * recip_nr(delta);
 }
 
 // Smallest positive v of the block into *dst (the bits of positive doubles order like integers):
@@ -457,9 +468,9 @@ __device__ __forceinline__ double edge_flux(const EdgeEnd& lo, const EdgeEnd& hi
   const long long ad = abs_bits(delta), an = abs_bits(num);
   if (lim == AVIP_LIM_SWEBY && beta == 1.0) {  // min-mod: psi = clamp(r, 0, 1)
     const bool same = ((__double2hiint(delta) ^ __double2hiint(num)) >= 0);
-    if (ad != 0 && same) hpsi = an >= ad ? 0.5 : (0.5 * num) * recip_nr(delta);
+    if (ad != 0 && same) hpsi = an >= ad ? 0.5 : 0.5 * slope_ratio(num, delta);
   } else if (ad != 0) {
-    hpsi = 0.5 * limiter(num * recip_nr(delta), beta, lim);
+    hpsi = 0.5 * limiter(slope_ratio(num, delta), beta, lim);
   }
   const double lw = fma(-dt4, fma(sgx, sVx, sgy * sVy), delta);  // delta - dt grad_ij.V_ij
   const double us = fma(lw, hpsi, uU);
