@@ -383,7 +383,7 @@ struct EdgeEnd {
 // Bernoulli function B(x) = x / (e^x - 1) for x >= 0 (B(0) = 1; 0 where it is below 1e-300).
 // B(-x) = x + B(x), so one expm1 gives both values without cancellation.
 __device__ __forceinline__ double bernoulli_pos(double x) {
-  if (abs_bits(x) == 0) return 1.0;
+  if (__double2hiint(x) < 0x3c300000) return 1.0;  // below 2^-60: 1 - x/2 rounds to 1 (and 1 / x may overflow)
   return x > 700.0 ? 0.0 : x * recip_nr(expm1(x));
 }
 

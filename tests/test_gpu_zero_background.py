@@ -47,3 +47,29 @@ def test_limiter_on_subnormal_differences(avip, limiter, beta, batch):
         assert normwise(m.density(s), n[s]) <= 1e-10
     assert normwise(m.phi(), phi) <= 1e-10
     m.close()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_bernoulli_function_at_subnormal_arguments(avip, batch):
+    """Scharfetter-Gummel fluxes in a field so weak that h V.e / D is subnormal: B = 1, plain
+    diffusion.  Tolerance: one explicit step moves a density by less than itself through at most
+    ten edges of some ten roundings each, 1e-14."""
+    p = W.plates_problem(23, 19, 1e-2, 1e-2, 1e-309, seed=3, opts=W.Opts(scheme=W.FLUX_SG))
+    o = O.Oracle(p)
+    n0 = o.initial_state()
+    _, E, _, _, vel, _ = o.fields(n0)
+    d = p.xy[o.edges[:, 1]] - p.xy[o.edges[:, 0]]
+    a = np.abs(0.5 * np.einsum("ij,ij->i", vel[0][o.edges[:, 0]] + vel[0][o.edges[:, 1]], d) / p.species[0].D)
+    assert np.any((a > 0) & (a < 2.0 ** -1024))
+    n, _ = o.step(n0, dt_fixed=1e-8)
+    assert np.abs(n[0] - n0[0]).max() > 1e-3 * np.abs(n[0]).max()
+    m = avip.Mesh(p, rtol=1e-13, dt_fixed=1e-8)
+    if batch:
+        b = avip.Batch([m], cluster_size=8)
+        b.run(1)
+        b.close()
+    else:
+        assert m.step() == 1e-8
+    for s in range(2):
+        assert normwise(m.density(s), n[s]) <= 1e-14
+    m.close()
