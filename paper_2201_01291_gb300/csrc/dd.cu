@@ -384,7 +384,7 @@ struct EdgeEnd {
 // B(-x) = x + B(x), so one expm1 gives both values without cancellation.
 __device__ __forceinline__ double bernoulli_pos(double x) {
   if (__double2hiint(x) < 0x3c300000) return 1.0;  // below 2^-60: 1 - x/2 rounds to 1 (and 1 / x may overflow)
-  return x > 700.0 ? 0.0 : x * recip_nr(expm1(x));
+  return x > 700.0 ? 0.0 : quotient_nr(x, expm1(x));
 }
 
 // Geometry of one edge for the Scharfetter-Gummel split (species independent), canonical
