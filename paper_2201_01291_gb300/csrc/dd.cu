@@ -396,7 +396,7 @@ __device__ __forceinline__ SgGeo sg_geometry(double dx, double dy, double Sx, do
   SgGeo g;
   g.dx = dx;
   g.dy = dy;
-  g.sh = fma(Sx, dx, Sy * dy) * recip_nr(fma(dx, dx, dy * dy));
+  g.sh = quotient_nr(fma(Sx, dx, Sy * dy), fma(dx, dx, dy * dy));
   g.spx = fma(-g.sh, dx, Sx);
   g.spy = fma(-g.sh, dy, Sy);
   return g;
