@@ -290,6 +290,9 @@ __device__ __forceinline__ void dt_cells_body(const DDArgs& a, int bid, int nblo
   __shared__ float s_cur;
   const int ns = a.ph.ns, stride = nblocks * blockDim.x;
   constexpr float kEps = 1e-6f;  // FP32 rounding of the sums below, relative to the sum of magnitudes
+  // below this the squares (and sums) come near FP32's subnormals, where kEps does not bound their
+  // rounding: such a cell counts as this large above and as nothing below
+  constexpr float kTiny = 1e-30f;
   if (threadIdx.x < 2) {
     s_max[threadIdx.x] = 0;
     s_lo[threadIdx.x] = 0;
@@ -318,17 +321,20 @@ __device__ __forceinline__ void dt_cells_body(const DDArgs& a, int bid, int nblo
         const float vx = fabsf((p0.x + p1.x) + (p2.x + p3.x)), vy = fabsf((p0.y + p1.y) + (p2.y + p3.y));
         const float ex = kEps * ((fabsf(p0.x) + fabsf(p1.x)) + (fabsf(p2.x) + fabsf(p3.x)));
         const float ey = kEps * ((fabsf(p0.y) + fabsf(p1.y)) + (fabsf(p2.y) + fabsf(p3.y)));
-        const float hx = vx + ex, hy = vy + ey, lx = fmaxf(vx - ex, 0.f), ly = fmaxf(vy - ey, 0.f);
+        const float hx = (vx + ex) * w, hy = (vy + ey) * w;
+        const float lx = fmaxf(vx - ex, 0.f) * w, ly = fmaxf(vy - ey, 0.f) * w;
         // !(x <= v): a NaN becomes an upper bound that no test excludes
-        const float h2 = (hx * hx + hy * hy) * (w * w);
+        const float h2 = hx * hx + hy * hy;
         if (!(h2 <= v)) v = h2;
-        vl = fmaxf(vl, (lx * lx + ly * ly) * (w * w));
+        vl = fmaxf(vl, lx * lx + ly * ly);
         sig += fabsf((p0.z + p1.z) + (p2.z + p3.z));
         sige += kEps * ((fabsf(p0.z) + fabsf(p1.z)) + (fabsf(p2.z) + fabsf(p3.z)));
       }
       const float inv_nv = n3 >= 0 ? 0.25f : 1.f / 3.f;
+      if (v < kTiny) v = kTiny;
+      sige += kTiny;
       vhi[k] = v * (1.f + 4.f * kEps);
-      vlo = fmaxf(vlo, vl * (1.f - 4.f * kEps));
+      if (vl >= kTiny) vlo = fmaxf(vlo, vl * (1.f - 4.f * kEps));
       shi[k] = (sig + sige) * inv_nv * (1.f + 4.f * kEps);
       slo = fmaxf(slo, fmaxf(sig - sige, 0.f) * inv_nv * (1.f - 4.f * kEps));
     }
