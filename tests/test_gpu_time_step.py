@@ -32,3 +32,68 @@ def test_vanishing_fields(avip, voltage, seed):
     dt = m.step()
     assert abs(dt - info["dt"]) <= 1e-10 * info["dt"]
     m.close()
+
+
+def _neutral(kind, nx, ny, seed, quads, ns):
+    """Constant mobilities and neutral pairs (no space charge), so that the dielectric limit sets the
+    step whatever the solve's tolerance: densities over twenty decades, nearly equal ones (within the
+    screening's margin of 1e-6 of each other), or of either sign, cancelling within the cells."""
+    rng = np.random.default_rng(seed)
+    if quads > 0:
+        p = W.hybrid_plates_problem(nx, ny, 1e-2, 1e-2, 1e4, seed, quad_fraction=quads, n_species=ns)
+    else:
+        p = W.plates_problem(nx, ny, 1e-2, 1e-2, 1e4, seed, n_species=ns)
+    size = p.n_nodes
+    if kind == "decades":
+        n0 = 10.0 ** rng.uniform(0.0, 20.0, size) * np.where(rng.uniform(size=size) < 0.05, -1.0, 1.0)
+    elif kind == "ties":
+        n0 = 1e19 * (1.0 + 1e-8 * rng.uniform(-1.0, 1.0, size))
+    else:
+        n0 = 1e19 * rng.choice([-1.0, 1.0], size) * (1.0 + 0.2 * rng.uniform(size=size))
+    p.species[0].n0[:] = n0
+    p.species[1].n0[:] = n0
+    return p
+
+
+def _dielectric_limit(p):
+    groups = [np.asarray(c) for c in (p.tris, p.quads) if c is not None and len(c)]
+    return min(p.opts.a_diel * W.EPS0 / W.E_CHARGE /
+               sum(abs((s.n0 * s.mob_params[0])[c].mean(axis=1)) for s in p.species).max() for c in groups)
+
+
+# (200,000 cells: above four blocks per SM a thread takes several cells)
+CASES = [(kind, nx, ny, seed, quads, ns) for kind in ("decades", "ties", "signs") for nx, ny, seed, quads, ns in
+         ((9, 7, 1, 0.0, 2), (61, 83, 2, 0.0, 3), (61, 83, 3, 0.5, 2), (33, 29, 4, 1.0, 2), (301, 335, 5, 0.0, 2))]
+
+
+@pytest.mark.parametrize("kind,nx,ny,seed,quads,ns", CASES)
+def test_dielectric_limit(avip, kind, nx, ny, seed, quads, ns):
+    """Tolerance: some ten roundings of 1.1e-16 each in FP64; in mixed precision the FP32 mobilities
+    (6e-8 each)."""
+    p = _neutral(kind, nx, ny, seed, quads, ns)
+    want = _dielectric_limit(p)
+    o = O.Oracle(p)
+    assert abs(o.step(o.initial_state())[1]["dt"] - want) <= 1e-13 * want  # this limit decides
+    for precision, tol in ((avip.PREC_FP64, 1e-13), (avip.PREC_MIXED, 2e-7)):
+        m = avip.Mesh(p, precision=precision, rtol=1e-10)
+        dt = m.step()
+        assert abs(dt - want) <= tol * want, precision
+        m.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_dielectric_limit_in_a_batch(avip, mixed):
+    ps = [_neutral(*c) for c in CASES if c[1] <= 61]
+    precision, tol = (avip.PREC_MIXED, 2e-7) if mixed else (avip.PREC_FP64, 1e-13)
+    meshes = [avip.Mesh(p, precision=precision, rtol=1e-10) for p in ps]
+    b = avip.Batch(meshes, cluster_size=16)
+    for threads in (256, 128):
+        assert avip.batch_set_dd_threads(b.b, threads) == avip.AVIP_OK
+        for m, p in zip(meshes, ps):
+            m.set_state(np.concatenate([s.n0 for s in p.species] + [np.zeros(4 * p.n_nodes + 2)]))
+        for st, p in zip(b.run(1), ps):
+            want = _dielectric_limit(p)
+            assert abs(st["dt_min"] - want) <= tol * want
+    b.close()
+    for m in meshes:
+        m.close()
