@@ -94,9 +94,10 @@ __global__ void __launch_bounds__(TPB, 1) pcg_amg_kernel(PcgArgs a) {
 //   rh.t -> omega, rho', beta;  P4  x += alpha p^ + omega s^, r = s - omega t,
 //   p = r + beta (p - omega v), r.r -> stop test
 // (van der Vorst's iteration with M^-1 applied on the right, so x is updated directly and the
-// stopping test stays on the true scaled residual of the free rows).  P2 is folded into the finest
-// down phase of the second V-cycle, as the residual update is in amg_cg_solve; with an FP32
-// hierarchy the down phases gather FP32 copies of p, r and v.  Two V-cycles per
+// stopping test stays on the true scaled residual of the free rows).  With an FP32 hierarchy the down
+// phases gather FP32 copies of p and s, each rounded once from its FP64 value (s formed from FP32
+// copies of r and v inside the second down phase saves P2's phase, nothing at 491,000 nodes and 1.7 %
+// at 63,000 with photoionisation, and is off by the FP32 rounding of r, not of s).  Two V-cycles per
 // iteration; breakdowns and a true residual still too large restart from the true residual.
 // The products with A stream the matrix by contiguous slice shares (stream_rows, each row's own
 // operands fetched ahead), the elementwise phases take slices round-robin.
@@ -119,15 +120,14 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
   double* __restrict__ rh = a.bcg + 2 * Np;
   double* __restrict__ ph = a.bcg + 3 * Np;
   double* __restrict__ sh = a.bcg + 4 * Np;
-  const int mat = C.mat_phase(), dl = C.D.level;
+  const int mat = C.mat_phase();
   struct Two {
     double u, w;
   };
   // the vectors the finest down phases gather, in the hierarchy's type (amg_cg_solve)
   constexpr bool kCopies = sizeof(T) == 4;
   T* __restrict__ tp = kCopies ? (T*)a.rq32 : (T*)p;
-  T* __restrict__ tr = kCopies ? (T*)a.rq32 + Np : (T*)r;
-  T* __restrict__ tv32 = kCopies ? (T*)a.rq32 + 2 * Np : (T*)v;
+  T* __restrict__ ts = kCopies ? (T*)a.rq32 + Np : (T*)sv;
 
   const double gain = C.gain;
   const int hist = history_length(a);
@@ -177,7 +177,7 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
                   r[i] = ri;
                   rh[i] = ri;
                   p[i] = ri;
-                  if (kCopies) tr[i] = tp[i] = (T)ri;
+                  if (kCopies) tp[i] = (T)ri;
                   r2[0] = fma(ri, ri, r2[0]);
                 });
           }
@@ -206,7 +206,6 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
               ops.ring, mat, lane, [phv](int c) { return __ldca(phv + c); }, [rhv](int i) { return rhv[i]; },
               [&](int i, double w, double rhi) {
                 v[i] = w;
-                if (kCopies) tv32[i] = (T)w;
                 rv[0] = fma(rhi, w, rv[0]);
               });
         }
@@ -225,33 +224,18 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
           continue;
         }
         const double alpha = al[0];
-        // ---- P2 in the finest down phase of s^ = M s: s = r - alpha v (own rows), s.s
+        // ---- P2: s = r - alpha v, s.s
         double ss = 0.0;
+        for (int sl = gwarp; sl < nsl; sl += nwarps) {
+          const int i = sl * kSlice + lane;
+          if (i >= N) continue;
+          const double si = fma(-alpha, v[i], r[i]);
+          sv[i] = si;
+          if (kCopies) ts[i] = (T)si;
+          ss = fma(si, si, ss);
+        }
         bool small;
         {
-          const T alT = (T)alpha;
-          const T* __restrict__ trv = tr;
-          const T* __restrict__ tvv = tv32;
-          auto src = [trv, tvv, alT](int c) { return fma_t(-alT, __ldca(tvv + c), __ldca(trv + c)); };
-          struct Hook {
-            const double *rv, *vv;
-            double *sv, *ss;
-            double al;
-            __device__ Two begin(int i) const { return Two{rv[i], vv[i]}; }
-            __device__ void end(int i, const Two& o) const {
-              const double si = fma(-al, o.w, o.u);
-              sv[i] = si;
-              *ss = fma(si, si, *ss);
-            }
-          } hook{r, v, sv, &ss, alpha};
-          if (dl == 0) {
-            for (int sl = gwarp; sl < nsl; sl += nwarps) {
-              const int i = sl * kSlice + lane;
-              if (i < N) hook.end(i, hook.begin(i));
-            }
-          } else {
-            amg_down(C, ops, 0, src, hook, gwarp, nwarps, lane);
-          }
           double tot[1];
           if (!ops.template sum_epi<1>(ss, tot, small, [thresh](double t, double* o) {
                 o[0] = t;
@@ -269,20 +253,8 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
           if (!ops.barrier()) return false;
           continue;
         }
-        // ---- the rest of s^ = M s, then P3: t = A s^
-        struct Out {
-          double* z;
-          __device__ NoPre begin(int) const { return NoPre(); }
-          __device__ void end(int i, T v, NoPre) const { z[i] = (double)v; }
-        } out{sh};
-        if (dl == 0) {
-          const double* __restrict__ svv = sv;
-          amg_dense(C, ops, [svv](int k) { return (T)__ldca(svv + k); }, out, lane);
-        } else {
-          if (!amg_inner(C, ops, gwarp, nwarps, lane)) return false;
-          amg_up(C, ops, 0, out, lane);
-        }
-        if (!ops.barrier()) return false;
+        // ---- s^ = M s, then P3: t = A s^
+        if (!vcycle(C, (const T*)ts, sh, ops, gwarp, nwarps, lane)) return false;
         double d4[4] = {0.0, 0.0, 0.0, 0.0};  // t.s, t.t, rh.s, rh.t
         {
           const double* __restrict__ shv = sh;
@@ -321,10 +293,7 @@ __device__ bool amg_bicgstab_solve(const PcgArgs& a, const AmgCtx<T>& C, GridOps
           r[i] = ri;
           const double pn = fma(beta, fma(-omega, v[i], pi), ri);
           p[i] = pn;
-          if (kCopies) {
-            tr[i] = (T)ri;
-            tp[i] = (T)pn;
-          }
+          if (kCopies) tp[i] = (T)pn;
           rn2[0] = fma(ri, ri, rn2[0]);
         }
         // (a flag from one thread: a comparison by every thread costs the block 19 cycles per warp)
