@@ -133,8 +133,9 @@ typedef struct avip_opts {
                                           (a grid-wide barrier) may last before the kernel gives
                                           up: its blocks leave, the call returns AVIP_ETIMEOUT and
                                           the handle stays usable.  Default 2; 0 gives up at the
-                                          first wait that is not already satisfied (a test of the
-                                          failure path); at most 60 */
+                                          first wait that is not already satisfied, and the AMG
+                                          solvers (kinds 8 to 11) at their first wait for a part
+                                          of an operator (a test of the failure path); at most 60 */
   int32_t precond_fp64;                /* AMG solvers of the FP64 path: 0 (default) applies the
                                           V-cycle preconditioner with FP32 values and vectors
                                           (the Krylov iterate, the products with the Poisson

@@ -58,7 +58,7 @@ struct SolveShared {
   unsigned long long H[sizeof(AmgDevT<double>) / 8];
   unsigned long long bar[128];      // the rings' mbarriers, kDepth per warp
   double gain;
-  int bad;                          // a warp's copy did not arrive (Ring::wait)
+  int bad;                          // a warp gave up the wait for a copy (Ring::wait)
 };
 // Dynamic shared memory of a solve: the rings, then the dense product's right-hand side.
 constexpr size_t kRhsBytes = sizeof(float) * kInverseRows;
@@ -125,7 +125,8 @@ __device__ AmgCtx<T> solve_begin(SolveShared& sh, R& ring, char* dyn, const PcgA
   }
   __syncthreads();
   ring.init(sh.tab, 2 * dl + 2, dyn + (threadIdx.x >> 5) * R::kWarpBytes,
-            sh.bar + (threadIdx.x >> 5) * R::kDepth, &sh.bad, gwarp, nwarps, lane, matrix_first ? 2 * dl + 1 : 0);
+            sh.bar + (threadIdx.x >> 5) * R::kDepth, &sh.bad, gwarp, nwarps, lane, matrix_first ? 2 * dl + 1 : 0,
+            a.spin_ns == 0);
   return C;
 }
 
@@ -820,9 +821,9 @@ struct GridOps {
 struct ClusterSums {
   double thr[1024];     // per-thread values
   double grp[4];
-  double part[2][16];   // [parity][rank]
+  double2 part[2][16];  // [parity][rank]: the CTA's sum and its SolveShared::bad
   double res[4];
-  int flag;
+  int flag;             // bit 0: the epilogue's, bit 1: a CTA gave up a wait
 };
 template <class R, bool kKeep = false>
 struct ClusterOps {
@@ -830,6 +831,7 @@ struct ClusterOps {
   ClusterSums& sh;
   R ring;
   unsigned seq;
+  const volatile int* bad;  // SolveShared::bad: travels with the sums, so that all CTAs leave at the same one
   __device__ bool barrier() {
     cluster_sync();
     return true;
@@ -847,8 +849,10 @@ struct ClusterOps {
   __device__ bool sum_epi(double v, double (&out)[NE], bool& flag, Epi epi) {
     static_assert(NE <= 4, "ClusterSums::res");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = (int)cl.num_blocks();
-    double* part = sh.part[seq++ & 1];
+    const int par = (int)(seq++ & 1);
+    double2* part = sh.part[par];
     double s[1] = {v}, bt[1];
+    int lost;
     if constexpr (kKeep) {
       // the mixed-precision solves' order (see block_group_sum): a tree in every warp, then the
       // warps in turn
@@ -856,26 +860,30 @@ struct ClusterOps {
       for (int o = 16; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
       if (lane == 0) sh.thr[warp] = s[0];
       __syncthreads();
+      lost = *bad;
       if (warp == 0) {
         bt[0] = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) bt[0] += sh.thr[w];
       }
     } else {
-      block_group_sum<1>(s, bt, sh.thr, sh.grp);
+      lost = block_group_sum<1>(s, bt, sh.thr, sh.grp, bad);
     }
-    if (warp == 0 && lane < C) *cl.map_shared_rank(part + cl.block_rank(), lane) = bt[0];
+    if (warp == 0 && lane < C) *cl.map_shared_rank(part + cl.block_rank(), lane) = make_double2(bt[0], lost ? 1.0 : 0.0);
     cluster_sync();
     if (warp == 0) {
-      double t = lane < C ? part[lane] : 0.0;
+      const double2 p = lane < C ? part[lane] : make_double2(0.0, 0.0);
+      const bool any = __any_sync(0xffffffffu, __double2hiint(p.y) != 0);
+      double t = p.x;
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) sh.flag = epi(t, sh.res) ? 1 : 0;
+      if (lane == 0) sh.flag = (epi(t, sh.res) ? 1 : 0) | (any ? 2 : 0);
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < NE; ++k) out[k] = sh.res[k];
-    flag = sh.flag != 0;
-    return true;
+    const int f = sh.flag;
+    flag = (f & 1) != 0;
+    return f < 2;
   }
   __device__ bool sum(double (&v)[1]) {
     bool f;

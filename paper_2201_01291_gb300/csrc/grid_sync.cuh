@@ -130,16 +130,20 @@ __device__ __forceinline__ AllsumScratch<MAXV>& allsum_scratch() {
 // 2,200 cycles.  Every thread stores its values, four warps per value (one per sub-partition) add
 // a quarter of them each and finish with a shuffle tree, and warp 0 adds the four group sums.
 //
+// Returns *bad (0 without one), read while the sums are formed.
+//
 // kOneGroup keeps the order of a single adding warp.  The mixed-precision solves take it: their FP32
 // inner solves and the FP32 drift-diffusion stage turn a last-bit difference of one of these sums
 // into differences of 1e-9 of the densities within ten steps, so that mixed-precision results are
 // kept bit for bit when a kernel is reworked; it costs them 1,200 cycles per sum.
 template <int NV, bool kOneGroup = false>
-__device__ __forceinline__ void block_group_sum(const double (&v)[NV], double (&bt)[NV], double* thr, double* grp) {
+__device__ __forceinline__ int block_group_sum(const double (&v)[NV], double (&bt)[NV], double* thr, double* grp,
+                                               const volatile int* bad) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) thr[k * 1024 + threadIdx.x] = v[k];
   __syncthreads();
+  const int lost = bad ? *bad : 0;
   const int G = !kOneGroup && nw >= 4 * NV ? 4 : 1;  // groups per value
   if (warp < G * NV) {
     const int k = warp / G, j = warp % G;
@@ -158,6 +162,7 @@ __device__ __forceinline__ void block_group_sum(const double (&v)[NV], double (&
     for (int k = 0; k < NV; ++k)
       bt[k] = G == 4 ? (grp[4 * k] + grp[4 * k + 1]) + (grp[4 * k + 2] + grp[4 * k + 3]) : grp[k];
   }
+  return lost;
 }
 
 struct NoEpilogue {
@@ -192,17 +197,18 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[NV], double (&out)[NE > 
   int& s_ok = scr.ok;
   (void)smem;
   double bt[NV];
-  block_group_sum<NV, kOneGroup>(v, bt, scr.thr, scr.grp);
+  const int lost = block_group_sum<NV, kOneGroup>(v, bt, scr.thr, scr.grp, fs.bad);
   if (warp == 0) {
-    int ok = 1;
-    if (nb > 1) {
+    // (a block that gave up a wait of its own does not arrive: nobody passes a sum with its part in it)
+    int ok = !lost;
+    if (nb > 1 && ok) {
       if (lane == 0) {
         double* mine = fs.parts + ((size_t)par * nb + fs.rank) * 4;
 #pragma unroll
         for (int k = 0; k < NV; ++k) __stcg(mine + k, bt[k]);
         red_add_release_u32(fs.flags, 1u);
       }
-      if ((fs.bad && *fs.bad) || !wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
+      if (!wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
       ok = __all_sync(0xffffffffu, ok);
       double acc[NV];
 #pragma unroll
@@ -276,11 +282,11 @@ __device__ __forceinline__ bool grid_barrier(FlagSync& fs) {
   AllsumScratch<MAXV>& scr = allsum_scratch<MAXV>();
   __syncthreads();
   if (threadIdx.x == 0) {
-    int ok = 1;
+    int ok = !(fs.bad && *fs.bad);
     const int nb = fs.nb;
-    if (nb > 1) {
+    if (nb > 1 && ok) {
       red_add_release_u32(fs.flags, 1u);
-      if ((fs.bad && *fs.bad) || !wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
+      if (!wait_arrivals(fs, seq * (unsigned)nb)) ok = 0;
     }
     if (!ok) atomicExch(&fs.gs->abort, 1);
     scr.ok = ok;

@@ -587,26 +587,30 @@ __device__ void cluster_amg_solve(const PcgArgs& a, ClusterAmgShared& sh, char* 
   const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
   const int gw = rank * wpb + (int)(threadIdx.x >> 5), nw = C * wpb, lane = (int)(threadIdx.x & 31);
   const bool leader = rank == 0 && threadIdx.x == 0;
+  bool ok;
   if (a.amg_mixed) {
-    ClusterOps<R, true> ops{cl, sh.sums, R(), 0u};
+    ClusterOps<R, true> ops{cl, sh.sums, R(), 0u, &sh.solve.bad};
     const AmgCtx<float> ctx =
         solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.aval32, C, gw, nw, lane, false, true);
-    amg_mixed_solve(a, ctx, ops, gw, nw, lane, leader);
+    ok = amg_mixed_solve(a, ctx, ops, gw, nw, lane, leader);
     ops.ring.finish(lane);
   } else if (a.amg32) {
-    ClusterOps<R> ops{cl, sh.sums, R(), 0u};
+    ClusterOps<R> ops{cl, sh.sums, R(), 0u, &sh.solve.bad};
     const AmgCtx<float> ctx =
         solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.A.aval, C, gw, nw, lane, true);
-    amg_cg_solve<float>(a, ctx, a.z, ops, gw, nw, lane, leader);
+    ok = amg_cg_solve<float>(a, ctx, a.z, ops, gw, nw, lane, leader);
     ops.ring.finish(lane);
   } else {
-    ClusterOps<R> ops{cl, sh.sums, R(), 0u};
+    ClusterOps<R> ops{cl, sh.sums, R(), 0u, &sh.solve.bad};
     const AmgCtx<double> ctx =
         solve_begin<double>(sh.solve, ops.ring, ring_mem, a, a.amg, a.A.aval, C, gw, nw, lane, true);
-    amg_cg_solve<double>(a, ctx, a.z, ops, gw, nw, lane, leader);
+    ok = amg_cg_solve<double>(a, ctx, a.z, ops, gw, nw, lane, leader);
     ops.ring.finish(lane);
   }
-  if (sh.solve.bad && lane == 0) atomicCAS(&a.sc->status, AVIP_OK, AVIP_ETIMEOUT);  // (a copy never arrived)
+  if (!ok && leader) {  // the wait for a copy was given up
+    a.res->pcg_status = AVIP_ETIMEOUT;
+    atomicCAS(&a.sc->status, AVIP_OK, AVIP_ETIMEOUT);
+  }
   cl.sync();  // the next instance reuses the shared memory
 }
 

@@ -83,7 +83,9 @@ __host__ __device__ constexpr int steps_per_slot() {
 // One warp's ring and its shares: lane p holds the share of phase p.
 template <int kSlots>
 struct Ring {
+  static_assert(kSlots <= 8, "bits of state");
   static constexpr int kDepth = kSlots;
+  static constexpr unsigned kAll = (1u << kSlots) - 1u;
   static constexpr int kWarpBytes = kSlots * kSlotBytes;
   const PhaseDesc* tab;  // shared memory
   char* buf;             // this warp's slots
@@ -92,13 +94,14 @@ struct Ring {
   unsigned live;         // phases in which this warp has steps
   int cph;               // phase whose first step the oldest slot holds
   int slot;              // oldest slot
-  unsigned parity;       // bit k: parity of slot k's current fetch
+  unsigned state;        // bit k: parity of slot k's current fetch; bit 31: this lane gave up a wait; bit 30: the warp
+                         // has, bits 8 + k then: slot k has a copy in flight
   int pph, prem;         // next phase to fetch from and its steps left
   const char *pcol, *pval;
   int rs;                // lane p: first slot of phase p when everything stays resident
   bool resident;         // the warp's shares of all phases fit its slots: fetched once per solve
   unsigned long long policy;
-  volatile int* bad;     // shared memory: set when a copy did not arrive within the bound
+  volatile int* bad;     // shared memory: set when a wait for a copy is given up
 
   __device__ __forceinline__ int next_live(int ph) const {
     const unsigned above = live & ~((2u << ph) - 1u);
@@ -131,39 +134,54 @@ struct Ring {
     prem -= cap;
     if (prem <= 0) point(next_live(pph));
   }
-  // Wait for slot k's fetch (all lanes).
+  __device__ __forceinline__ bool given_up() const { return state >> 30 & 1u; }
+  // Mask of a slot's columns: without the end-of-slice bit; 0 on a lane that gave up.
+  __device__ __forceinline__ int column_mask() const { return ~((int)state >> 31) & 0x7fffffff; }
+  __device__ __forceinline__ bool arrived(int k) const { return mbar_try(bar + k * 8, (state >> k) & 1u); }
+  // Wait for slot k's fetch.  A lane that gives up, or sees that another warp of the block has, goes on
+  // with columns of 0 (a stale one would gather from anywhere); the warp agrees on it where it has to
+  // meet anyway, before it refills the slot (advance: a vote here costs 0.4 to 0.8 % of a solve).
   __device__ __forceinline__ void wait(int k) {
-    const unsigned par = (parity >> k) & 1u;
-    if (!mbar_try(bar + k * 8, par)) {
+    if (!arrived(k)) {
       int t = 0;
-      while (!mbar_try(bar + k * 8, par))
+      while (!arrived(k))
         if (*bad || ++t == kCopyTries) {
           *bad = 1;
-          break;
+          state |= 1u << 31;
+          return;
         }
     }
-    parity ^= 1u << k;
+    state ^= 1u << k;
+  }
+  // (all lanes) No steps any more: the slots of `flying` keep their copies in flight for finish(), and the
+  // solve leaves at its next sum or grid barrier, which look at *bad.
+  __device__ __forceinline__ void give_up(unsigned flying) {
+    if (!given_up()) state |= 1u << 30 | flying << 8;
+    ns = 0;
+    *bad = 1;
   }
   // Drop what was fetched and fetch from the start of phase ph on.
   __device__ __forceinline__ void restart(int ph, int lane) {
     drain();
     slot = 0;
     cph = ph;
+    if (given_up()) return;
     point(ph);
 #pragma unroll 1
     for (int k = 0; k < kSlots; ++k) issue(k, lane);
   }
   // This warp's shares of the n phases of `t` (shared memory, complete); the first fetches
-  // start at phase `first`.  `b`: this warp's slots, `mb`: its kSlots mbarriers.
+  // start at phase `first`.  `b`: this warp's slots, `mb`: its kSlots mbarriers; no_wait: give up the
+  // first wait (the failure path's test).
   __device__ __forceinline__ void init(const PhaseDesc* t, int n, char* b, unsigned long long* mb, int* bad_flag, int gwarp,
-                                       int nwarps, int lane, int first) {
+                                       int nwarps, int lane, int first, bool no_wait) {
     tab = t;
     buf = b;
     sbuf = (uint32_t)__cvta_generic_to_shared(b);
     bar = (uint32_t)__cvta_generic_to_shared(mb);
     bad = bad_flag;
     policy = evict_first_policy();
-    parity = 0;
+    state = 0;
     if (lane < kSlots) mbar_init(bar + lane * 8);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -208,9 +226,14 @@ struct Ring {
       const int n0 = resident ? total : kSlots;
 #pragma unroll 1
       for (int k = 0; k < n0; ++k) issue(k, lane);
-      if (resident) {
+      if (no_wait) {
+        give_up((1u << n0) - 1u);
+      } else if (resident) {
 #pragma unroll 1
-        for (int k = 0; k < n0; ++k) wait(k);
+        for (int k = 0; k < n0; ++k) {
+          wait(k);
+          if (!agree(k, (1u << n0) - (1u << k))) break;
+        }
       }
     }
   }
@@ -220,23 +243,42 @@ struct Ring {
     if (cph != ph) restart(ph, lane);
     return slot;
   }
-  __device__ __forceinline__ int advance(int k, int lane) {
-    if (resident) return k + 1;
-    __syncwarp();
+  __device__ __forceinline__ bool agree(int k, unsigned flying) {
+    if (__all_sync(0xffffffffu, (int)state >= 0)) return true;
+    if ((int)state >= 0) state ^= 1u << k;
+    give_up(flying);
+    return false;
+  }
+  // False (on all lanes) when a lane gave up the wait for slot k.
+  __device__ __forceinline__ bool advance(int& k, int lane) {
+    if (resident) {
+      ++k;
+      return true;
+    }
+    if (!agree(k, kAll)) return false;
     issue(k, lane);
-    slot = k + 1 == kSlots ? 0 : k + 1;
-    return slot;
+    k = slot = k + 1 == kSlots ? 0 : k + 1;
+    return true;
   }
   __device__ __forceinline__ void leave(int ph) {
     if (!resident) cph = next_live(ph);
   }
-  // Wait for every copy in flight: none may be when the slots are given back or refilled out of
-  // order.
+  // Wait for every copy in flight, whatever was given up: none may be when the slots are given back or
+  // refilled out of order.
   __device__ __forceinline__ void drain() {
-    if (live && !resident) {
+    const unsigned flying = given_up() ? state >> 8 & kAll : live && !resident ? kAll : 0u;
+    state &= ~(kAll << 8);
 #pragma unroll 1
-      for (int k = 0; k < kSlots; ++k) wait(k);
-    }
+    for (int k = 0; k < kSlots; ++k)
+      if (flying >> k & 1u) {
+        int t = 0;
+        while (!__all_sync(0xffffffffu, arrived(k)))
+          if (++t == kCopyTries) {
+            give_up(0u);
+            break;
+          }
+        state ^= 1u << k;
+      }
     __syncwarp();
   }
   // End of a solve: nothing in flight, and the mbarriers may be initialised again.
@@ -280,9 +322,10 @@ __device__ __forceinline__ void stream_rows(R& ring, int ph, int lane, G g, Begi
     const char* s = ring.buf + k * kSlotBytes;
     const int32_t* cs = reinterpret_cast<const int32_t*>(s) + lane;
     const TV* vs = reinterpret_cast<const TV*>(s + K * 128) + lane;
+    const int cmask = ring.column_mask();
     TA x[K], v[K];
 #pragma unroll
-    for (int u = 0; u < K; ++u) x[u] = (TA)g(cs[u * 32] & 0x7fffffff);
+    for (int u = 0; u < K; ++u) x[u] = (TA)g(cs[u * 32] & cmask);
     // bit u: step u ends a slice (lane u looks at step u)
     unsigned ends = __ballot_sync(0xffffffffu, lane < K && lane < left && cs[lane * 32 - lane] < 0);
 #pragma unroll
@@ -303,7 +346,7 @@ __device__ __forceinline__ void stream_rows(R& ring, int ph, int lane, G g, Begi
       if (lead && row < nrows && (ends || left > K)) pre = begin(row);
       if (!ends && left <= K) break;
     }
-    k = ring.advance(k, lane);
+    if (!ring.advance(k, lane)) return;
   }
   ring.leave(ph);
 }
@@ -371,7 +414,7 @@ __device__ __forceinline__ void stream_dense(R& ring, int ph, int lane, const T*
         if (++k == w) end_row();
       }
     }
-    slot = ring.advance(slot, lane);
+    if (!ring.advance(slot, lane)) return;
   }
   ring.leave(ph);
 }
