@@ -813,6 +813,11 @@ struct GridOps {
   }
 };
 
+// The two halves of a cluster barrier.  A solve passes one before its first write to another CTA's shared
+// memory, which is there only once that CTA has started.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
 // Synchronisation of one thread-block cluster: hardware cluster barrier (release / acquire at
 // cluster scope, so global-memory writes of the cluster are visible after it) and sums through
 // distributed shared memory (at most 16 CTAs; deterministic: fixed order of threads and ranks).
@@ -885,7 +890,9 @@ struct ClusterOps {
     flag = (f & 1) != 0;
     return f < 2;
   }
+  // The first sum of amg_cg_solve, and its only one of this form.
   __device__ bool sum(double (&v)[1]) {
+    cluster_wait();
     bool f;
     return sum_epi<1>(v[0], v, f, [](double t, double* o) {
       o[0] = t;

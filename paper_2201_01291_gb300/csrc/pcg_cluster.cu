@@ -44,6 +44,8 @@ struct ClusterShared {
 // memory (read only at the start and by the true-residual passes).
 // One complete solve of the system described by (a, L) by the calling cluster.
 __device__ void cluster_solve(const PcgArgs& a, const ClusterLayout& L, ClusterShared& sh) {
+  cluster_arrive();
+  cluster_wait();
   if (solve_skipped(a.sc)) return;  // every CTA of the cluster reads the same status
   extern __shared__ __align__(16) double dsm[];
   auto& s_part = sh.part;
@@ -295,6 +297,8 @@ struct KahanF {
 // Shared memory per CTA: x64[R + H] (FP64), r64[R] (FP64), r32[R + H], e32[R], p32[R], q32[R]
 // (FP32), then vals32[max_elems] (FP32) and cols[max_elems] (int32) when the matrix fits.
 __device__ void cluster_solve_mixed(const PcgArgs& a, const ClusterLayout& L, ClusterShared& sh) {
+  cluster_arrive();
+  cluster_wait();
   if (solve_skipped(a.sc)) return;  // every CTA of the cluster reads the same status
   extern __shared__ __align__(16) double dsm[];
   auto& s_part = sh.part;
@@ -580,7 +584,11 @@ struct ClusterAmgShared {
 // The FP64 CG with an FP32 (default) or FP64 hierarchy, or the mixed-precision solve.
 template <int TPB>
 __device__ void cluster_amg_solve(const PcgArgs& a, ClusterAmgShared& sh, char* ring_mem) {
-  if (solve_skipped(a.sc)) return;  // every CTA of the cluster reads the same status
+  cluster_arrive();  // (the set-up runs before the wait)
+  if (solve_skipped(a.sc)) {  // every CTA of the cluster reads the same status
+    cluster_wait();
+    return;
+  }
   using R = ClusterRing<TPB>;
   cg::cluster_group cl = cg::this_cluster();
   constexpr int wpb = TPB / 32;
@@ -592,6 +600,7 @@ __device__ void cluster_amg_solve(const PcgArgs& a, ClusterAmgShared& sh, char* 
     ClusterOps<R, true> ops{cl, sh.sums, R(), 0u, &sh.solve.bad};
     const AmgCtx<float> ctx =
         solve_begin<float>(sh.solve, ops.ring, ring_mem, a, a.amg32, a.aval32, C, gw, nw, lane, false, true);
+    cluster_wait();
     ok = amg_mixed_solve(a, ctx, ops, gw, nw, lane, leader);
     ops.ring.finish(lane);
   } else if (a.amg32) {
