@@ -472,6 +472,8 @@ int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
     }
     L.lmax = lambda_max(A, L.dinv);
     if (A.n <= coarse_max || H.lv.size() + 1 >= (size_t)kAmgMaxLevels) {
+      // (the dense product's right-hand side has kInverseRows floats of shared memory)
+      if (A.n > kInverseRows / 2) return fail("AMG set-up: coarsening stalls");
       std::vector<double> dense((size_t)A.n * A.n, 0.0);
       for (int32_t i = 0; i < A.n; ++i)
         for (int32_t e = A.rp[i]; e < A.rp[i + 1]; ++e) dense[(size_t)i * A.n + A.ci[e]] += A.v[e];
