@@ -72,34 +72,59 @@ __device__ __forceinline__ void store_tile(float* g, int ld, const float (&v)[4]
 }
 
 // Thread block j: P = A_kk^-1, R_j = P A_kj (R_k = P) and the copy C_j = A_jk (j != k).
+//
+// The pivot tile is inverted in registers, 16 columns of one row per thread (four neighbouring lanes
+// hold a row): a step takes the pivot row from shared memory, two rows in turn so that one barrier per
+// step suffices, and the thread's element of the pivot column from its quad by a shuffle.  Held in
+// shared memory, with two barriers and 48 conflicting accesses per thread and step, the inversion took
+// 77 us a launch.
 __global__ void __launch_bounds__(kThreads) dense_pivot_kernel(const float* __restrict__ M, int np, int k,
                                                                float* __restrict__ R, float* __restrict__ Cc) {
   __shared__ float P[kB][kB + 4], Y[kB][kB + 4];
+  __shared__ __align__(16) float pivot_row[2][kB];
   const int j = blockIdx.x;
-  load_tile(P, M + (size_t)k * kB * np + k * kB, np);
   if (j != k) load_tile(Y, M + (size_t)k * kB * np + j * kB, np);
-  const int r = threadIdx.x >> 2, c0 = (threadIdx.x & 3) * 16;
-  for (int p = 0; p < kB; ++p) {
-    __syncthreads();
-    const float piv = 1.f / P[p][p], f = P[r][p] * piv;
-    float row[16];
+  const int r = threadIdx.x >> 2, q = threadIdx.x & 3, c0 = 16 * q;
+  float v[16];
+  const float4* src = reinterpret_cast<const float4*>(M + ((size_t)k * kB + r) * np + k * kB + c0);
 #pragma unroll
-    for (int c = 0; c < 16; ++c) row[c] = P[p][c0 + c];
-    __syncthreads();
+  for (int c = 0; c < 4; ++c) {
+    const float4 t = src[c];
+    v[4 * c] = t.x, v[4 * c + 1] = t.y, v[4 * c + 2] = t.z, v[4 * c + 3] = t.w;
+  }
+#pragma unroll 1
+  for (int pq = 0; pq < kB / 16; ++pq) {  // the pivot's quarter of the columns
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const bool pc = c0 + c == p;
-      if (r == p)
-        P[r][c0 + c] = pc ? piv : row[c] * piv;
-      else
-        P[r][c0 + c] = pc ? -f : fmaf(-f, row[c], P[r][c0 + c]);
+    for (int pc = 0; pc < 16; ++pc) {
+      const int p = 16 * pq + pc;
+      float* row = pivot_row[pc & 1];
+      if (r == p) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          *reinterpret_cast<float4*>(row + c0 + 4 * c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+      }
+      __syncthreads();
+      const float piv = 1.f / row[p], f = __shfl_sync(0xffffffffu, v[pc], pq, 4) * piv;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const bool pivot_column = q == pq && c == pc;
+        if (r == p)
+          v[c] = pivot_column ? piv : v[c] * piv;
+        else
+          v[c] = pivot_column ? -f : fmaf(-f, row[c0 + c], v[c]);
+      }
     }
   }
-  __syncthreads();
   if (j == k) {
-    for (int t = threadIdx.x; t < kB * kB; t += kThreads) R[(size_t)(t / kB) * np + k * kB + t % kB] = P[t / kB][t % kB];
+    float4* dst = reinterpret_cast<float4*>(R + (size_t)r * np + k * kB + c0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) dst[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
     return;
   }
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    *reinterpret_cast<float4*>(&P[r][c0 + 4 * c]) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+  __syncthreads();
   float acc[4][4];
   tile_product(acc, P, Y);
   store_tile(R + j * kB, np, acc);
