@@ -431,7 +431,7 @@ int lanes_per_row(const Csr& A, bool mixed) {
   return lpr;
 }
 
-int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
+int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen, bool tail) {
   // the axisymmetric matrix is not symmetric: no symmetrisation, LU instead of Cholesky
   const bool symmetric = m.geometry != AVIP_GEOM_AXISYMMETRIC;
   const int32_t coarse_max = std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
@@ -555,6 +555,7 @@ int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen) {
     B.swap(Bc);
   }
   H.dlev = (int32_t)H.lv.size() - 1;
+  if (!tail) return AVIP_OK;
   H.dmat = H.cinv;
   while (H.dlev > 0 && H.lv[H.dlev - 1].A.n <= kAmgDenseRows) {
     const AmgHostLevel& L = H.lv[H.dlev - 1];

@@ -720,7 +720,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // the hierarchy, built here where the Jacobi form takes over if it cannot be
   AmgHost H;
   auto hierarchy = [&]() {
-    if (amg_setup(m, H, g_err, sizeof(g_err)) == AVIP_OK) return true;
+    if (amg_setup(m, H, g_err, sizeof(g_err), fp64) == AVIP_OK) return true;
     H = AmgHost();
     g_err[0] = 0;
     return false;
@@ -756,7 +756,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   if (bicg_amg || (!bicg && h->opts.precision == AVIP_PREC_FP64 &&
                    (h->opts.pcg_kind == 8 ||
                     (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -784,7 +784,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // AMG V-cycle, FP64 iterative refinement of the residual
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
       (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -795,7 +795,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
   }
   if (amg_cluster.kind == 11) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err)) : AVIP_OK;
+    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -1032,7 +1032,7 @@ int photo_set(avip_mesh_t h, int32_t n_terms, const double* a, const double* kap
       hm.aval = std::move(val);
       hm.dsq.assign(dh.begin(), dh.begin() + m.N);
       AmgHost H;
-      if (amg_setup(hm, H, g_err, sizeof(g_err)) != AVIP_OK) return AVIP_EINVAL;
+      if (amg_setup(hm, H, g_err, sizeof(g_err), true) != AVIP_OK) return AVIP_EINVAL;
       if (h->amg)
         ok = upload_amg_t<double>(h, H, t.amg, false);
       else

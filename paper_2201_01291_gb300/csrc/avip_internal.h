@@ -102,8 +102,9 @@ constexpr int kAmgDenseRows = 1536;
 // rows are 85 MB in FP32, which stay in the 129 MB L2 from one product to the next.
 constexpr int kInverseRows = 4608;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
-// composite operators of every non-coarsest level.
-int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen);
+// composite operators of every non-coarsest level and, if `tail`, its last levels as one dense matrix
+// (which the mixed-precision solves do not take).
+int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen, bool tail);
 
 // SELL-32 form of a CSR matrix with `lpr` lanes per row (1, 2, 4, 8, 16 or 32): a slice holds
 // 32 / lpr consecutive rows; step k of a slice is 32 contiguous elements, entries k*lpr ..
