@@ -370,25 +370,36 @@ void composite_operators(AmgHostLevel& L, bool symmetric) {
 }
 
 // M = U Q + Pf (M' Rf): the V-cycle of level L and below as one dense n x n matrix, from the
-// dense matrix M' of the next level (n' x n').
+// dense matrix M' of the next level (n' x n').  The rows are independent: spread over the host cores.
 void dense_vcycle(const AmgHostLevel& L, const std::vector<double>& Mn, std::vector<double>& M) {
   const int32_t n = L.A.n, nn = L.P.m;
   std::vector<double> W((size_t)nn * n, 0.0);  // M' Rf
-  for (int32_t i = 0; i < nn; ++i)
-    for (int32_t k = 0; k < nn; ++k) {
-      const double m = Mn[(size_t)i * nn + k];
-      for (int32_t e = L.Rf.rp[k]; e < L.Rf.rp[k + 1]; ++e) W[(size_t)i * n + L.Rf.ci[e]] += m * L.Rf.v[e];
-    }
   M.assign((size_t)n * n, 0.0);
-  for (int32_t i = 0; i < n; ++i) {
-    double* __restrict__ row = &M[(size_t)i * n];
-    for (int32_t e = L.Pf.rp[i]; e < L.Pf.rp[i + 1]; ++e) {
-      const double v = L.Pf.v[e];
-      const double* __restrict__ w = &W[(size_t)L.Pf.ci[e] * n];
-      for (int32_t j = 0; j < n; ++j) row[j] += v * w[j];
+  const int nt = n < 768 ? 1 : host_threads(n);  // (starting the threads takes longer below)
+  auto spread = [nt](auto&& rows) {
+    std::vector<std::thread> pool;
+    for (int t = 1; t < nt; ++t) pool.emplace_back(rows, t);
+    rows(0);
+    for (auto& th : pool) th.join();
+  };
+  spread([&](int first) {
+    for (int32_t i = first; i < nn; i += nt)
+      for (int32_t k = 0; k < nn; ++k) {
+        const double m = Mn[(size_t)i * nn + k];
+        for (int32_t e = L.Rf.rp[k]; e < L.Rf.rp[k + 1]; ++e) W[(size_t)i * n + L.Rf.ci[e]] += m * L.Rf.v[e];
+      }
+  });
+  spread([&](int first) {
+    for (int32_t i = first; i < n; i += nt) {
+      double* __restrict__ row = &M[(size_t)i * n];
+      for (int32_t e = L.Pf.rp[i]; e < L.Pf.rp[i + 1]; ++e) {
+        const double v = L.Pf.v[e];
+        const double* __restrict__ w = &W[(size_t)L.Pf.ci[e] * n];
+        for (int32_t j = 0; j < n; ++j) row[j] += v * w[j];
+      }
+      for (int32_t e = L.U.rp[i]; e < L.U.rp[i + 1]; ++e) row[L.U.ci[e]] += L.U.v[e] * L.Q.v[L.U.ci[e]];
     }
-    for (int32_t e = L.U.rp[i]; e < L.U.rp[i + 1]; ++e) row[L.U.ci[e]] += L.U.v[e] * L.Q.v[L.U.ci[e]];
-  }
+  });
 }
 
 }  // namespace
