@@ -54,7 +54,11 @@ struct avip_mesh {
   HostMesh hm;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  std::vector<void*> allocs;
+  struct Alloc {
+    void* p;
+    size_t bytes;
+  };
+  std::vector<Alloc> allocs;
   size_t bytes = 0;  // device bytes held
   // device arrays
   int32_t *sl_ptr = nullptr, *sl_w = nullptr, *rlen = nullptr, *col = nullptr, *cell = nullptr, *flen = nullptr;
@@ -149,20 +153,33 @@ void* dev_alloc(avip_mesh* h, size_t bytes) {
     p = nullptr;
   }
   if (p) {
-    h->allocs.push_back(p);
+    h->allocs.push_back({p, bytes});
     h->bytes += bytes;
   }
   return p;
 }
 
+void give_back(avip_mesh* h, const avip_mesh::Alloc& a) {
+  if (h->opts.free)
+    h->opts.free(a.p, h->opts.alloc_ctx);
+  else
+    cudaFree(a.p);
+  h->bytes -= a.bytes;
+}
+
 void dev_free_all(avip_mesh* h) {
-  for (void* p : h->allocs) {
-    if (h->opts.free)
-      h->opts.free(p, h->opts.alloc_ctx);
-    else
-      cudaFree(p);
-  }
+  for (const auto& a : h->allocs) give_back(h, a);
   h->allocs.clear();
+}
+
+// One allocation before the handle's end (null is accepted); nothing queued may use it any more.
+void dev_free(avip_mesh* h, void* p) {
+  for (size_t k = h->allocs.size(); p && k-- > 0;)
+    if (h->allocs[k].p == p) {
+      give_back(h, h->allocs[k]);
+      h->allocs.erase(h->allocs.begin() + k);
+      return;
+    }
 }
 
 template <typename T>
@@ -548,18 +565,29 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
 }
 
 // The FP32 inverse of the scaled matrix (dense_inverse.cu) in `inverse`, or null there when it is too
-// ill-conditioned for one; false if memory or a launch failed.
+// ill-conditioned for one or memory does not suffice for it (the solvers do without); false if a
+// launch failed.
 bool build_inverse(avip_mesh* h, float*& inverse) {
   const size_t np = (size_t)dense_inverse_rows(h->hm.N);
   float *M = nullptr, *scratch = nullptr;
   int *bad = nullptr, host_bad = 1;
-  if (!zalloc(h, M, np * np + kStreamPad) || !zalloc(h, scratch, dense_inverse_scratch(h->hm.N)) || !zalloc(h, bad, 1) ||
-      launch_dense_inverse(sell_view(h), M, scratch, bad, h->stream) != cudaSuccess ||
-      cudaMemcpyAsync(&host_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-      cudaStreamSynchronize(h->stream) != cudaSuccess)
-    return false;
-  inverse = host_bad ? nullptr : M;
-  return true;
+  const size_t work = dense_inverse_scratch(h->hm.N);
+  const bool room = zalloc(h, M, np * np + kStreamPad) && zalloc(h, scratch, work + 1);
+  if (room) bad = reinterpret_cast<int*>(scratch + work);
+  cudaError_t e = cudaSuccess;
+  if (room) {
+    e = launch_dense_inverse(sell_view(h), M, scratch, bad, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&host_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  }
+  const cudaError_t done = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = done;
+  dev_free(h, scratch);
+  if (e != cudaSuccess || host_bad) {
+    dev_free(h, M);
+    M = nullptr;
+  }
+  inverse = M;
+  return e == cudaSuccess;
 }
 
 // Upload the hierarchy in the handle's preconditioner precision (FP64 values when asked for and
@@ -725,7 +753,10 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     g_err[0] = 0;
     return false;
   };
-  if (inverse && m.N <= kClusterJacobiRows && !hierarchy()) inverse = nullptr;
+  if (inverse && m.N <= kClusterJacobiRows && !hierarchy()) {
+    dev_free(h, inverse);
+    inverse = nullptr;
+  }
   if (!bicg && (h->opts.pcg_kind == 11 ||
                 (automatic && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
                  (inverse || m.N > kClusterJacobiRows))))

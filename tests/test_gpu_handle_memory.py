@@ -26,3 +26,40 @@ def test_mixed_handles_hold_no_dense_tail(avip, nx, ny):
     m = avip.Mesh(_plates(nx, ny), precision=avip.PREC_MIXED)
     assert m.info["device_bytes"] <= 1800 * nx * ny
     m.close()
+
+
+@pytest.mark.parametrize("nx,ny,lx,kind", [(4, 100, 1e-4, 5), (25, 50, 3e-4, 11), (30, 45, 1e-3, 11)])
+def test_a_rejected_inverse_is_given_back(avip, nx, ny, lx, kind):
+    """Meshes too ill-conditioned for an FP32 inverse: as many bytes as with their solver asked for."""
+    p = W.plates_problem(nx, ny, lx, 1.0, 5e3, seed=nx + ny)
+    m, f = avip.Mesh(p), avip.Mesh(p, pcg_kind=kind)
+    assert m.info["pcg_kind"] == f.info["pcg_kind"] == kind
+    assert m.info["device_bytes"] == f.info["device_bytes"]
+    m.close()
+    f.close()
+
+
+@pytest.mark.parametrize("nx,ny,largest,kind", [(65, 65, 60e6, 11), (65, 65, 2e6, 11), (20, 23, 5e5, 5)])
+def test_no_memory_for_the_inverse(avip, monkeypatch, nx, ny, largest, kind):
+    """An allocator that gives no block above `largest` bytes: the handle does without the inverse, which
+    only speeds its solves up."""
+    inner, free = avip.torch_allocator()
+    refused = []
+
+    @avip.ALLOC_FN
+    def alloc(nbytes, ctx):
+        if nbytes > largest:
+            refused.append(nbytes)
+            return None
+        return inner(nbytes, ctx)
+
+    monkeypatch.setattr(avip, "torch_allocator", lambda: (alloc, free))
+    p = _plates(nx, ny)
+    m = avip.Mesh(p, rtol=1e-13, use_torch_allocator=True)
+    assert refused and m.info["pcg_kind"] == kind
+    m.run(3)
+    n, phi, _ = O.Oracle(p).run(3)
+    for s in range(2):
+        assert normwise(m.density(s), n[s]) <= 1e-10
+    assert normwise(m.phi(), phi) <= 1e-10
+    m.close()
