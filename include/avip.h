@@ -319,7 +319,8 @@ int mesh_info(avip_mesh_t h, int64_t* info8);
 
 /* Multigrid hierarchy of the AMG-preconditioned solvers (kinds 8-11; the paper names no solver, this
  * reports the set-up built for this project's preconditioner).  Returns the number of levels
- * (finest first, the last one inverted densely), or 0 when the handle uses another solver; for
+ * (finest first, the last one inverted densely; one level for a handle whose preconditioner is the
+ * inverse of its matrix), or 0 when the handle uses another solver; for
  * the first min(levels, max_levels) levels writes AVIP_LEVEL_STATS values per level at
  * out[AVIP_LEVEL_STATS * l]: rows, stored entries of the level matrix A, of the prolongator P
  * from the next level, and of the composite operators the V-cycle applies, Rf = R (I - A Q),

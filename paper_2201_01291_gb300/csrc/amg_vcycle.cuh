@@ -72,11 +72,10 @@ struct AmgCtx {
   __device__ __forceinline__ int mat_phase() const { return 2 * D.level + 1; }
 };
 
-// The finest dense operator whose share per CTA and product stays within a bound: 576 KB for the
-// inverse of the matrix (11,000 cycles of L2 bandwidth, which save every other level and three
-// quarters of the iterations), 256 KB for the V-cycle's tail, which saves a few phases; the
+// The finest dense operator whose share per CTA and product stays within a bound: kInverseBytesPerCta
+// for the inverse of the matrix, 256 KB for the V-cycle's tail, which saves a few phases; the
 // coarsest inverse on fewer CTAs.
-constexpr size_t kInverseBytesPerCta = 576 * 1024, kDenseBytesPerCta = 256 * 1024;
+constexpr size_t kDenseBytesPerCta = 256 * 1024;
 template <typename T>
 __device__ __forceinline__ int dense_choice(const AmgDevT<T>& H, int nctas) {
   auto bytes = [&](int k) {

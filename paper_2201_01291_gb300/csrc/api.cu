@@ -83,6 +83,8 @@ struct avip_mesh {
   double* r2 = nullptr;             // second buffer of the AMG-CG residual
   float* rq32 = nullptr;            // FP32 copies of both residual buffers and of q (FP32 hierarchy)
   int32_t* colS = nullptr;          // col with the end of every slice marked (AMG solvers)
+  float* inverse = nullptr;         // the inverse of the matrix (amg32's dense[0]), or null
+  bool inverse_only = false;        // amg32 holds no hierarchy beside it
   int32_t amg_levels = 0;
   std::vector<int64_t> amg_stats;  // per level: rows, nnz(A), nnz(P)
   float *aval32 = nullptr, *e32 = nullptr, *r32 = nullptr, *p32 = nullptr, *q32 = nullptr;  // mixed precision
@@ -479,13 +481,15 @@ void invalidate_graph(avip_mesh* h) {
 
 // Device copy of the AMG hierarchy with values of type T (float by default, or double): per
 // non-coarsest level the composite operators Q, Rf, U, Pf in SELL-32 and the vectors xp (and,
-// below the finest level, x and b); the coarsest level's x, b and its dense inverse.
+// below the finest level, x and b); the coarsest level's x, b and its dense inverse.  An H without
+// levels leaves the inverse of the matrix alone.  The descriptors go to `out`, allocated if null.
 template <typename T>
 bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record = true,
                   const float* inverse = nullptr) {
   AmgDevT<T> D;
   std::memset(&D, 0, sizeof(D));
-  D.nlev = (int32_t)H.lv.size();
+  const bool levels = !H.lv.empty();
+  D.nlev = levels ? (int32_t)H.lv.size() : 1;
   auto put = [&](const Csr& M, SellMatT<T>& dst) {
     SellHost S;
     sell_from_csr(M, S, lanes_per_row(M, h->opts.precision == AVIP_PREC_MIXED));
@@ -529,7 +533,8 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
     return C;
   };
   bool ok = true;
-  for (int32_t l = 0; l < D.nlev && ok; ++l) {
+  D.L[0].n = h->hm.N;
+  for (int32_t l = 0; l < (int32_t)H.lv.size() && ok; ++l) {
     const AmgHostLevel& L = H.lv[l];
     AmgLevelT<T>& dl = D.L[l];
     dl.n = L.A.n;
@@ -544,19 +549,24 @@ bool upload_amg_t(avip_mesh* h, const AmgHost& H, AmgDevT<T>*& out, bool record 
     }
     if (l > 0) ok = ok && zalloc(h, dl.b, npad);
   }
-  ok = ok && put_dense(H.cinv, D.nlev - 1, D.dense[2]);
-  if (H.dlev == D.nlev - 1)
-    D.dense[1] = D.dense[2];
-  else
-    ok = ok && put_dense(H.dmat, H.dlev, D.dense[1]);
-  if (inverse) D.dense[0] = AmgDenseT<T>{(const T*)inverse, 0, dense_inverse_rows(H.lv[0].A.n) / kSlice};
-  auto* dd = static_cast<AmgDevT<T>*>(dev_alloc(h, sizeof(D)));
+  if (inverse) D.dense[0] = AmgDenseT<T>{(const T*)inverse, 0, dense_inverse_rows(h->hm.N) / kSlice};
+  if (levels) {
+    ok = ok && put_dense(H.cinv, D.nlev - 1, D.dense[2]);
+    if (H.dlev == D.nlev - 1)
+      D.dense[1] = D.dense[2];
+    else
+      ok = ok && put_dense(H.dmat, H.dlev, D.dense[1]);
+  } else {
+    D.dense[1] = D.dense[2] = D.dense[0];
+  }
+  auto* dd = out ? out : static_cast<AmgDevT<T>*>(dev_alloc(h, sizeof(D)));
   ok = ok && dd && cudaMemcpyAsync(dd, &D, sizeof(D), cudaMemcpyHostToDevice, h->stream) == cudaSuccess &&
        cudaStreamSynchronize(h->stream) == cudaSuccess;
   out = dd;
-  if (!record) return ok;
+  if (!record || !ok) return ok;
   h->amg_levels = D.nlev;
   h->amg_stats.clear();
+  if (!levels) h->amg_stats = {h->hm.N, h->hm.nnz, 0, 0, 0, 0};
   for (const AmgHostLevel& L : H.lv) {
     auto nz = [](const Csr& M) -> int64_t { return M.rp.empty() ? 0 : M.rp[M.n]; };
     for (int64_t v : {(int64_t)L.A.n, nz(L.A), nz(L.P), nz(L.Rf), nz(L.U), nz(L.Pf)}) h->amg_stats.push_back(v);
@@ -590,9 +600,32 @@ bool build_inverse(avip_mesh* h, float*& inverse) {
   return e == cudaSuccess;
 }
 
+// The solvers on `ctas` CTAs apply the inverse of n rows (dense_choice).
+bool inverse_fits(int32_t n, int ctas) {
+  return sizeof(float) * n * (size_t)dense_inverse_rows(n) <= kInverseBytesPerCta * (size_t)ctas;
+}
+
+// A handle whose own solves apply the inverse has no hierarchy.  For batches on clusters of `least` CTAs
+// and more it gets one if those cannot apply the inverse.  The handle is idle.
+int prepare_for_batch(avip_mesh* h, int least) {
+  if (!h->inverse) return AVIP_OK;
+  if (h->inverse_only && !inverse_fits(h->hm.N, least)) {
+    AmgHost H;
+    if (amg_setup(h->hm, H, g_err, sizeof(g_err), true) != AVIP_OK) {
+      g_err[0] = 0;  // (the inverse serves any number of CTAs)
+      return AVIP_OK;
+    }
+    if (!upload_amg_t<float>(h, H, h->amg32, true, h->inverse)) return AVIP_ENOMEM;
+    h->inverse_only = false;
+  }
+  return AVIP_OK;
+}
+
 // Upload the hierarchy in the handle's preconditioner precision (FP64 values when asked for and
 // the solve is not the mixed-precision one) with its preconditioned-residual vector.
 bool upload_amg(avip_mesh* h, const AmgHost& H, size_t Np, float* inverse = nullptr) {
+  h->inverse = inverse;
+  h->inverse_only = H.lv.empty();
   if (!zalloc(h, h->colS, h->hm.col.size() + kStreamPad) ||
       launch_mark_slices(h->sl_ptr, h->hm.nslices, h->col, h->colS, h->stream) != cudaSuccess)
     return false;
@@ -753,10 +786,12 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     g_err[0] = 0;
     return false;
   };
-  if (inverse && m.N <= kClusterJacobiRows && !hierarchy()) {
-    dev_free(h, inverse);
-    inverse = nullptr;
-  }
+  // the hierarchy of a solve on `ctas` CTAs: none where these apply the inverse (creating a handle of
+  // 65 x 65 nodes: 17.8 -> 10.1 ms, 17 x 17: 1.44 -> 0.80)
+  auto build_hierarchy = [&](int ctas) {
+    if (!H.lv.empty() || (inverse && inverse_fits(m.N, ctas))) return (int)AVIP_OK;
+    return amg_setup(m, H, g_err, sizeof(g_err), fp64);
+  };
   if (!bicg && (h->opts.pcg_kind == 11 ||
                 (automatic && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
                  (inverse || m.N > kClusterJacobiRows))))
@@ -787,7 +822,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   if (bicg_amg || (!bicg && h->opts.precision == AVIP_PREC_FP64 &&
                    (h->opts.pcg_kind == 8 ||
                     (h->opts.pcg_kind == 0 && h->plan.kind != 5 && amg_cluster.kind != 11)))) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
+    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, bicg ? 9 : 8, h->opts.precond_fp64 ? 1 : 0, inverse ? m.N : 0);
+    int rc = build_hierarchy(h->plan.blocks);
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -795,7 +831,6 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
       return rc;
     }
     ok = ok && upload_amg(h, H, Np, inverse);
-    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, bicg ? 9 : 8, h->amg ? 1 : 0, inverse ? m.N : 0);
   }
   if (h->opts.precision == AVIP_PREC_MIXED) {
     std::vector<float> a32(m.aval.begin(), m.aval.end());
@@ -826,7 +861,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
     h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
   }
   if (amg_cluster.kind == 11) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
+    int rc = build_hierarchy(amg_cluster.blocks);
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -1543,6 +1578,11 @@ int batch_create(const avip_mesh_t* meshes, int32_t count, int32_t cluster_size,
     cudaStreamSynchronize(h->stream);
     b->m.push_back(h);
   }
+  for (avip_mesh* h : b->m)
+    if (const int rc = prepare_for_batch(h, cluster_size ? cluster_size : 2); rc != AVIP_OK) {
+      delete b;
+      return rc;
+    }
   if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     delete b;

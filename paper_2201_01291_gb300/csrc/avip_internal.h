@@ -101,6 +101,9 @@ constexpr int kAmgDenseRows = 1536;
 // Planar FP64 meshes up to this size get the inverse of the matrix itself (dense_inverse.cu): 4,608
 // rows are 85 MB in FP32, which stay in the 129 MB L2 from one product to the next.
 constexpr int kInverseRows = 4608;
+// A solve applies the inverse where its share per CTA stays below this: 11,000 cycles of L2 bandwidth a
+// product, which save every other level and three quarters of the iterations.
+constexpr size_t kInverseBytesPerCta = 576 * 1024;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
 // composite operators of every non-coarsest level and, if `tail`, its last levels as one dense matrix
 // (which the mixed-precision solves do not take).
@@ -182,7 +185,8 @@ struct AmgDevT {
   int32_t pad;
   // dense[0]: the inverse of the finest matrix (small planar meshes, dense_inverse.cu; null
   // otherwise); dense[1]: the V-cycle from the finest level of at most kAmgDenseRows rows down, as
-  // one matrix; dense[2]: the inverse of the coarsest matrix (see dense_choice)
+  // one matrix; dense[2]: the inverse of the coarsest matrix (see dense_choice).  Without a hierarchy
+  // (nlev 1) all three are the first.
   AmgDenseT<T> dense[3];
   AmgLevelT<T> L[kAmgMaxLevels];
 };

@@ -63,3 +63,36 @@ def test_no_memory_for_the_inverse(avip, monkeypatch, nx, ny, largest, kind):
         assert normwise(m.density(s), n[s]) <= 1e-10
     assert normwise(m.phi(), phi) <= 1e-10
     m.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(31, 37), (65, 65)])
+def test_handles_with_the_inverse_hold_no_hierarchy(avip, nx, ny):
+    """Less than the inverse (64-row tiles) beside a handle of the V-cycle, which has its levels."""
+    p = _plates(nx, ny)
+    m, f = avip.Mesh(p), avip.Mesh(p, pcg_kind=11)
+    rows = (nx * ny + 63) // 64 * 64
+    assert len(f.info["levels"]) > 1
+    assert m.info["levels"] == [(nx * ny, m.info["nnz"], 0, 0, 0, 0)]
+    assert m.info["device_bytes"] < f.info["device_bytes"] + 4 * rows * rows
+    m.close()
+    f.close()
+
+
+@pytest.mark.parametrize("nx,ny,cluster", [
+    (16, 32, 2), (27, 19, 2), (31, 37, 2), (31, 37, 16), (32, 48, 16), (29, 53, 16), (65, 65, 0), (65, 65, 2)])
+def test_inverse_in_a_batch(avip, nx, ny, cluster):
+    """512 and 513 rows: the last that two CTAs apply and the first that they do not; 1,536 and 1,537: likewise
+    for 16.  The handle then still steps on its own."""
+    p, q = _plates(nx, ny), _plates(17, 17)
+    m, other = avip.Mesh(p, rtol=1e-13), avip.Mesh(q, rtol=1e-13)
+    b = avip.Batch([m, other], cluster_size=cluster)
+    b.run(2)
+    b.close()
+    for mesh, prob in ((m, p), (other, q)):
+        mesh.run(2)
+        n, phi, _ = O.Oracle(prob).run(4)
+        for s in range(2):
+            assert normwise(mesh.density(s), n[s]) <= 1e-10
+        assert normwise(mesh.phi(), phi) <= 1e-10
+    for h in (m, other):
+        h.close()
