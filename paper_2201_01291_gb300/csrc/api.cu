@@ -606,7 +606,9 @@ bool inverse_fits(int32_t n, int ctas) {
 }
 
 // A handle whose own solves apply the inverse has no hierarchy.  For batches on clusters of `least` CTAs
-// and more it gets one if those cannot apply the inverse.  The handle is idle.
+// and more it gets one if those cannot apply the inverse; an inverse that no batch can apply (16 CTAs:
+// above 1,536 nodes) is given back, 10 to 85 MB, and the handle's own solves go to one cluster as
+// without it.  The handle is idle.
 int prepare_for_batch(avip_mesh* h, int least) {
   if (!h->inverse) return AVIP_OK;
   if (h->inverse_only && !inverse_fits(h->hm.N, least)) {
@@ -618,6 +620,15 @@ int prepare_for_batch(avip_mesh* h, int least) {
     if (!upload_amg_t<float>(h, H, h->amg32, true, h->inverse)) return AVIP_ENOMEM;
     h->inverse_only = false;
   }
+  if (h->inverse_only || inverse_fits(h->hm.N, 16)) return AVIP_OK;
+  const AmgDenseT<float> none = {};
+  cudaError_t e = cudaMemcpyAsync(&h->amg32->dense[0], &none, sizeof(none), cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) return cuda_status(e);
+  dev_free(h, h->inverse);
+  h->inverse = nullptr;
+  if (const PcgPlan pl = amg_cluster_plan(h->opts.cluster_size, h->hm.N); pl.kind == 11) h->plan = pl;
+  invalidate_graph(h);
   return AVIP_OK;
 }
 

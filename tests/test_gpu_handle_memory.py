@@ -82,10 +82,13 @@ def test_handles_with_the_inverse_hold_no_hierarchy(avip, nx, ny):
     (16, 32, 2), (27, 19, 2), (31, 37, 2), (31, 37, 16), (32, 48, 16), (29, 53, 16), (65, 65, 0), (65, 65, 2)])
 def test_inverse_in_a_batch(avip, nx, ny, cluster):
     """512 and 513 rows: the last that two CTAs apply and the first that they do not; 1,536 and 1,537: likewise
-    for 16.  The handle then still steps on its own."""
+    for 16.  Above, no batch can, and the inverse is given back.  The handle then still steps on its own."""
     p, q = _plates(nx, ny), _plates(17, 17)
-    m, other = avip.Mesh(p, rtol=1e-13), avip.Mesh(q, rtol=1e-13)
+    m, other, f = avip.Mesh(p, rtol=1e-13), avip.Mesh(q, rtol=1e-13), avip.Mesh(p, pcg_kind=11)
     b = avip.Batch([m, other], cluster_size=cluster)
+    if nx * ny > 1536:
+        # (the solver's partials and flags are those of the whole GPU)
+        assert avip.mesh_info(m.h)["device_bytes"] <= f.info["device_bytes"] + (1 << 15)
     b.run(2)
     b.close()
     for mesh, prob in ((m, p), (other, q)):
@@ -94,5 +97,5 @@ def test_inverse_in_a_batch(avip, nx, ny, cluster):
         for s in range(2):
             assert normwise(mesh.density(s), n[s]) <= 1e-10
         assert normwise(mesh.phi(), phi) <= 1e-10
-    for h in (m, other):
+    for h in (m, other, f):
         h.close()
