@@ -442,7 +442,7 @@ int lanes_per_row(const Csr& A, bool mixed) {
   return lpr;
 }
 
-int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen, bool tail) {
+int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen, size_t tail) {
   // the axisymmetric matrix is not symmetric: no symmetrisation, LU instead of Cholesky
   const bool symmetric = m.geometry != AVIP_GEOM_AXISYMMETRIC;
   const int32_t coarse_max = std::min(kCoarseMax, std::max(kCoarseMin, m.N / 64));
@@ -566,8 +566,10 @@ int amg_setup(const HostMesh& m, AmgHost& H, char* err, size_t errlen, bool tail
     B.swap(Bc);
   }
   H.dlev = (int32_t)H.lv.size() - 1;
-  if (!tail) return AVIP_OK;
   H.dmat = H.cinv;
+  int32_t first = H.dlev;
+  while (first > 0 && H.lv[first - 1].A.n <= kAmgDenseRows) --first;
+  if ((size_t)H.lv[first].A.n * ((H.lv[first].A.n + kSlice - 1) / kSlice * kSlice) > tail) return AVIP_OK;
   while (H.dlev > 0 && H.lv[H.dlev - 1].A.n <= kAmgDenseRows) {
     const AmgHostLevel& L = H.lv[H.dlev - 1];
     std::vector<double> M;

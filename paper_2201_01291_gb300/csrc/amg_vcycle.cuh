@@ -73,9 +73,8 @@ struct AmgCtx {
 };
 
 // The finest dense operator whose share per CTA and product stays within a bound: kInverseBytesPerCta
-// for the inverse of the matrix, 256 KB for the V-cycle's tail, which saves a few phases; the
-// coarsest inverse on fewer CTAs.
-constexpr size_t kDenseBytesPerCta = 256 * 1024;
+// for the inverse of the matrix, kDenseBytesPerCta for the V-cycle's tail; the coarsest inverse on
+// fewer CTAs.
 template <typename T>
 __device__ __forceinline__ int dense_choice(const AmgDevT<T>& H, int nctas) {
   auto bytes = [&](int k) {

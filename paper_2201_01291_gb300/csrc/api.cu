@@ -479,6 +479,14 @@ void invalidate_graph(avip_mesh* h) {
   h->graph_valid = false;
 }
 
+// Entries of the V-cycle's dense tail that solves on `ctas` CTAs, or in a batch, apply (dense_choice; the
+// mixed-precision solves take the coarsest inverse whatever the hierarchy).  A larger one would be
+// 4 to 9 MB for nothing (FP64 handle of 95 x 95 nodes: TAIL_MB).
+size_t tail_entries(const avip_mesh* h, int ctas) {
+  if (h->opts.precision == AVIP_PREC_MIXED) return 0;
+  return kDenseBytesPerCta * std::max(ctas, 16) / (h->opts.precond_fp64 ? sizeof(double) : sizeof(float));
+}
+
 // Device copy of the AMG hierarchy with values of type T (float by default, or double): per
 // non-coarsest level the composite operators Q, Rf, U, Pf in SELL-32 and the vectors xp (and,
 // below the finest level, x and b); the coarsest level's x, b and its dense inverse.  An H without
@@ -613,7 +621,7 @@ int prepare_for_batch(avip_mesh* h, int least) {
   if (!h->inverse) return AVIP_OK;
   if (h->inverse_only && !inverse_fits(h->hm.N, least)) {
     AmgHost H;
-    if (amg_setup(h->hm, H, g_err, sizeof(g_err), true) != AVIP_OK) {
+    if (amg_setup(h->hm, H, g_err, sizeof(g_err), tail_entries(h, 16)) != AVIP_OK) {
       g_err[0] = 0;  // (the inverse serves any number of CTAs)
       return AVIP_OK;
     }
@@ -789,10 +797,11 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   const bool automatic = h->opts.pcg_kind == 0;
   float* inverse = nullptr;
   if (!bicg && automatic && fp64 && !h->opts.precond_fp64 && m.N <= kInverseRows) ok = ok && build_inverse(h, inverse);
-  // the hierarchy, built here where the Jacobi form takes over if it cannot be
+  // BiCGStab's hierarchy, built here where the Jacobi form takes over if it cannot be
   AmgHost H;
   auto hierarchy = [&]() {
-    if (amg_setup(m, H, g_err, sizeof(g_err), fp64) == AVIP_OK) return true;
+    const int ctas = amg_plan(m.nslices, h->opts.pcg_threads, 9, h->opts.precond_fp64 ? 1 : 0).blocks;
+    if (amg_setup(m, H, g_err, sizeof(g_err), tail_entries(h, ctas)) == AVIP_OK) return true;
     H = AmgHost();
     g_err[0] = 0;
     return false;
@@ -801,7 +810,7 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // 65 x 65 nodes: 17.8 -> 10.1 ms, 17 x 17: 1.44 -> 0.80)
   auto build_hierarchy = [&](int ctas) {
     if (!H.lv.empty() || (inverse && inverse_fits(m.N, ctas))) return (int)AVIP_OK;
-    return amg_setup(m, H, g_err, sizeof(g_err), fp64);
+    return amg_setup(m, H, g_err, sizeof(g_err), tail_entries(h, ctas));
   };
   if (!bicg && (h->opts.pcg_kind == 11 ||
                 (automatic && m.N <= (inverse ? kClusterInverseRows : kClusterAutoRows) &&
@@ -861,7 +870,8 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
   // AMG V-cycle, FP64 iterative refinement of the residual
   if (h->opts.precision == AVIP_PREC_MIXED && !bicg &&
       (h->opts.pcg_kind == 10 || (h->opts.pcg_kind == 0 && h->plan.kind != 6 && amg_cluster.kind != 11))) {
-    int rc = H.lv.empty() ? amg_setup(m, H, g_err, sizeof(g_err), fp64) : AVIP_OK;
+    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
+    int rc = build_hierarchy(h->plan.blocks);
     if (rc != AVIP_OK) {
       dev_free_all(h);
       if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -869,7 +879,6 @@ int mesh_create_hybrid(const double* xy, int32_t n_nodes, const int32_t* tris, i
       return rc;
     }
     ok = ok && upload_amg(h, H, Np);
-    h->plan = amg_plan(m.nslices, h->opts.pcg_threads, 10, 0);
   }
   if (amg_cluster.kind == 11) {
     int rc = build_hierarchy(amg_cluster.blocks);
@@ -1109,7 +1118,8 @@ int photo_set(avip_mesh_t h, int32_t n_terms, const double* a, const double* kap
       hm.aval = std::move(val);
       hm.dsq.assign(dh.begin(), dh.begin() + m.N);
       AmgHost H;
-      if (amg_setup(hm, H, g_err, sizeof(g_err), true) != AVIP_OK) return AVIP_EINVAL;
+      const int ctas = group ? (h->plan.blocks + n_terms - 1) / n_terms : h->plan.blocks;
+      if (amg_setup(hm, H, g_err, sizeof(g_err), tail_entries(h, ctas)) != AVIP_OK) return AVIP_EINVAL;
       if (h->amg)
         ok = upload_amg_t<double>(h, H, t.amg, false);
       else

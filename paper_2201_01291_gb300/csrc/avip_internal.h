@@ -104,10 +104,12 @@ constexpr int kInverseRows = 4608;
 // A solve applies the inverse where its share per CTA stays below this: 11,000 cycles of L2 bandwidth a
 // product, which save every other level and three quarters of the iterations.
 constexpr size_t kInverseBytesPerCta = 576 * 1024;
+// Likewise for the V-cycle's tail as one matrix, which saves a few phases.
+constexpr size_t kDenseBytesPerCta = 256 * 1024;
 // Builds the smoothed-aggregation hierarchy of the scaled Poisson matrix of `m`, with the
-// composite operators of every non-coarsest level and, if `tail`, its last levels as one dense matrix
-// (which the mixed-precision solves do not take).
-int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen, bool tail);
+// composite operators of every non-coarsest level and its last levels as one dense matrix, unless that
+// has more than `tail` entries (rows padded to 32: more than the solves apply).
+int amg_setup(const HostMesh& m, AmgHost& out, char* err, size_t errlen, size_t tail);
 
 // SELL-32 form of a CSR matrix with `lpr` lanes per row (1, 2, 4, 8, 16 or 32): a slice holds
 // 32 / lpr consecutive rows; step k of a slice is 32 contiguous elements, entries k*lpr ..

@@ -28,6 +28,15 @@ def test_mixed_handles_hold_no_dense_tail(avip, nx, ny):
     m.close()
 
 
+@pytest.mark.parametrize("nx,ny,kind", [(95, 95, 0), (65, 65, 11)])
+def test_fp64_handles_hold_only_a_tail_they_apply(avip, nx, ny, kind):
+    """One cluster of 16 CTAs applies a tail of at most 4.2 MB (256 KB each); some 1,500 bytes a node beside."""
+    m = avip.Mesh(_plates(nx, ny), pcg_kind=kind)
+    assert m.info["pcg_kind"] == 11
+    assert m.info["device_bytes"] <= 1600 * nx * ny + 16 * 256 * 1024
+    m.close()
+
+
 @pytest.mark.parametrize("nx,ny,lx,kind", [(4, 100, 1e-4, 5), (25, 50, 3e-4, 11), (30, 45, 1e-3, 11)])
 def test_a_rejected_inverse_is_given_back(avip, nx, ny, lx, kind):
     """Meshes too ill-conditioned for an FP32 inverse: as many bytes as with their solver asked for."""
