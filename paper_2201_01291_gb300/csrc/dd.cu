@@ -419,7 +419,7 @@ __device__ __forceinline__ double sg_flux(double ulo, double uhi, const SgGeo& G
                                           double sgy, const SpeciesParams& sp) {
   const double Vd = 0.5 * fma(sVx, G.dx, sVy * G.dy);  // V.d
   double fpar;
-  if (sp.D > 0.0) {
+  if (sp.invD > 0.0) {  // (else the upwind limit: also for D below 2^-1024, whose part of the flux is nothing)
     const double a = Vd * sp.invD;
     const double aa = fabs(a);
     const double Bp = bernoulli_pos(aa), Bm = aa + Bp;  // B(|a|), B(-|a|)

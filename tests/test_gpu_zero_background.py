@@ -1,6 +1,8 @@
 """Densities on a zero background: an explicit front that runs into it decays through the subnormal
 numbers (an edge's difference below 2^-1024 has no finite reciprocal), and the step stays that of the
 oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -72,4 +74,24 @@ def test_bernoulli_function_at_subnormal_arguments(avip, batch):
         assert m.step() == 1e-8
     for s in range(2):
         assert normwise(m.density(s), n[s]) <= 1e-14
+    m.close()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_diffusion_without_a_finite_reciprocal(avip, batch):
+    """D = 1e-310 (1 / D overflows) in Scharfetter-Gummel fluxes without a field: nothing moves.  Tolerance:
+    the update adds nothing to a density, one rounding."""
+    p = W.plates_problem(23, 19, 1e-2, 1e-2, 0.0, seed=3, opts=W.Opts(scheme=W.FLUX_SG))
+    p = dataclasses.replace(p, species=[dataclasses.replace(s, D=1e-310) for s in p.species])
+    o = O.Oracle(p)
+    n, _ = o.step(o.initial_state(), dt_fixed=1e-8)
+    m = avip.Mesh(p, rtol=1e-13, dt_fixed=1e-8)
+    if batch:
+        b = avip.Batch([m], cluster_size=8)
+        b.run(1)
+        b.close()
+    else:
+        assert m.step() == 1e-8
+    for s in range(2):
+        assert normwise(m.density(s), n[s]) <= 2.3e-16
     m.close()
