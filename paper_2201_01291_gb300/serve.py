@@ -32,14 +32,23 @@ import numpy as np
 
 from . import avip
 
-# Device bytes of one handle, per node and per stored matrix entry (SELL elements plus the
-# per-node vectors of the solver and of the drift-diffusion stage); used for admission.
-BYTES_PER_NODE = 1400
+# Device bytes of one handle, for admission: per node and per cell (the mesh's slots and the vectors and
+# operators of the solver and of the drift-diffusion stage; measured from 2,300 to 300,000 nodes: 1,618 a
+# node on triangles and 1,770 on quadrangles in mixed precision, 1,390-1,500 and 1,500-1,550 in FP64),
+# per photoionisation term, and the largest dense operator of an FP64 hierarchy, in rows, on one
+# cluster and on the whole GPU (below 500 nodes: the inverse).
+BYTES_PER_NODE = 1620
+BYTES_PER_NODE_FP64 = 1440
 BYTES_PER_TRI = 24
+BYTES_PER_QUAD = 200
+BYTES_PER_NODE_PHOTO = 550
+DENSE_ROWS_CLUSTER = 1024
+DENSE_ROWS = 1536
+AXISYM_AMG_NODES = 3000  # axisymmetric meshes up to this size have no hierarchy
 SHARED_MAX_NODES = 300000  # requests up to this size solve on one thread-block cluster (shared)
 AUTO_CLUSTER_NODES = 20000  # up to this the library's automatic choice is a cluster solver (mixed)
-# FP64: above this the library's automatic choice keeps an inverse of the matrix that estimate_bytes
-# does not count (4 bytes x nodes squared) and, from 1,201 nodes on, takes the whole GPU with it
+# FP64: above this the library's automatic choice keeps an inverse of the matrix (4 bytes x nodes
+# squared) and, from 1,201 nodes on, takes the whole GPU with it
 AUTO_CLUSTER_NODES_FP64 = 500
 CLUSTER_KINDS = (5, 6, 11)  # solver kinds that occupy one thread-block cluster, not the whole GPU
 FREE_MARGIN = 512 << 20  # device memory kept free for the CUDA runtime and the caching allocator
@@ -49,8 +58,17 @@ FREE_MARGIN = 512 << 20  # device memory kept free for the CUDA runtime and the 
 CLUSTER_CTAS_BY_NODES = ((SHARED_MAX_NODES, 16),)
 
 
-def estimate_bytes(problem) -> int:
-    return int(problem.n_nodes * BYTES_PER_NODE + problem.n_tris * BYTES_PER_TRI) + (1 << 20)
+def estimate_bytes(problem, precision: int = avip.PREC_MIXED) -> int:
+    """Device bytes that a request's handle holds, at most."""
+    n, quads, photo = problem.n_nodes, getattr(problem, "quads", None), getattr(problem, "photo", None)
+    cells = problem.n_tris * BYTES_PER_TRI + (0 if quads is None else len(quads)) * BYTES_PER_QUAD + (1 << 20)
+    if precision == avip.PREC_MIXED:
+        return int(n * BYTES_PER_NODE + cells)
+    rows = min(n, DENSE_ROWS_CLUSTER if solver_kind(problem, precision) == 11 else DENSE_ROWS)
+    if getattr(problem, "axisymmetric", False) and n <= AXISYM_AMG_NODES:
+        rows = 0
+    terms = 0 if photo is None else len(photo.a)
+    return int(n * (BYTES_PER_NODE_FP64 + terms * BYTES_PER_NODE_PHOTO) + (1 + terms) * 4 * rows * rows + cells)
 
 
 def solver_kind(problem, precision: int = avip.PREC_MIXED) -> int:
@@ -187,7 +205,7 @@ class Server:
         def release_for(req):
             def _rel():
                 with cv:
-                    used[0] -= estimate_bytes(req.problem)
+                    used[0] -= estimate_bytes(req.problem, self.precision)
                     slots[0] -= 1
                     cv.notify_all()
             return _rel
@@ -195,14 +213,14 @@ class Server:
         def built_for(req):
             def _built():
                 with cv:
-                    reserved[0] -= estimate_bytes(req.problem)
+                    reserved[0] -= estimate_bytes(req.problem, self.precision)
                     cv.notify_all()
             return _built
 
         i = 0
         while i < len(pending):
             req = pending[i]
-            need = estimate_bytes(req.problem)
+            need = estimate_bytes(req.problem, self.precision)
             if need > self.budget:
                 req.status = avip.AVIP_ENOMEM       # can never fit: rejected, not attempted
                 req.done = req.arrival

@@ -1,4 +1,6 @@
 """Device memory a handle holds (mesh_info), and what creating one does when memory runs short."""
+import dataclasses
+
 import pytest
 
 import avip_oracle as O
@@ -108,3 +110,28 @@ def test_inverse_in_a_batch(avip, nx, ny, cluster):
         assert normwise(mesh.phi(), phi) <= 1e-10
     for h in (m, other, f):
         h.close()
+
+
+@pytest.mark.parametrize("n", [7, 21, 37, 67, 95, 201])
+@pytest.mark.parametrize("mesh", ["triangles", "quads", "mixed cells", "axisym", "photo", "axisym photo"])
+def test_serving_reserves_what_a_handle_holds(avip, n, mesh):
+    """A request's estimate covers the handle it is served with, and is not twice as much beside the dense
+    operators and a megabyte."""
+    from paper_2201_01291_gb300 import serve
+    kw = dict(field_dependent=True, source=W.SRC_TOWNSEND)
+    axisym = mesh.startswith("axisym")
+    if axisym:
+        p = W.axisym_problem(n, n, 1.25e-2, 1.25e-2, 18750.0, seed=n, n_peak=5e18, n_back=1e13, sigma=4e-4,
+                             x0=1e-2, **kw)
+    elif mesh in ("quads", "mixed cells"):
+        p = W.hybrid_plates_problem(n, n, 1e-2, 1e-2, 1e4, n, quad_fraction=1.0 if mesh == "quads" else 0.5, **kw)
+    else:
+        p = W.plates_problem(n, n, 1e-2, 1e-2, 5e3, seed=n, **kw)
+    if mesh.endswith("photo"):
+        p = dataclasses.replace(p, photo=W.photo_air())
+    for prec in (avip.PREC_FP64,) if axisym or p.photo is not None else (avip.PREC_FP64, avip.PREC_MIXED):
+        m = avip.Mesh(p, pcg_kind=serve.solver_kind(p, prec), cluster_size=serve.cluster_ctas(p), precision=prec)
+        held, reserved = avip.mesh_info(m.h)["device_bytes"], serve.estimate_bytes(p, prec)
+        m.close()
+        dense = 4 * 4 * min(p.n_nodes, serve.DENSE_ROWS) ** 2
+        assert held <= reserved <= 2 * held + dense + (1 << 20), (prec, held, reserved)
