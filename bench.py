@@ -219,7 +219,7 @@ KERNEL_NAMES = {1: "pcg_fp64_kernel (streaming)", 2: "pcg_fp64_res_kernel (regis
                 9: "bicgstab_amg_kernel (BiCGStab + AMG V-cycle, axisymmetric)",
                 10: "pcg_amg_mixed_kernel (FP32 CG + FP32 AMG V-cycle, FP64 refinement)",
                 11: "pcg_amg_cluster_kernel (AMG-preconditioned CG on one cluster)"}
-INVERSE_NODES = 4608  # planar FP64 meshes up to this size: the inverse of the matrix as the preconditioner
+L2_BYTES = 129e6
 
 # DRAM bytes per solver iteration measured by ncu on the pin-plane 500 x 1000 workload (the
 # counters of one captured launch divided by its iterations), keyed by solver kind; valid for the
@@ -403,9 +403,8 @@ def run_ours(args, rank, world, local_rank):
     # ---- roofline of the dominant kernel (PCG)
     peaks = measured_peaks()
     kernel_name = KERNEL_NAMES.get(info["pcg_kind"], str(info["pcg_kind"]))
-    if (args.precision == "fp64" and not args.precond_fp64 and args.pcg_kind == 0 and info["pcg_kind"] in (8, 11)
-            and info["n_nodes"] <= INVERSE_NODES):
-        info["levels"] = info["levels"][:1]  # the inverse of the matrix takes the place of the V-cycle
+    inverse = info["pcg_kind"] in (8, 11) and len(info["levels"]) == 1  # of the matrix, in the V-cycle's place
+    if inverse:
         kernel_name += ", preconditioned by the inverse of the matrix"
     if info["pcg_kind"] == 11:  # the one-cluster AMG solve moves the bytes of kind 8 or 10
         info = dict(info, pcg_kind=10 if args.precision == "mixed" else 8)
@@ -449,11 +448,14 @@ def run_ours(args, rank, world, local_rank):
         "scaling": "weak", "vs_baseline": None, "dtype": "f64" if args.precision == "fp64" else "f32+f64",
         "data": "synthetic",
         "config": workload_config(problem, desc, args),
-        "preconditioner": ("AMG V-cycle in " + ("FP64" if info["precond_bytes"] == 8 else "FP32") +
+        "preconditioner": (("inverse of the matrix in " if inverse else "AMG V-cycle in ") +
+                           ("FP64" if info["precond_bytes"] == 8 else "FP32") +
                            "; Krylov iterate, residuals, products with the Poisson matrix and stopping test in FP64")
         if info["pcg_kind"] in (8, 9, 11) else None,
         "parallelism": f"replicas x{world}", "nnz": info["nnz"],
-        "l2": "working set per step far larger than L2 (the solver streams ~2 GB of operators per step); no flush",
+        "l2": ("working set per step larger than L2 (the solver streams its operators every iteration); no flush"
+               if info["device_bytes"] > L2_BYTES else
+               f"the handle's {info['device_bytes'] / 1e6:.1f} MB stay in L2 from step to step, as in a run; no flush"),
         "e2e": {"value": world * T * e2e_steps / e2e_t, "unit": UNIT, "h2d_bytes_per_step": state_bytes,
                 "d2h_bytes_per_step": state_bytes,
                 "how": "per step: state_set from pinned host memory, run_steps(1), state_get to pinned host memory"},
