@@ -127,7 +127,8 @@ void sell_from_csr(const Csr& A, SellHost& out, int lpr = 1);
 // Lanes per row for a streamed operator: the smallest power of two (at most 32) that leaves
 // at most 8 stored entries per lane on an average row, or fewer lanes when that gives a slice to
 // every warp of the whole-GPU solvers already (a row's epilogue runs on one of its lanes only, and
-// the finest level's has FP64 operations).
+// the finest level's has FP64 operations).  The layout depends on the mesh alone: a hierarchy solved on
+// one cluster has the same.
 // `mixed`: always the former (the mixed-precision solves keep one arithmetic, see block_group_sum).
 int lanes_per_row(const Csr& A, bool mixed);
 // Elements a streamed array must be readable past its end (a ring slot is always filled).

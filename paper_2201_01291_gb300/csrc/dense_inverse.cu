@@ -213,10 +213,10 @@ int dense_inverse_rows(int N) { return (N + kB - 1) / kB * kB; }
 size_t dense_inverse_scratch(int N) { return (size_t)2 * kB * dense_inverse_rows(N); }
 
 // M (dense_inverse_rows squared, zeroed) becomes the inverse of A; *bad (zeroed) is set when FP32
-// does not suffice: a matrix whose condition comes near 1e7 (cells of aspect 100 and more between
+// does not suffice: a matrix whose condition comes near 1e7 (cells of aspect 50 and more between
 // electrodes at the long ends).  A spectral radius of A M - I of at most 1/2 keeps M positive
 // definite and the CG's iterations few (condition of A M at most 3); ordinary meshes have 1e-6 to
-// 1e-3.  Costs 0.3 ms at 4,608 nodes.
+// 1e-3.  With its memory it adds 8.3 ms to creating a handle of 4,608 nodes (4,225: 6.9, 1,353: 1.2).
 cudaError_t launch_dense_inverse(const SellView& A, float* M, float* scratch, int* bad, cudaStream_t st) {
   const int np = dense_inverse_rows(A.N), nb = np / kB;
   float *R = scratch, *Cc = scratch + (size_t)kB * np;
