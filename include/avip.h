@@ -118,7 +118,12 @@ typedef struct avip_opts {
                                           10 the mixed-precision form of 8, 11 the AMG solve on
                                           one thread-block cluster (auto for planar meshes up
                                           to 20,000 nodes: with the inverse up to 1,200, FP64;
-                                          in mixed precision from 501 nodes on, 6 below) */
+                                          in mixed precision from 501 nodes on, 6 below).  The
+                                          inverse takes 4 bytes x nodes squared (85 MB at most);
+                                          a matrix too ill-conditioned for it, memory that does
+                                          not suffice, or precond_fp64 leave the V-cycle on one
+                                          cluster (5 up to 500 nodes), and a batch gives an
+                                          inverse of more than 1,536 nodes back */
   void* stream;                        /* cudaStream_t for all work; NULL = default stream    */
   avip_alloc_fn alloc;                 /* optional device allocator (both or neither)         */
   avip_free_fn free;
